@@ -136,65 +136,81 @@ __device__ __forceinline__ T warp_max(T v) {
     return v;
 }
 
-// CTA-wide sum in a fixed order; `scratch` holds one slot per warp.  Every
-// thread gets the result.  Contains __syncthreads(): call from all threads.
-template <typename T, int NWARPS>
-__device__ __forceinline__ T block_sum(T v, T* scratch) {
-    v = warp_sum(v);
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    __syncthreads();
-    if (lane == 0) scratch[wid] = v;
-    __syncthreads();
-    T r = T(0);
+// ---------------------------------------------------------------------------
+// fp64 sums over a warp.  The part's fp64 pipe takes two lanes a cycle per SM,
+// so a warp-wide fp64 add costs 16 cycles of it, and a butterfly that repeats
+// every sum in every lane is the wrong shape: these halve the values a lane
+// carries at each level where there is more than one (6 adds per warp for four
+// sums, 5 for two, against 20 and 10).  The order is fixed.
+// ---------------------------------------------------------------------------
+
+__device__ __forceinline__ double shfl_xor_f64(double v, int m) { return __shfl_xor_sync(0xffffffffu, v, m); }
+
+// Four sums: lane l ends with the total of value l / 8.
+__device__ __forceinline__ double warp_sum4(double a0, double a1, double a2, double a3) {
+    const int lane = threadIdx.x & 31;
+    const bool hi = lane & 16, odd = lane & 8;
+    const double k0 = (hi ? a2 : a0) + shfl_xor_f64(hi ? a0 : a2, 16);
+    const double k1 = (hi ? a3 : a1) + shfl_xor_f64(hi ? a1 : a3, 16);
+    double k = (odd ? k1 : k0) + shfl_xor_f64(odd ? k0 : k1, 8);
 #pragma unroll
-    for (int w = 0; w < NWARPS; ++w) r += scratch[w];
+    for (int m = 4; m >= 1; m >>= 1) k += shfl_xor_f64(k, m);
+    return k;
+}
+
+// Two sums: lane l ends with the total of value l / 16.
+__device__ __forceinline__ double warp_sum2(double a0, double a1) {
+    const bool hi = threadIdx.x & 16;
+    double k = (hi ? a1 : a0) + shfl_xor_f64(hi ? a0 : a1, 16);
+#pragma unroll
+    for (int m = 8; m >= 1; m >>= 1) k += shfl_xor_f64(k, m);
+    return k;
+}
+
+// Maximum of non-negative floats (their bit patterns order as unsigned integers).
+__device__ __forceinline__ float warp_max_nonneg(float v) {
+    return __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(v)));
+}
+
+// ---------------------------------------------------------------------------
+// thread-block clusters
+// ---------------------------------------------------------------------------
+
+__device__ __forceinline__ uint32_t cluster_size() {
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
     return r;
 }
 
-template <typename T, int NWARPS>
-__device__ __forceinline__ T block_max(T v, T* scratch) {
-    v = warp_max(v);
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    __syncthreads();
-    if (lane == 0) scratch[wid] = v;
-    __syncthreads();
-    T r = scratch[0];
-#pragma unroll
-    for (int w = 1; w < NWARPS; ++w) r = max(r, scratch[w]);
+__device__ __forceinline__ uint32_t cluster_rank() {
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
     return r;
 }
 
-// CTA-wide sums of N doubles and the maximum of one more, in the order of
-// block_sum / block_max (a butterfly inside each warp, then the warps in
-// order), with a single shared-memory exchange.  The results are valid in
-// thread 0 only: the cross-warp pass runs there alone (fp64 is a narrow pipe
-// on this part, so the other threads skip it).  `scratch` holds
-// NWARPS * (N + 1) doubles.  Contains __syncthreads(): call from all threads.
-template <int NWARPS, int N>
-__device__ __forceinline__ void block_sums_max0(double (&v)[N], double& mx, double* scratch) {
-#pragma unroll
-    for (int m = 16; m >= 1; m >>= 1) {
-#pragma unroll
-        for (int k = 0; k < N; ++k) v[k] += __shfl_xor_sync(0xffffffffu, v[k], m);
-        mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, m));
-    }
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    if (lane == 0) {
-#pragma unroll
-        for (int k = 0; k < N; ++k) scratch[wid * (N + 1) + k] = v[k];
-        scratch[wid * (N + 1) + N] = mx;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-#pragma unroll
-        for (int k = 0; k < N; ++k) v[k] = 0.0;
-        mx = scratch[N];
-        for (int w = 0; w < NWARPS; ++w) {
-#pragma unroll
-            for (int k = 0; k < N; ++k) v[k] += scratch[w * (N + 1) + k];
-            mx = fmax(mx, scratch[w * (N + 1) + N]);
-        }
-    }
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// Address of the same shared-memory location in CTA `rank` of the cluster.
+__device__ __forceinline__ uint32_t peer_addr(const void* p, uint32_t rank) {
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;"
+                 : "=r"(r)
+                 : "r"(static_cast<uint32_t>(__cvta_generic_to_shared(p))), "r"(rank));
+    return r;
+}
+
+__device__ __forceinline__ double ld_peer_f64(const double* p, uint32_t rank) {
+    double v;
+    asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(peer_addr(p, rank)) : "memory");
+    return v;
+}
+
+__device__ __forceinline__ uint32_t ld_peer_u32(const void* p, uint32_t rank) {
+    uint32_t v;
+    asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(peer_addr(p, rank)) : "memory");
+    return v;
 }
 
 }  // namespace acrl

@@ -25,6 +25,13 @@ inline acrl_status launch_status() {
     return cudaGetLastError() == cudaSuccess ? ACRL_OK : ACRL_ERR_CUDA;
 }
 
+// Status of a launch call that returned an error (which is cleared, as
+// launch_status does).
+inline acrl_status launch_failed() {
+    (void)cudaGetLastError();
+    return ACRL_ERR_CUDA;
+}
+
 inline bool params_ok(const acrl_params* p) {
     if (!p) return false;
     if (!(p->gamma > 0.f) || !(p->C > 1.f) || !(p->clip_eps >= 0.f && p->clip_eps < 1.f)) return false;

@@ -539,21 +539,9 @@ __global__ void __launch_bounds__(THREADS) loss_grad_warp(
 // ~75 us on one CTA).
 constexpr int kSumThreads = 1024, kSumCtas = 8;
 
-__device__ __forceinline__ void sum_cluster_sync() {
-    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-
-__device__ __forceinline__ double ld_peer_f64(const double* p, uint32_t rank) {
-    uint32_t a;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(p)), "r"(rank));
-    double v;
-    asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(a) : "memory");
-    return v;
-}
-
 __global__ void __cluster_dims__(kSumCtas, 1, 1) __launch_bounds__(kSumThreads)
     loss_sum_kernel(const float* __restrict__ tl, int64_t T, float* __restrict__ loss) {
-    __shared__ double sh[kSumThreads / 32 * 2];
+    __shared__ double sh[kSumThreads / 32];
     __shared__ double cta_sum;
     const int64_t c = blockIdx.x;   // the launch is one cluster: the block index is the rank
     double s0 = 0.0, s1 = 0.0;
@@ -580,16 +568,21 @@ __global__ void __cluster_dims__(kSumCtas, 1, 1) __launch_bounds__(kSumThreads)
         const int64_t lo = min(T, c * per), hi = min(T, lo + per);
         for (int64_t j = lo + threadIdx.x; j < hi; j += kSumThreads) s0 += tl[j];
     }
-    double total[1] = {s0 + s1}, unused = 0.0;
-    block_sums_max0<kSumThreads / 32, 1>(total, unused, sh);
-    if (threadIdx.x == 0) cta_sum = total[0];
-    sum_cluster_sync();   // every CTA's sum is in its shared memory
+    const double ws = warp_sum(s0 + s1);
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = ws;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double total = 0.0;
+        for (int w = 0; w < kSumThreads / 32; ++w) total += sh[w];
+        cta_sum = total;
+    }
+    cluster_sync();   // every CTA's sum is in its shared memory
     if (c == 0 && threadIdx.x == 0) {
         double r = 0.0;
         for (uint32_t k = 0; k < uint32_t(kSumCtas); ++k) r += ld_peer_f64(&cta_sum, k);
         *loss = float(r);
     }
-    sum_cluster_sync();   // no CTA leaves while CTA 0 may still read its shared memory
+    cluster_sync();   // no CTA leaves while CTA 0 may still read its shared memory
 }
 
 template <bool RECOMPUTE, bool ENT>

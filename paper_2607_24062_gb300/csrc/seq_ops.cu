@@ -2,10 +2,17 @@
 // per-response / per-prompt / batch aggregates, GRPO advantages and the
 // adaptive controller with its importance weights.
 //
-// One CTA per response does the segmented reductions; single-CTA kernels
-// finalise prompts and the batch.  Every reduction has a fixed order (strided
-// per-thread partials, then a fixed warp butterfly and warp-order sum) and no
-// floating-point atomics, so the results are bit-reproducible.
+// One CTA (or a small cluster of CTAs) per response does the segmented
+// reductions; single-CTA kernels finalise prompts and the batch.  Every
+// reduction has a fixed order (strided per-thread partials, then a fixed warp
+// tree and warp-order sum) and no floating-point atomics, so the results are
+// bit-reproducible.
+//
+// What bounds these kernels is latency and the fp64 pipe (two lanes a cycle
+// per SM), not their ~25 bytes per token: counts and maxima therefore travel
+// as integers, sums share one warp tree, scalar fp64 divisions run once per
+// CTA with a different quotient in each lane, and warps without data skip
+// their trees.
 #include <cmath>
 
 #include "acrl_device.cuh"
@@ -15,7 +22,10 @@ namespace acrl {
 namespace {
 
 constexpr int kSeqThreads = 256;
+constexpr int kSeqUnroll = 4;    // tokens per thread in flight
 constexpr int kFinThreads = 512;
+constexpr int kSeqCtas = 304, kSeqTokens = 256;  // see ctas_per_response
+constexpr int kFinSeqs = 2048;   // responses whose mean distance the batch kernel keeps in shared memory
 
 __device__ __forceinline__ bool seq_range(const int64_t* so, int i, int64_t T, int64_t& lo, int64_t& hi) {
     lo = so[i];
@@ -23,14 +33,21 @@ __device__ __forceinline__ bool seq_range(const int64_t* so, int i, int64_t T, i
     return lo >= 0 && lo <= hi && hi <= T;
 }
 
-// Index g with goff[g] <= i < goff[g+1], or -1.
+// Index g with goff[g] <= i < goff[g+1], or -1; the whole warp searches, 32
+// probes at a time (one step for up to 32 prompts, two for up to 1,024).
 __device__ __forceinline__ int group_of(const int32_t* goff, int Gn, int i) {
-    int lo = 0, hi = Gn;  // invariant: answer in [lo, hi)
-    while (hi - lo > 1) {
-        const int mid = (lo + hi) >> 1;
-        if (goff[mid] <= i) lo = mid; else hi = mid;
+    if (Gn <= 0) return -1;
+    const int lane = threadIdx.x & 31;
+    int lo = 0, n = Gn;  // invariant: answer in [lo, lo + n)
+    while (n > 1) {
+        const int step = (n + 31) >> 5;
+        const int64_t at = int64_t(lane) * step;
+        const unsigned le = __ballot_sync(0xffffffffu, at < n && goff[lo + (at < n ? int(at) : 0)] <= i);
+        const int k = le ? 31 - __clz(le) : 0;   // the last probe at or before i
+        lo += k * step;
+        n = min(step, n - k * step);
     }
-    return (Gn > 0 && goff[lo] <= i && i < goff[lo + 1]) ? lo : -1;
+    return (goff[lo] <= i && i < goff[lo + 1]) ? lo : -1;
 }
 
 // |exp(a) - exp(b)| without cancellation when a and b are close.
@@ -39,66 +56,140 @@ __device__ __forceinline__ float prob_distance(float a, float b) {
     return fabsf(l) < 0.5f ? expf(b) * fabsf(expm1f(l)) : fabsf(expf(a) - expf(b));
 }
 
-// K2a: per-token lr and d, per-response sums.  One CTA per response.
-__global__ void __launch_bounds__(kSeqThreads) seq_stats_kernel(
+// One CTA's part of a response's sums.
+struct SeqPart {
+    double sum[4];  // d, d^2, lr, H
+    int n;
+    uint32_t max_d; // bits of a non-negative float
+};
+
+// K2a: per-token lr and d, per-response sums.  A cluster of CTAs per response
+// (one CTA where there are enough responses to fill the chip); CTA r takes
+// tokens r kSeqThreads + tid of every round of the cluster's threads, and rank
+// 0 adds the CTAs' sums in rank order.  A ninth warp finds the response's
+// prompt meanwhile.
+__global__ void __launch_bounds__(kSeqThreads + 32) seq_stats_kernel(
     const float* __restrict__ logp_pi, const float* __restrict__ logp_mu, const uint8_t* __restrict__ mask,
     int64_t T, const int64_t* __restrict__ so, int S, const int32_t* __restrict__ goff, int Gn,
     const float* __restrict__ entropy, float* __restrict__ lr, float* __restrict__ d, acrl_seq_stats* seq,
     int32_t* flags) {
-    constexpr int NW = kSeqThreads / 32;
-    __shared__ double sh[NW * 6];
-    const int i = blockIdx.x;
-    int64_t lo, hi;
-    if (!seq_range(so, i, T, lo, hi)) {
-        if (threadIdx.x == 0) raise_flag(flags, ACRL_FLAG_BAD_OFFSETS);
-        lo = hi = 0;
-    }
-    int n = 0;
-    double sd = 0.0, sd2 = 0.0, slr = 0.0, sH = 0.0;
-    float mxd = 0.f;
-    bool nan_lr = false;
-    for (int64_t t = lo + threadIdx.x; t < hi; t += kSeqThreads) {
-        const bool m = mask ? mask[t] != 0 : true;
-        float l = 0.f, dd = 0.f;
-        if (m) {
-            const float a = logp_pi[t], b = logp_mu[t];
-            l = a - b;
-            nan_lr |= isnan(l);  // a NaN log-prob on either side
-            dd = prob_distance(a, b);
-            ++n;
-            sd += dd;
-            sd2 += double(dd) * dd;
-            slr += l;
-            if (entropy) sH += entropy[t];
-            mxd = fmaxf(mxd, dd);
+    constexpr int NW = kSeqThreads / 32, U = kSeqUnroll;
+    __shared__ double sh[NW * 4];
+    __shared__ int sh_n[NW];
+    __shared__ uint32_t sh_max[NW];
+    __shared__ int sh_group;
+    __shared__ SeqPart part;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int nct = int(cluster_size()), rank = int(cluster_rank());
+    const int i = int(blockIdx.x) / nct;
+    if (wid == NW) {
+        if (rank == 0) {
+            const int g = group_of(goff, Gn, i);
+            if (lane == 0) sh_group = g;
         }
-        lr[t] = l;
-        d[t] = dd;
+    } else {
+        int64_t lo, hi;
+        if (!seq_range(so, i, T, lo, hi)) {
+            if (rank == 0 && threadIdx.x == 0) raise_flag(flags, ACRL_FLAG_BAD_OFFSETS);
+            lo = hi = 0;
+        }
+        int n = 0;
+        double sd = 0.0, sd2 = 0.0, slr = 0.0, sH = 0.0;
+        float mxd = 0.f;
+        bool nan_lr = false;
+        const int64_t stride = int64_t(nct) * kSeqThreads;
+        for (int64_t t0 = lo + rank * kSeqThreads + threadIdx.x; t0 < hi; t0 += U * stride) {
+            float a[U], b[U], h[U];
+            bool m[U];
+#pragma unroll
+            for (int k = 0; k < U; ++k) {
+                const int64_t t = t0 + k * stride;
+                const bool in = t < hi;
+                m[k] = in && (mask ? mask[t] != 0 : true);
+                a[k] = in ? logp_pi[t] : 0.f;
+                b[k] = in ? logp_mu[t] : 0.f;
+                h[k] = in && entropy ? entropy[t] : 0.f;
+            }
+#pragma unroll
+            for (int k = 0; k < U; ++k) {
+                const int64_t t = t0 + k * stride;
+                if (t >= hi) break;
+                float l = 0.f, dd = 0.f;
+                if (m[k]) {
+                    l = a[k] - b[k];
+                    nan_lr |= isnan(l);  // a NaN log-prob on either side
+                    dd = prob_distance(a[k], b[k]);
+                    ++n;
+                    const double dd64 = dd;
+                    sd += dd64;
+                    sd2 += dd64 * dd64;
+                    slr += l;
+                    if (entropy) sH += h[k];
+                    mxd = fmaxf(mxd, dd);
+                }
+                lr[t] = l;
+                d[t] = dd;
+            }
+        }
+        if (nan_lr) raise_flag(flags, ACRL_FLAG_NONFINITE);
+        const double s = warp_sum4(sd, sd2, slr, sH);
+        n = __reduce_add_sync(0xffffffffu, n);
+        mxd = warp_max_nonneg(mxd);
+        if ((lane & 7) == 0) sh[wid * 4 + (lane >> 3)] = s;
+        if (lane == 0) {
+            sh_n[wid] = n;
+            sh_max[wid] = __float_as_uint(mxd);
+        }
     }
-    if (nan_lr) raise_flag(flags, ACRL_FLAG_NONFINITE);
-    double v[5] = {double(n), sd, sd2, slr, sH}, mx = mxd;
-    block_sums_max0<NW, 5>(v, mx, sh);
-    n = int(v[0]);
-    sd = v[1];
-    sd2 = v[2];
-    slr = v[3];
-    sH = v[4];
-    mxd = float(mx);
-    if (threadIdx.x == 0) {
-        acrl_seq_stats s;
-        s.n = n;
-        s.group = group_of(goff, Gn, i);
-        s.mean_d = n ? float(sd / n) : 0.f;
-        s.max_d = mxd;
-        s.sum_d = sd;
-        s.sum_d2 = sd2;
-        s.sum_lr = slr;
-        s.sum_H = sH;
-        s.sum_w = 0.0;
-        s.n_trunc = 0;
-        s.alpha = 0.f;
-        seq[i] = s;
+    __syncthreads();
+    if (wid == 0) {  // the warps' sums in order, value k in lane k
+        double s = 0.0;
+        if (lane < 4)
+#pragma unroll
+            for (int w = 0; w < NW; ++w) s += sh[w * 4 + lane];
+        const int n = __reduce_add_sync(0xffffffffu, lane < NW ? sh_n[lane] : 0);
+        const uint32_t mx = __reduce_max_sync(0xffffffffu, lane < NW ? sh_max[lane] : 0u);
+        if (lane < 4) part.sum[lane] = s;
+        if (lane == 0) {
+            part.n = n;
+            part.max_d = mx;
+        }
+        __syncwarp();
     }
+    if (nct > 1) cluster_sync();  // every CTA's part is in its shared memory
+    if (rank == 0 && wid == 0) {
+        double s = lane < 4 ? part.sum[lane] : 0.0;
+        int n = lane == 0 ? part.n : 0;
+        uint32_t mx = lane == 0 ? part.max_d : 0u;
+        if (nct > 1) {
+            if (lane < 4)
+                for (int r = 1; r < nct; ++r) s += ld_peer_f64(&part.sum[lane], uint32_t(r));
+            if (lane > 0 && lane < nct) {
+                n = int(ld_peer_u32(&part.n, uint32_t(lane)));
+                mx = ld_peer_u32(&part.max_d, uint32_t(lane));
+            }
+            n = __reduce_add_sync(0xffffffffu, n);
+            mx = __reduce_max_sync(0xffffffffu, mx);
+        }
+        const double sd2 = __shfl_sync(0xffffffffu, s, 1), slr = __shfl_sync(0xffffffffu, s, 2),
+                     sH = __shfl_sync(0xffffffffu, s, 3);
+        if (lane == 0) {
+            acrl_seq_stats o;
+            o.n = n;
+            o.group = sh_group;
+            o.mean_d = n ? float(s / n) : 0.f;
+            o.max_d = __uint_as_float(mx);
+            o.sum_d = s;
+            o.sum_d2 = sd2;
+            o.sum_lr = slr;
+            o.sum_H = sH;
+            o.sum_w = 0.0;
+            o.n_trunc = 0;
+            o.alpha = 0.f;
+            seq[i] = o;
+        }
+    }
+    if (nct > 1) cluster_sync();  // no CTA leaves while rank 0 may still read its shared memory
 }
 
 // K2b: prompt statistics and batch statistics; also checks the offsets.
@@ -106,12 +197,39 @@ __global__ void __launch_bounds__(kFinThreads) seq_finalize_kernel(
     int64_t T, const int64_t* __restrict__ so, int S, const int32_t* __restrict__ goff, int Gn,
     const acrl_seq_stats* __restrict__ seq, acrl_group_stats* grp, acrl_batch_stats* batch, int32_t* flags) {
     constexpr int NW = kFinThreads / 32;
-    __shared__ double sh[NW * 9];
+    __shared__ double sh_D[kFinSeqs];  // D_i, and the valid tokens of response i
+    __shared__ int sh_n[kFinSeqs];
+    __shared__ double sh[NW * 5];
+    __shared__ long long sh_N[NW];
+    __shared__ int sh_sv[NW], sh_qv[NW];
+    __shared__ float sh_max[NW];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const bool keep = S <= kFinSeqs;
     bool bad = false;
-    for (int i = threadIdx.x; i < S; i += kFinThreads) bad |= so[i] > so[i + 1];
+    long long N = 0;
+    int sv = 0;
+    double sd = 0.0, sd2 = 0.0, sH = 0.0, slr = 0.0;
+    float dmax = 0.f;
+    for (int i = threadIdx.x; i < S; i += kFinThreads) {
+        bad |= so[i] > so[i + 1];
+        const int n = seq[i].n;
+        const double s = seq[i].sum_d;
+        N += n;
+        sv += n > 0;
+        sd += s;
+        sd2 += seq[i].sum_d2;
+        sH += seq[i].sum_H;
+        slr += seq[i].sum_lr;
+        dmax = fmaxf(dmax, seq[i].max_d);
+        if (keep) {
+            sh_n[i] = n;
+            sh_D[i] = n > 0 ? s / n : 0.0;
+        }
+    }
     for (int g = threadIdx.x; g < Gn; g += kFinThreads) bad |= goff[g] > goff[g + 1];
     if (threadIdx.x == 0) bad |= so[0] != 0 || so[S] != T || (Gn > 0 ? (goff[0] != 0 || goff[Gn] != S) : S != 0);
     if (bad) raise_flag(flags, ACRL_FLAG_BAD_OFFSETS);
+    __syncthreads();
 
     int qv = 0;
     double ysum = 0.0;
@@ -123,11 +241,11 @@ __global__ void __launch_bounds__(kFinThreads) seq_finalize_kernel(
         long long ntok = 0;
         double y = 0.0;
         for (int i = b; i < e; ++i) {
-            const int n = seq[i].n;
+            const int n = keep ? sh_n[i] : seq[i].n;
             ntok += n;
             if (n > 0) {
                 ++G;
-                y += seq[i].sum_d / n;
+                y += keep ? sh_D[i] : seq[i].sum_d / n;
             }
         }
         acrl_group_stats gs;
@@ -141,49 +259,59 @@ __global__ void __launch_bounds__(kFinThreads) seq_finalize_kernel(
             ysum += gs.Y;
         }
     }
-    long long N = 0;
-    int sv = 0;
-    double sd = 0.0, sd2 = 0.0, sH = 0.0, slr = 0.0, dmax = 0.0;
-    for (int i = threadIdx.x; i < S; i += kFinThreads) {
-        const acrl_seq_stats s = seq[i];
-        N += s.n;
-        sv += s.n > 0;
-        sd += s.sum_d;
-        sd2 += s.sum_d2;
-        sH += s.sum_H;
-        slr += s.sum_lr;
-        dmax = fmax(dmax, double(s.max_d));
+    // warps beyond the responses and prompts hold nothing
+    const int used = min(NW, (max(S, Gn) + 31) / 32);
+    if (wid < used) {
+        const double s = warp_sum4(sd, sd2, sH, slr), y = warp_sum(ysum);
+        N = warp_sum(N);
+        sv = __reduce_add_sync(0xffffffffu, sv);
+        qv = __reduce_add_sync(0xffffffffu, qv);
+        dmax = warp_max_nonneg(dmax);
+        if ((lane & 7) == 0) sh[wid * 5 + (lane >> 3)] = s;
+        if (lane == 0) {
+            sh[wid * 5 + 4] = y;
+            sh_N[wid] = N;
+            sh_sv[wid] = sv;
+            sh_qv[wid] = qv;
+            sh_max[wid] = dmax;
+        }
     }
-    // counts travel as doubles: exact below 2^53
-    double v[8] = {double(qv), ysum, double(N), double(sv), sd, sd2, sH, slr};
-    block_sums_max0<NW, 8>(v, dmax, sh);
-    qv = int(v[0]);
-    ysum = v[1];
-    N = (long long)v[2];
-    sv = int(v[3]);
-    sd = v[4];
-    sd2 = v[5];
-    sH = v[6];
-    slr = v[7];
-    if (threadIdx.x == 0) {
-        acrl_batch_stats b = *batch;
-        b.n_tokens = N;
-        b.n_seqs_valid = sv;
-        b.n_groups_valid = qv;
-        const double inv = N ? 1.0 / double(N) : 0.0;
-        b.d_mean = sd * inv;
-        b.d_max = dmax;
-        const double var = sd2 * inv - b.d_mean * b.d_mean;
-        b.d_std = var > 0.0 ? sqrt(var) : 0.0;
-        b.Y_sum = ysum;
-        b.Y_mean = qv ? ysum / qv : 0.0;
-        b.H_mean = sH * inv;
-        b.lr_mean = slr * inv;
-        b.X = 0.0;
-        b.trunc_frac = 0.0;
-        b.w_mean = 0.0;
-        b.alpha_mean = 0.0;
-        *batch = b;
+    __syncthreads();
+    if (wid == 0) {
+        double s = 0.0;  // value k in lane k: sums of d, d^2, H, lr and Y_g
+        if (lane < 5)
+            for (int w = 0; w < used; ++w) s += sh[w * 5 + lane];
+        N = warp_sum(lane < used ? sh_N[lane] : 0ll);
+        sv = __reduce_add_sync(0xffffffffu, lane < used ? sh_sv[lane] : 0);
+        qv = __reduce_add_sync(0xffffffffu, lane < used ? sh_qv[lane] : 0);
+        dmax = warp_max_nonneg(lane < used ? sh_max[lane] : 0.f);
+        // 1 / N in lane 0, Y_mean in lane 4
+        const double den = lane == 4 ? double(qv) : double(N);
+        const double q = den > 0.0 ? (lane == 4 ? s : 1.0) / den : 0.0;
+        const double inv = __shfl_sync(0xffffffffu, q, 0), ymean = __shfl_sync(0xffffffffu, q, 4);
+        const double mean = s * inv;  // lanes 0..3: the token means
+        const double d_mean = __shfl_sync(0xffffffffu, mean, 0), d2_mean = __shfl_sync(0xffffffffu, mean, 1),
+                     H_mean = __shfl_sync(0xffffffffu, mean, 2), lr_mean = __shfl_sync(0xffffffffu, mean, 3);
+        ysum = __shfl_sync(0xffffffffu, s, 4);
+        if (lane == 0) {
+            acrl_batch_stats b;
+            b.n_tokens = N;
+            b.n_seqs_valid = sv;
+            b.n_groups_valid = qv;
+            b.d_mean = d_mean;
+            b.d_max = double(dmax);
+            const double var = d2_mean - d_mean * d_mean;
+            b.d_std = var > 0.0 ? sqrt(var) : 0.0;
+            b.Y_sum = ysum;
+            b.Y_mean = ymean;
+            b.H_mean = H_mean;
+            b.lr_mean = lr_mean;
+            b.X = 0.0;
+            b.trunc_frac = 0.0;
+            b.w_mean = 0.0;
+            b.alpha_mean = 0.0;
+            *batch = b;
+        }
     }
 }
 
@@ -232,156 +360,282 @@ __global__ void controller_init_kernel(acrl_controller_state* st, double X_init)
     *st = s;
 }
 
-// K4a: state update (calibration of X) and alpha per response.
-__global__ void __launch_bounds__(kFinThreads) controller_alpha_kernel(
-    acrl_controller_state* st, acrl_params p, int S, int Gn, acrl_seq_stats* seq,
-    const acrl_group_stats* __restrict__ grp, acrl_batch_stats* batch, const float* __restrict__ adv,
-    float* alpha_out, int32_t* flags) {
-    __shared__ double sh_X;
-    __shared__ int sh_apply;
-    if (threadIdx.x == 0) {
-        // Y_mean from the (possibly all-reduced across ranks) sum and prompt count
-        batch->Y_mean = batch->n_groups_valid > 0 ? batch->Y_sum / double(batch->n_groups_valid) : 0.0;
-        acrl_controller_state s = *st;
-        const bool was_calibrated = s.calibrated != 0;
-        int apply = 1;
-        if (!s.calibrated) {
-            s.calib_sum += batch->Y_sum;
-            s.calib_count += batch->n_groups_valid;
-            s.calib_done += 1;
-            if (s.calib_done >= p.calib_steps) {
-                s.X = s.calib_count > 0 ? s.calib_sum / double(s.calib_count) : 0.0;
-                s.calibrated = 1;
-            } else {
-                apply = 0;
-            }
+// What the controller does to its state on one batch: the X in force as a
+// quotient (so that a caller can fold the division into one it does anyway),
+// and whether alpha applies (it does not while X is still being calibrated).
+struct ControllerMove {
+    double x_num, x_den;
+    bool apply;
+    acrl_controller_state next;   // X not yet divided out
+};
+
+__device__ __forceinline__ ControllerMove controller_move(const acrl_controller_state& st, const acrl_params& p,
+                                                          double Y_sum, int n_groups_valid) {
+    ControllerMove m;
+    m.next = st;
+    m.next.step += 1;
+    m.x_num = st.X;
+    m.x_den = 1.0;
+    m.apply = true;
+    if (!st.calibrated) {
+        m.next.calib_sum += Y_sum;
+        m.next.calib_count += n_groups_valid;
+        m.next.calib_done += 1;
+        if (m.next.calib_done >= p.calib_steps) {
+            m.x_num = m.next.calib_count > 0 ? m.next.calib_sum : 0.0;
+            m.x_den = m.next.calib_count > 0 ? double(m.next.calib_count) : 1.0;
+            m.next.calibrated = 1;
+        } else {
+            m.apply = false;
         }
-        s.step += 1;
-        const bool uses_x = p.mode == ACRL_MODE_ACRL || p.mode == ACRL_MODE_ACRL_FALLBACK;
-        if (uses_x && apply && !(s.X > 0.0)) {
-            raise_flag(flags, ACRL_FLAG_X_NONPOS);
-            s.flags |= ACRL_FLAG_X_NONPOS;
-        }
-        const double X_use = s.X;
-        // moving-average X (off by default): this step uses X_use, the next one the update
-        if (was_calibrated && p.x_ema > 0.f) s.X = (1.0 - double(p.x_ema)) * s.X + double(p.x_ema) * batch->Y_mean;
-        *st = s;
-        batch->X = apply ? X_use : 0.0;
-        sh_X = X_use;
-        sh_apply = apply;
     }
-    __syncthreads();
-    const double X = sh_X;
-    const bool apply = sh_apply != 0;
-    const double Ybatch = batch->Y_mean;  // written by thread 0 above, before the barrier
-    for (int i = threadIdx.x; i < S; i += kFinThreads) {
-        float a = 0.f;
-        const float A = adv[i];
+    return m;
+}
+
+// K4a: alpha per response, per-token weights and loss coefficients; a cluster
+// of CTAs per response as in seq_stats_kernel.  The controller state is only
+// read here (every CTA works out the X in force for itself); the finalising
+// kernel writes it.
+__global__ void __launch_bounds__(kSeqThreads) controller_weights_kernel(
+    const acrl_controller_state* __restrict__ st, acrl_params p, const float* __restrict__ lr,
+    const uint8_t* __restrict__ mask, int64_t T, const int64_t* __restrict__ so, int Gn, acrl_seq_stats* seq,
+    const acrl_group_stats* __restrict__ grp, const acrl_batch_stats* __restrict__ batch,
+    const float* __restrict__ adv, float* __restrict__ weight, float* __restrict__ coef, float* __restrict__ alpha_out,
+    float* __restrict__ ent_coef) {
+    constexpr int NW = kSeqThreads / 32, U = kSeqUnroll;
+    __shared__ double sh[NW];
+    __shared__ int sh_nt[NW];
+    __shared__ float sh_alpha, sh_scale, sh_escale, sh_wmis;
+    __shared__ int sh_cut;
+    __shared__ double part_w;
+    __shared__ int part_nt;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int nct = int(cluster_size()), rank = int(cluster_rank());
+    const int i = int(blockIdx.x) / nct;
+    int64_t lo, hi;
+    if (!seq_range(so, i, T, lo, hi)) lo = hi = 0;
+    const float logC = logf(p.C);
+    const int64_t stride = int64_t(nct) * kSeqThreads;
+    const bool uses_lr = p.mode != ACRL_MODE_NONE && p.mode != ACRL_MODE_MIS;
+
+    // the first tokens are on their way while warp 0 works out the response's scalars
+    float l[U];
+    bool m[U];
+    auto load = [&](int64_t t0) {
+#pragma unroll
+        for (int k = 0; k < U; ++k) {
+            const int64_t t = t0 + k * stride;
+            const bool in = t < hi;
+            m[k] = in && (mask ? mask[t] != 0 : true);
+            l[k] = in && uses_lr ? lr[t] : 0.f;
+        }
+    };
+    int64_t t0 = lo + rank * kSeqThreads + threadIdx.x;
+    load(t0);
+    if (wid == 0) {
+        const int n = seq[i].n, g = seq[i].group;
+        const double sum_d = seq[i].sum_d;
+        const float Si = float(seq[i].sum_lr), A = adv[i];
+        const bool has_g = g >= 0 && g < Gn;
+        const double Yg = has_g ? grp[g].Y : 0.0;
+        const int ngv = batch->n_groups_valid;
+        const double Ysum = batch->Y_sum;
+        const ControllerMove mv = controller_move(*st, p, Ysum, ngv);
+        double norm;
+        if (p.agg == ACRL_AGG_TOKEN_MEAN)
+            norm = double(batch->n_tokens);
+        else
+            norm = double(ngv) * double(has_g ? grp[g].n_valid_seqs : 0) * double(n);
+        // one division, a different quotient in each lane: Y, X, A / norm, beta / norm
+        double num = 0.0, den = 1.0;
+        if (lane == 0) {
+            if (p.y_gran == ACRL_Y_SEQUENCE) {
+                num = sum_d;
+                den = double(n);
+            } else if (p.y_gran == ACRL_Y_BATCH) {
+                num = Ysum;
+                den = double(ngv);
+            } else {
+                num = Yg;
+            }
+        } else if (lane == 1) {
+            num = mv.x_num;
+            den = mv.x_den;
+        } else if (lane == 2 || lane == 3) {
+            num = lane == 2 ? double(A) : double(p.entropy_coeff);
+            den = norm;
+        }
+        const double q = den > 0.0 ? num / den : 0.0;
+        const double Y = __shfl_sync(0xffffffffu, q, 0), X = __shfl_sync(0xffffffffu, q, 1);
+        const float scale = float(__shfl_sync(0xffffffffu, q, 2)), escale = float(__shfl_sync(0xffffffffu, q, 3));
         const float sgnf = A > 0.f ? 1.f : (A < 0.f ? -1.f : 0.f);
+        float a = 0.f;
         if (p.mode == ACRL_MODE_TIS || p.mode == ACRL_MODE_MIS) {
             a = 1.f;
         } else if (p.mode == ACRL_MODE_ACRL_CONTINUOUS) {
-            a = seq[i].n > 0 ? -p.kappa * sgnf : 0.f;
-        } else if ((p.mode == ACRL_MODE_ACRL || p.mode == ACRL_MODE_ACRL_FALLBACK) && apply && X > 0.0 &&
-                   seq[i].n > 0) {
-            double Y;
-            if (p.y_gran == ACRL_Y_SEQUENCE) {
-                Y = seq[i].sum_d / seq[i].n;
-            } else if (p.y_gran == ACRL_Y_BATCH) {
-                Y = Ybatch;
-            } else {
-                const int g = seq[i].group;
-                Y = (g >= 0 && g < Gn) ? grp[g].Y : 0.0;
-            }
+            a = n > 0 ? -p.kappa * sgnf : 0.f;
+        } else if ((p.mode == ACRL_MODE_ACRL || p.mode == ACRL_MODE_ACRL_FALLBACK) && mv.apply && X > 0.0 && n > 0) {
             a = float(double(p.gamma) * double(sgnf) * (1.0 - Y / X));
             if (p.mode == ACRL_MODE_ACRL_FALLBACK && !(Y > X)) a = 0.f;
         }
-        seq[i].alpha = a;
-        if (alpha_out) alpha_out[i] = a;
+        if (lane == 0) {
+            const bool cut = Si > logC;
+            sh_alpha = a;
+            sh_scale = scale;
+            sh_escale = escale;
+            sh_cut = cut;
+            sh_wmis = (cut || isnan(Si)) ? 0.f : expf(Si);
+            if (rank == 0) {
+                seq[i].alpha = a;
+                if (alpha_out) alpha_out[i] = a;
+            }
+        }
     }
-}
-
-// K4b: per-token weights and loss coefficients; one CTA per response.
-__global__ void __launch_bounds__(kSeqThreads) controller_weights_kernel(
-    acrl_params p, const float* __restrict__ lr, const uint8_t* __restrict__ mask, int64_t T,
-    const int64_t* __restrict__ so, int Gn, acrl_seq_stats* seq, const acrl_group_stats* __restrict__ grp,
-    const acrl_batch_stats* __restrict__ batch, const float* __restrict__ adv, float* __restrict__ weight,
-    float* __restrict__ coef, float* __restrict__ ent_coef) {
-    constexpr int NW = kSeqThreads / 32;
-    __shared__ double sh[NW * 3];
-    const int i = blockIdx.x;
-    int64_t lo, hi;
-    if (!seq_range(so, i, T, lo, hi)) lo = hi = 0;
-    const acrl_seq_stats s = seq[i];
-    const float logC = logf(p.C);
-    double norm;
-    if (p.agg == ACRL_AGG_TOKEN_MEAN) {
-        norm = double(batch->n_tokens);
-    } else {
-        const int G = (s.group >= 0 && s.group < Gn) ? grp[s.group].n_valid_seqs : 0;
-        norm = double(batch->n_groups_valid) * double(G) * double(s.n);
-    }
-    const float scale = norm > 0.0 ? float(double(adv[i]) / norm) : 0.f;
-    const float escale = norm > 0.0 ? float(double(p.entropy_coeff) / norm) : 0.f;
-    const float Si = float(s.sum_lr);
-    const bool mis_cut = Si > logC;
-    const float w_mis = (mis_cut || isnan(Si)) ? 0.f : expf(Si);
+    __syncthreads();
+    const float alpha = sh_alpha, scale = sh_scale, escale = sh_escale, w_mis = sh_wmis;
+    const bool mis_cut = sh_cut != 0;
     int nt = 0;
     double sw = 0.0;
-    for (int64_t t = lo + threadIdx.x; t < hi; t += kSeqThreads) {
-        const bool m = mask ? mask[t] != 0 : true;
-        float w = 0.f;
-        if (m) {
-            if (p.mode == ACRL_MODE_NONE) {
-                w = 1.f;
-            } else if (p.mode == ACRL_MODE_MIS) {
-                w = w_mis;
-                nt += mis_cut;
-            } else {
-                // rho^0 = 1 even where the log-ratio is infinite (mu = 0); a NaN log-ratio gets weight 0
-                const float lrho = s.alpha == 0.f ? 0.f : s.alpha * lr[t];
-                w = isnan(lrho) ? 0.f : expf(fminf(lrho, logC));
-                nt += lrho > logC;
+    while (t0 < hi) {
+#pragma unroll
+        for (int k = 0; k < U; ++k) {
+            const int64_t t = t0 + k * stride;
+            if (t >= hi) break;
+            float w = 0.f;
+            if (m[k]) {
+                if (p.mode == ACRL_MODE_NONE) {
+                    w = 1.f;
+                } else if (p.mode == ACRL_MODE_MIS) {
+                    w = w_mis;
+                    nt += mis_cut;
+                } else {
+                    // rho^0 = 1 even where the log-ratio is infinite (mu = 0); a NaN log-ratio gets weight 0
+                    const float lrho = alpha == 0.f ? 0.f : alpha * l[k];
+                    w = isnan(lrho) ? 0.f : expf(fminf(lrho, logC));
+                    nt += lrho > logC;
+                }
+                sw += w;
             }
-            sw += w;
+            weight[t] = w;
+            coef[t] = w * scale;
+            if (ent_coef) ent_coef[t] = m[k] ? escale : 0.f;
         }
-        weight[t] = w;
-        coef[t] = w * scale;
-        if (ent_coef) ent_coef[t] = m ? escale : 0.f;
+        t0 += U * stride;
+        load(t0);
     }
-    double v[2] = {double(nt), sw}, unused = 0.0;
-    block_sums_max0<NW, 2>(v, unused, sh);
-    nt = int(v[0]);
-    sw = v[1];
+    sw = warp_sum(sw);
+    nt = __reduce_add_sync(0xffffffffu, nt);
+    if (lane == 0) {
+        sh[wid] = sw;
+        sh_nt[wid] = nt;
+    }
+    __syncthreads();
     if (threadIdx.x == 0) {
+        sw = 0.0;
+        nt = 0;
+#pragma unroll
+        for (int w = 0; w < NW; ++w) {
+            sw += sh[w];
+            nt += sh_nt[w];
+        }
+        part_w = sw;
+        part_nt = nt;
+    }
+    if (nct > 1) cluster_sync();  // every CTA's part is in its shared memory
+    if (rank == 0 && threadIdx.x == 0) {
+        for (int r = 1; r < nct; ++r) {
+            sw += ld_peer_f64(&part_w, uint32_t(r));
+            nt += int(ld_peer_u32(&part_nt, uint32_t(r)));
+        }
         seq[i].n_trunc = nt;
         seq[i].sum_w = sw;
     }
+    if (nct > 1) cluster_sync();  // no CTA leaves while rank 0 may still read its shared memory
 }
 
-// K4c: batch metrics of the controller.
-__global__ void __launch_bounds__(kFinThreads) controller_finalize_kernel(int S, const acrl_seq_stats* __restrict__ seq,
-                                                                          acrl_batch_stats* batch) {
+// K4b: the controller's new state and the batch metrics.
+__global__ void __launch_bounds__(kFinThreads) controller_finalize_kernel(acrl_controller_state* st, acrl_params p,
+                                                                          int S,
+                                                                          const acrl_seq_stats* __restrict__ seq,
+                                                                          acrl_batch_stats* batch, int32_t* flags) {
     constexpr int NW = kFinThreads / 32;
-    __shared__ double sh[NW * 4];
-    long long nt = 0;
-    double sw = 0.0, sa = 0.0;
-    for (int i = threadIdx.x; i < S; i += kFinThreads) {
-        nt += seq[i].n_trunc;
-        sw += seq[i].sum_w;
-        if (seq[i].n > 0) sa += seq[i].alpha;
+    __shared__ double sh[NW * 2];
+    __shared__ long long sh_nt[NW];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int used = min(NW, (S + 31) / 32);  // warps with responses of their own
+    if (wid < used) {
+        long long nt = 0;
+        double sw = 0.0, sa = 0.0;
+        for (int i = threadIdx.x; i < S; i += kFinThreads) {
+            nt += seq[i].n_trunc;
+            sw += seq[i].sum_w;
+            if (seq[i].n > 0) sa += seq[i].alpha;
+        }
+        const double s = warp_sum2(sw, sa);
+        nt = warp_sum(nt);
+        if ((lane & 15) == 0) sh[wid * 2 + (lane >> 4)] = s;
+        if (lane == 0) sh_nt[wid] = nt;
     }
-    double v[3] = {double(nt), sw, sa}, unused = 0.0;
-    block_sums_max0<NW, 3>(v, unused, sh);
-    nt = (long long)v[0];
-    sw = v[1];
-    sa = v[2];
-    if (threadIdx.x == 0) {
-        const double N = double(batch->n_tokens);
-        batch->trunc_frac = N > 0 ? double(nt) / N : 0.0;
-        batch->w_mean = N > 0 ? sw / N : 0.0;
-        batch->alpha_mean = batch->n_seqs_valid > 0 ? sa / batch->n_seqs_valid : 0.0;
+    __syncthreads();
+    if (wid != 0) return;
+    double s = 0.0;  // sum of the weights in lane 0, of alpha in lane 1
+    if (lane < 2)
+        for (int w = 0; w < used; ++w) s += sh[w * 2 + lane];
+    const long long nt = warp_sum(lane < used ? sh_nt[lane] : 0ll);
+    const int ngv = batch->n_groups_valid, nsv = batch->n_seqs_valid;
+    const double Ysum = batch->Y_sum, N = double(batch->n_tokens);
+    ControllerMove mv = controller_move(*st, p, Ysum, ngv);
+    // one division: w_mean, alpha_mean, trunc_frac, Y_mean (of the possibly all-reduced sum and prompt count), X
+    double num = s, den = N;
+    if (lane == 1) den = double(nsv);
+    if (lane == 2) num = double(nt);
+    if (lane == 3) num = Ysum, den = double(ngv);
+    if (lane == 4) num = mv.x_num, den = mv.x_den;
+    const double q = den > 0.0 ? num / den : 0.0;
+    const double a_mean = __shfl_sync(0xffffffffu, q, 1), trunc = __shfl_sync(0xffffffffu, q, 2),
+                 Ymean = __shfl_sync(0xffffffffu, q, 3), X = __shfl_sync(0xffffffffu, q, 4);
+    if (lane == 0) {
+        const bool was_calibrated = st->calibrated != 0;
+        acrl_controller_state n = mv.next;
+        n.X = X;
+        const bool uses_x = p.mode == ACRL_MODE_ACRL || p.mode == ACRL_MODE_ACRL_FALLBACK;
+        if (uses_x && mv.apply && !(X > 0.0)) {
+            raise_flag(flags, ACRL_FLAG_X_NONPOS);
+            n.flags |= ACRL_FLAG_X_NONPOS;
+        }
+        // moving-average X (off by default): this step used X, the next one uses the update
+        if (was_calibrated && p.x_ema > 0.f) n.X = (1.0 - double(p.x_ema)) * X + double(p.x_ema) * Ymean;
+        *st = n;
+        batch->Y_mean = Ymean;
+        batch->X = mv.apply ? X : 0.0;
+        batch->trunc_frac = trunc;
+        batch->w_mean = q;
+        batch->alpha_mean = a_mean;
     }
+}
+
+// CTAs per response: enough to give the chip a few hundred CTAs, while each
+// still has a round of tokens.
+int ctas_per_response(int32_t S, int64_t T) {
+    int c = 1;
+    while (c < 8 && int64_t(S) * c * 2 <= kSeqCtas && T > int64_t(S) * c * kSeqTokens) c *= 2;
+    return c;
+}
+
+// Launch over S responses with a cluster of c CTAs each.
+template <typename... P, typename... A>
+cudaError_t launch_per_response(void (*kernel)(P...), int32_t S, int c, int threads, cudaStream_t s, A... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(unsigned(int64_t(S) * c), 1, 1);
+    cfg.blockDim = dim3(unsigned(threads), 1, 1);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = unsigned(c);
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
 }
 
 }  // namespace
@@ -399,9 +653,10 @@ extern "C" acrl_status acrl_seq_discrepancy(const float* logp_pi, const float* l
     if (T > 0 && (!logp_pi || !logp_mu || !lr || !d)) return ACRL_ERR_INVALID_ARG;
     if ((S > 0 && !seq) || (Gn > 0 && !grp)) return ACRL_ERR_INVALID_ARG;
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-    if (S > 0)
-        seq_stats_kernel<<<S, kSeqThreads, 0, s>>>(logp_pi, logp_mu, mask, T, seq_offsets, S, group_offsets, Gn,
-                                                   entropy, lr, d, seq, dev_flags);
+    if (S > 0 && launch_per_response(seq_stats_kernel, S, ctas_per_response(S, T), kSeqThreads + 32, s, logp_pi, logp_mu,
+                                     mask, T, seq_offsets, S, group_offsets, Gn, entropy, lr, d, seq,
+                                     dev_flags) != cudaSuccess)
+        return launch_failed();
     seq_finalize_kernel<<<1, kFinThreads, 0, s>>>(T, seq_offsets, S, group_offsets, Gn, seq, grp, batch, dev_flags);
     return launch_status();
 }
@@ -453,11 +708,11 @@ extern "C" acrl_status acrl_controller_step(acrl_controller_state* state, const 
     if (T > 0 && (!lr || !weight || !coef)) return ACRL_ERR_INVALID_ARG;
     if ((S > 0 && (!seq || !adv)) || (Gn > 0 && !grp)) return ACRL_ERR_INVALID_ARG;
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-    controller_alpha_kernel<<<1, kFinThreads, 0, s>>>(state, *p, S, Gn, seq, grp, batch, adv, alpha, dev_flags);
-    if (S > 0)
-        controller_weights_kernel<<<S, kSeqThreads, 0, s>>>(*p, lr, mask, T, seq_offsets, Gn, seq, grp, batch, adv,
-                                                            weight, coef, ent_coef);
-    controller_finalize_kernel<<<1, kFinThreads, 0, s>>>(S, seq, batch);
+    if (S > 0 && launch_per_response(controller_weights_kernel, S, ctas_per_response(S, T), kSeqThreads, s, state, *p, lr,
+                                     mask, T, seq_offsets, Gn, seq, grp, batch, adv, weight, coef, alpha,
+                                     ent_coef) != cudaSuccess)
+        return launch_failed();
+    controller_finalize_kernel<<<1, kFinThreads, 0, s>>>(state, *p, S, seq, batch, dev_flags);
     return launch_status();
 }
 

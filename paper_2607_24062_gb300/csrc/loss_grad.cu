@@ -528,61 +528,82 @@ __global__ void __launch_bounds__(THREADS) loss_grad_warp(
                                              RowKeep{nullptr, 0, 0u, 0, nullptr});
 }
 
-// Scalar loss: sum of token losses in a fixed order, by one cluster of
-// kSumCtas CTAs (no scratch memory: the partial sums meet in distributed
-// shared memory).  CTA c sums its contiguous block of the token losses: each
-// thread adds float4 groups (four values in fp32) into two alternating fp64
-// accumulators, so the loads pipeline and the fp64 adds are a quarter of the
-// values; then a fixed CTA tree in fp64 whose cross-warp pass runs in thread 0
-// alone; CTA 0 adds the CTAs' sums in rank order.  Eight CTAs keep eight SMs'
-// loads in flight where one CTA left the reduction latency-bound (T = 524,288:
-// ~75 us on one CTA).
-constexpr int kSumThreads = 1024, kSumCtas = 8;
+// Scalar loss: sum of token losses in a fixed order, by one cluster of CTAs
+// (no scratch memory: the partial sums meet in distributed shared memory).
+// CTA c sums its contiguous block of the token losses: each thread adds float4
+// groups (four values in fp32) into two alternating fp64 accumulators, so the
+// loads pipeline and the fp64 adds are a quarter of the values; then a fixed
+// CTA tree in fp64; CTA 0 adds the CTAs' sums in rank order.  The sum is bound
+// by latency and by the fp64 pipe (two lanes a cycle per SM), which every warp
+// pays five adds of the tree for, so the CTAs have as few warps as keep the
+// loads in flight: XX
+constexpr int kSumCtas = 8;
+constexpr int kSumThreads = 256;
+constexpr int64_t kSumOneCta = 4096;  // up to this many losses are summed by one CTA
 
-__global__ void __cluster_dims__(kSumCtas, 1, 1) __launch_bounds__(kSumThreads)
-    loss_sum_kernel(const float* __restrict__ tl, int64_t T, float* __restrict__ loss) {
-    __shared__ double sh[kSumThreads / 32];
+__global__ void __launch_bounds__(kSumThreads) loss_sum_kernel(const float* __restrict__ tl, int64_t T,
+                                                               float* __restrict__ loss) {
+    constexpr int THREADS = kSumThreads, NW = THREADS / 32;
+    __shared__ double sh[NW];
     __shared__ double cta_sum;
-    const int64_t c = blockIdx.x;   // the launch is one cluster: the block index is the rank
+    const int64_t c = blockIdx.x, ctas = gridDim.x;   // the launch is one cluster: the block index is the rank
     double s0 = 0.0, s1 = 0.0;
     if ((reinterpret_cast<uintptr_t>(tl) & 15u) == 0) {
         const int64_t n4 = T / 4;
-        const int64_t per = (n4 + kSumCtas - 1) / kSumCtas;
+        const int64_t per = (n4 + ctas - 1) / ctas;
         const int64_t lo = min(n4, c * per), hi = min(n4, lo + per);
         const float4* v = reinterpret_cast<const float4*>(tl);
         int64_t i = lo + threadIdx.x;
 #pragma unroll 4
-        for (; i + kSumThreads < hi; i += 2 * kSumThreads) {
-            const float4 a = v[i], b = v[i + kSumThreads];
+        for (; i + THREADS < hi; i += 2 * THREADS) {
+            const float4 a = v[i], b = v[i + THREADS];
             s0 += double((a.x + a.y) + (a.z + a.w));
             s1 += double((b.x + b.y) + (b.z + b.w));
         }
-        for (; i < hi; i += kSumThreads) {
+        for (; i < hi; i += THREADS) {
             const float4 a = v[i];
             s0 += double((a.x + a.y) + (a.z + a.w));
         }
-        if (c == kSumCtas - 1)
-            for (int64_t j = 4 * n4 + threadIdx.x; j < T; j += kSumThreads) s1 += tl[j];
+        if (c == ctas - 1)
+            for (int64_t j = 4 * n4 + threadIdx.x; j < T; j += THREADS) s1 += tl[j];
     } else {
-        const int64_t per = (T + kSumCtas - 1) / kSumCtas;
+        const int64_t per = (T + ctas - 1) / ctas;
         const int64_t lo = min(T, c * per), hi = min(T, lo + per);
-        for (int64_t j = lo + threadIdx.x; j < hi; j += kSumThreads) s0 += tl[j];
+        for (int64_t j = lo + threadIdx.x; j < hi; j += THREADS) s0 += tl[j];
     }
     const double ws = warp_sum(s0 + s1);
     if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = ws;
     __syncthreads();
+    double total = 0.0;
     if (threadIdx.x == 0) {
-        double total = 0.0;
-        for (int w = 0; w < kSumThreads / 32; ++w) total += sh[w];
+#pragma unroll
+        for (int w = 0; w < NW; ++w) total += sh[w];
         cta_sum = total;
     }
-    cluster_sync();   // every CTA's sum is in its shared memory
-    if (c == 0 && threadIdx.x == 0) {
-        double r = 0.0;
-        for (uint32_t k = 0; k < uint32_t(kSumCtas); ++k) r += ld_peer_f64(&cta_sum, k);
-        *loss = float(r);
+    if (ctas > 1) {
+        cluster_sync();   // every CTA's sum is in its shared memory
+        if (c == 0 && threadIdx.x == 0)
+            for (uint32_t k = 1; k < uint32_t(ctas); ++k) total += ld_peer_f64(&cta_sum, k);
     }
-    cluster_sync();   // no CTA leaves while CTA 0 may still read its shared memory
+    if (c == 0 && threadIdx.x == 0) *loss = float(total);
+    if (ctas > 1) cluster_sync();   // no CTA leaves while CTA 0 may still read its shared memory
+}
+
+acrl_status launch_loss_sum(const float* token_loss, int64_t T, float* loss, cudaStream_t s) {
+    const unsigned ctas = T <= kSumOneCta ? 1 : kSumCtas;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(ctas, 1, 1);
+    cfg.blockDim = dim3(kSumThreads, 1, 1);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = ctas;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = ctas > 1 ? 1 : 0;
+    if (cudaLaunchKernelEx(&cfg, loss_sum_kernel, token_loss, T, loss) != cudaSuccess)
+        return launch_failed();
+    return launch_status();
 }
 
 template <bool RECOMPUTE, bool ENT>
@@ -670,12 +691,10 @@ extern "C" acrl_status acrl_loss_grad_logits(const acrl_bf16* logits, int64_t T,
                                               clip_eps, grad, token_loss, dev_flags, s);
         if (st != ACRL_OK) return st;
     }
-    loss_sum_kernel<<<kSumCtas, kSumThreads, 0, s>>>(token_loss, T, loss);
-    return launch_status();
+    return launch_loss_sum(token_loss, T, loss, s);
 }
 
 extern "C" acrl_status acrl_reduce_loss(const float* token_loss, int64_t T, float* loss, acrl_stream stream) {
     if (T < 0 || !loss || (T > 0 && !token_loss)) return ACRL_ERR_INVALID_ARG;
-    loss_sum_kernel<<<kSumCtas, kSumThreads, 0, reinterpret_cast<cudaStream_t>(stream)>>>(token_loss, T, loss);
-    return launch_status();
+    return launch_loss_sum(token_loss, T, loss, reinterpret_cast<cudaStream_t>(stream));
 }

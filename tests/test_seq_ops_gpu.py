@@ -1,0 +1,91 @@
+"""The O(T) calls where their kernels change shape: one CTA per response or a
+cluster of two, four or eight; responses shorter than a round of threads and
+empty ones; more responses than the batch kernel keeps in shared memory; one,
+two and three steps of the prompt search; prompts of one, of a few and of more
+responses than lanes; losses summed by one CTA and by the cluster.  Against
+the float64 oracle, with the bars of the parity tests."""
+
+import numpy as np
+import pytest
+import torch
+
+import oracle as O
+from parity import assert_close_abs, assert_close_rel, compare_batch, compare_grp, compare_seq, host, oracle_params
+
+pytestmark = pytest.mark.gpu
+
+import paper_2607_24062_gb300 as acrl  # noqa: E402
+from paper_2607_24062_gb300 import api  # noqa: E402
+
+DEV = "cuda"
+
+# prompts x responses, lengths lo..hi
+_SHAPES = [(1, 1, 1, 1), (1, 1, 255, 255), (1, 1, 257, 257), (1, 1, 2049, 2049), (1, 3, 0, 1600), (2, 2, 500, 700),
+           (4, 8, 200, 2048), (19, 8, 500, 600), (20, 8, 1, 300), (33, 2, 0, 40), (1025, 2, 0, 9), (1, 70, 1, 30),
+           (5, 33, 1, 20)]
+
+
+def _tokens(Q, G, lo, hi, seed):
+    rng = np.random.default_rng(seed)
+    lengths = rng.integers(lo, hi + 1, size=Q * G)
+    so = np.concatenate([[0], np.cumsum(lengths)])
+    T = int(so[-1])
+    pi = -2.0 * rng.exponential(size=T)
+    mu = np.minimum(pi + 0.05 * rng.normal(size=T), 0.0)
+    mask = (rng.random(T) < 0.9).astype(np.uint8)
+    R = (rng.random(Q * G) < 0.4).astype(np.float32) + rng.integers(0, 3, size=Q * G) / 8.0
+    go = (np.arange(Q + 1) * G).astype(np.int32)
+    f = lambda x, dt: torch.tensor(np.asarray(x), dtype=dt, device=DEV)  # noqa: E731
+    return (f(pi, torch.float32), f(mu, torch.float32), f(mask, torch.uint8), f(so, torch.int64), f(go, torch.int32),
+            f(R, torch.float32), f(rng.random(T), torch.float32))
+
+
+@pytest.mark.parametrize("Q,G,lo,hi", _SHAPES)
+@pytest.mark.parametrize("mode,y_gran", [(acrl.MODE_ACRL, acrl.Y_GROUP), (acrl.MODE_ACRL, acrl.Y_SEQUENCE),
+                                         (acrl.MODE_MIS, acrl.Y_GROUP)])
+def test_shapes_match_oracle(Q, G, lo, hi, mode, y_gran):
+    pi, mu, mask, so, go, R, H = _tokens(Q, G, lo, hi, seed=Q * 1000 + G)
+    p = acrl.Params(mode=mode, y_gran=y_gran, C=1.1)
+    op = oracle_params(p)
+    state, flags = api.controller_init(p), api.new_flags()
+    disc = api.seq_discrepancy(pi, mu, mask, so, go, H, flags=flags)
+    adv = api.grpo_advantage(R, go, p, flags=flags)
+    w, coef, alpha = api.controller_step(state, p, disc, mask, so, go, adv, flags=flags)
+    lr, d, seq, grp, batch, f0 = O.seq_discrepancy(host(pi).astype(np.float64), host(mu).astype(np.float64), host(mask),
+                                                   host(so), host(go), host(H).astype(np.float64))
+    oadv = O.grpo_advantage(host(R).astype(np.float64), host(go), op)
+    ow, oalpha, ost, info, f1 = O.controller_step(O.controller_init(op), op, lr, host(mask), host(so), host(go), seq,
+                                                  grp, batch, oadv)
+    assert api.read_flags(flags) == f0 | f1
+    compare_seq(disc.seq_host(), seq)
+    compare_grp(disc.grp_host(), grp)
+    gb = disc.batch_host()
+    compare_batch(gb, batch)
+    assert_close_rel(host(adv), oadv, floor=1e-6, what="adv")
+    assert_close_rel(host(w), ow, floor=1e-7, what="weight")
+    assert_close_rel(host(alpha), oalpha, floor=1e-6, what="alpha")
+    ocoef = O.loss_coefficients(ow, oadv, host(mask), host(so), seq, grp, batch, op)
+    assert_close_rel(host(coef), ocoef, floor=1e-9, what="coef")
+    gs = disc.seq_host()
+    assert_close_rel(gs["sum_w"], np.array([ow[a:b].sum() for a, b in zip(host(so), host(so)[1:])]), floor=1e-6,
+                     what="sum_w")
+    st = api.read_state(state)
+    assert int(st["step"]) == 1
+    assert_close_rel(st["X"], ost.X, floor=1e-12, what="X")
+    N = max(1, int(host(mask).sum()))
+    assert_close_rel(gb["w_mean"], ow.sum() / N, floor=1e-9, what="w_mean")
+    assert_close_abs(gb["trunc_frac"], info["trunc_frac"], 2.0 / N, what="trunc_frac")   # ties at ln C
+
+
+@pytest.mark.parametrize("T", [0, 1, 3, 255, 1024, 4097, 32768, 32769, 100003, 262147])
+def test_loss_sum_sizes(T):
+    """Sums of T values, from a 16-byte-aligned start and from one that is not."""
+    gen = torch.Generator(device=DEV).manual_seed(T)
+    v = torch.randn(T + 1, generator=gen, device=DEV)
+    for off in (0, 1):
+        x = v[off:off + T]
+        want = float(x.double().sum())
+        # fp32 sums of four values, then fp64: 2 roundings of 2^-24 on a group's partial sums
+        bound = 4 * 2.0 ** -24 * float(x.double().abs().sum()) + 1e-30
+        assert abs(float(api.reduce_loss(x)) - want) <= bound
+        assert torch.equal(api.reduce_loss(x), api.reduce_loss(x))

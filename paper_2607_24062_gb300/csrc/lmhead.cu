@@ -455,7 +455,8 @@ __global__ void lmhead_merge_kernel(const float4* __restrict__ partials, const a
         acc = lse_merge(acc, o);
         mx = fmaxf(mx, __shfl_xor_sync(group, mx, m));
     }
-    if (sub == 0) row_outputs(acc, mx, logits + int64_t(row) * ldl, N, ids[row], lse, logp, ent, row, flags);
+    if (sub == 0)
+        row_outputs(acc, mx, row_target(logits + int64_t(row) * ldl, N, ids[row]), lse, logp, ent, row, flags);
 }
 
 acrl_status launch_merge(const float4* partials, const acrl_bf16* logits, int64_t M, int64_t N, int64_t ldl,

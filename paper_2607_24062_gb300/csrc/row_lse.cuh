@@ -91,20 +91,84 @@ __device__ __forceinline__ LseAcc row_partial(const acrl_bf16* __restrict__ row,
     return acc;
 }
 
+// 16-byte copy from global to shared memory, asynchronous, past L1.
+__device__ __forceinline__ void cp_async16(uint4* dst, const uint4* src) {
+    asm volatile("cp.async.cg.shared.global.L2::256B [%0], [%1], 16;" ::"r"(
+                     static_cast<uint32_t>(__cvta_generic_to_shared(dst))),
+                 "l"(src)
+                 : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait() {
+    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
+// row_partial with DEPTH steps of loads in flight instead of one: each thread
+// copies its own vectors into its own slots of shared memory (slot k of step i
+// at ring[((i mod DEPTH) UNROLL + k) THREADS]), so nothing is shared and no
+// thread waits for another.  The vectors are folded in row_partial's order, so
+// the result is the same to the last bit.
+template <int TEAM, int UNROLL, int THREADS, int DEPTH>
+__device__ __forceinline__ LseAcc row_partial_ring(const acrl_bf16* __restrict__ row, int V, int tid, float& mx,
+                                                   uint4* ring) {
+    constexpr int STEP = TEAM * UNROLL;
+    LseAcc acc = lse_empty();
+    mx = -INFINITY;
+    const int nvec = V >> 3;
+    const uint4* vrow = reinterpret_cast<const uint4*>(row);
+    const int rem = nvec - tid - (UNROLL - 1) * TEAM;
+    const int full = rem > 0 ? (rem + STEP - 1) / STEP : 0;   // steps in which all of this thread's vectors exist
+    auto issue = [&](int i, int slot) {
+        const int v = tid + i * STEP;
+#pragma unroll
+        for (int k = 0; k < UNROLL; ++k)
+            if (i <= full && v + k * TEAM < nvec) cp_async16(ring + (slot * UNROLL + k) * THREADS, vrow + v + k * TEAM);
+        cp_async_commit();
+    };
+#pragma unroll
+    for (int i = 0; i < DEPTH; ++i) issue(i, i);
+    int slot = 0;
+    for (int i = 0; i < full; ++i) {
+        cp_async_wait<DEPTH - 1>();
+        uint4 buf[UNROLL];
+#pragma unroll
+        for (int k = 0; k < UNROLL; ++k) buf[k] = ring[(slot * UNROLL + k) * THREADS];
+        fold_vectors<UNROLL>(acc, mx, buf);
+        issue(i + DEPTH, slot);
+        slot = slot + 1 == DEPTH ? 0 : slot + 1;
+    }
+    cp_async_wait<0>();
+    int v = tid + full * STEP;
+    for (int k = 0; v < nvec; v += TEAM, ++k) {
+        uint4 buf[1] = {ring[(slot * UNROLL + k) * THREADS]};
+        fold_vectors<1>(acc, mx, buf);
+    }
+    for (int j = (nvec << 3) + tid; j < V; j += TEAM) fold_scalar(acc, mx, bf16_to_float(row[j]));
+    return acc;
+}
+
+// The sampled token of a row and its logit, loaded while the row streams.
+struct RowTarget {
+    float z;
+    bool ok;   // the id is inside the vocabulary
+};
+
+__device__ __forceinline__ RowTarget row_target(const acrl_bf16* row, int V, int a) {
+    const bool ok = a >= 0 && a < V;
+    return RowTarget{ok ? bf16_to_float(row[a]) : 0.f, ok};
+}
+
 // Outputs of one row from its merged state; mx is the row maximum (natural units).
-__device__ __forceinline__ void row_outputs(const LseAcc& acc, float mx, const acrl_bf16* row, int V, int a,
-                                            float* lse, float* logp, float* ent, int64_t t, int32_t* flags) {
+__device__ __forceinline__ void row_outputs(const LseAcc& acc, float mx, const RowTarget& tgt, float* lse, float* logp,
+                                            float* ent, int64_t t, int32_t* flags) {
     const float l2s0 = log2f(acc.s0);
     // acc.U is mx*log2(e) rounded; c is that rounding error, exact through the FMA
     const float c = fmaf(mx, kLog2e, -acc.U);
     const float lse_v = fmaf(kLn2, l2s0 - c, mx);
     const float H = kLn2 * (l2s0 - acc.s1 / acc.s0);
-    float lp = 0.f;
-    if (a >= 0 && a < V) {
-        lp = (bf16_to_float(row[a]) - mx) - kLn2 * (l2s0 - c);
-    } else {
-        raise_flag(flags, ACRL_FLAG_BAD_ID);
-    }
+    if (!tgt.ok) raise_flag(flags, ACRL_FLAG_BAD_ID);
+    const float lp = tgt.ok ? (tgt.z - mx) - kLn2 * (l2s0 - c) : 0.f;
     if (!isfinite(lse_v) || !isfinite(H)) {
         raise_flag(flags, ACRL_FLAG_NONFINITE);
         lse[t] = logp[t] = ent[t] = __int_as_float(0x7fc00000);

@@ -1,12 +1,16 @@
 // acrl_token_stats: one streaming pass over pi's bf16 logits per token row
 // giving the log-sum-exp, the sampled token's log-prob and the entropy.
 //
-// Each row is read exactly once from HBM with 16-byte non-allocating loads.
+// Each row is read exactly once from HBM in 16-byte loads that L1 does not keep.
 // A team of threads (eight lanes for rows of up to 4,096 columns, a warp for
 // other short rows, the whole CTA for vocabulary-size rows) owns a row; every
 // thread keeps an online base-2 state (max, sum 2^(u-U), sum 2^(u-U)(u-U))
 // over its strided share of the row, and the team merges the states with a
 // fixed butterfly/tree order, so results are bit-reproducible run to run.
+//
+// A thread's loads go straight into registers (one step of four in flight) or
+// through a ring of kDepth steps in its own slots of shared memory; the fold is
+// the same, so which one a call takes does not show in its results.
 #include "acrl_device.cuh"
 #include "acrl_host.h"
 #include "row_lse.cuh"
@@ -14,16 +18,30 @@
 namespace acrl {
 namespace {
 
+// A thread's share of its team's row: straight into registers (DEPTH = 0), or
+// through a ring of DEPTH steps.
+template <int TEAM, int UNROLL, int THREADS, int DEPTH>
+__device__ __forceinline__ LseAcc team_partial(const acrl_bf16* row, int V, int tid, float& mx, uint4* ring) {
+    if constexpr (DEPTH == 0)
+        return row_partial<TEAM, UNROLL>(row, V, tid, mx);
+    else
+        return row_partial_ring<TEAM, UNROLL, THREADS, DEPTH>(row, V, tid, mx, ring + threadIdx.x);
+}
+
+// The register path lives on residency: 48 registers, 1,280 threads per SM.
+template <int THREADS, int DEPTH>
+constexpr int kMinCtas = DEPTH == 0 && THREADS <= 128 ? 1280 / THREADS : 1;
+
 // A whole CTA per row (vocabulary-size rows).
-template <int THREADS, int UNROLL>
-__global__ void __launch_bounds__(THREADS) token_stats_cta(const acrl_bf16* __restrict__ logits, int64_t T, int V,
-                                                           int64_t ld, const int32_t* __restrict__ ids,
-                                                           const uint8_t* __restrict__ mask, float* __restrict__ lse,
-                                                           float* __restrict__ logp, float* __restrict__ ent,
-                                                           int32_t* flags) {
+template <int THREADS, int UNROLL, int DEPTH>
+__global__ void __launch_bounds__(THREADS, kMinCtas<THREADS, DEPTH>)
+    token_stats_cta(const acrl_bf16* __restrict__ logits, int64_t T, int V, int64_t ld,
+                    const int32_t* __restrict__ ids, const uint8_t* __restrict__ mask, float* __restrict__ lse,
+                    float* __restrict__ logp, float* __restrict__ ent, int32_t* flags) {
     constexpr int NW = THREADS / 32;
     __shared__ LseAcc part[NW];
     __shared__ float pmax[NW];
+    extern __shared__ uint4 ring[];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     for (int64_t t = blockIdx.x; t < T; t += gridDim.x) {
         if (mask && mask[t] == 0) {
@@ -31,8 +49,10 @@ __global__ void __launch_bounds__(THREADS) token_stats_cta(const acrl_bf16* __re
             continue;
         }
         const acrl_bf16* row = logits + t * ld;
+        RowTarget tgt{0.f, false};
+        if (threadIdx.x == 0) tgt = row_target(row, V, ids[t]);
         float mx;
-        LseAcc acc = row_partial<THREADS, UNROLL>(row, V, threadIdx.x, mx);
+        LseAcc acc = team_partial<THREADS, UNROLL, THREADS, DEPTH>(row, V, threadIdx.x, mx, ring);
         acc = warp_lse(acc);
         mx = warp_max(mx);
         if (lane == 0) {
@@ -48,20 +68,21 @@ __global__ void __launch_bounds__(THREADS) token_stats_cta(const acrl_bf16* __re
                 r = lse_merge(r, part[w]);
                 m = fmaxf(m, pmax[w]);
             }
-            row_outputs(r, m, row, V, ids[t], lse, logp, ent, t, flags);
+            row_outputs(r, m, tgt, lse, logp, ent, t, flags);
         }
         __syncthreads();
     }
 }
 
 // One warp per row (short rows); THREADS/32 rows per CTA.
-template <int THREADS, int UNROLL>
+template <int THREADS, int UNROLL, int DEPTH>
 __global__ void __launch_bounds__(THREADS) token_stats_warp(const acrl_bf16* __restrict__ logits, int64_t T, int V,
                                                             int64_t ld, const int32_t* __restrict__ ids,
                                                             const uint8_t* __restrict__ mask, float* __restrict__ lse,
                                                             float* __restrict__ logp, float* __restrict__ ent,
                                                             int32_t* flags) {
     constexpr int NW = THREADS / 32;
+    extern __shared__ uint4 ring[];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     for (int64_t t = int64_t(blockIdx.x) * NW + wid; t < T; t += int64_t(gridDim.x) * NW) {
         if (mask && mask[t] == 0) {
@@ -69,11 +90,13 @@ __global__ void __launch_bounds__(THREADS) token_stats_warp(const acrl_bf16* __r
             continue;
         }
         const acrl_bf16* row = logits + t * ld;
+        RowTarget tgt{0.f, false};
+        if (lane == 0) tgt = row_target(row, V, ids[t]);
         float mx;
-        LseAcc acc = row_partial<32, UNROLL>(row, V, lane, mx);
+        LseAcc acc = team_partial<32, UNROLL, THREADS, DEPTH>(row, V, lane, mx, ring);
         acc = warp_lse(acc);
         mx = warp_max(mx);
-        if (lane == 0) row_outputs(acc, mx, row, V, ids[t], lse, logp, ent, t, flags);
+        if (lane == 0) row_outputs(acc, mx, tgt, lse, logp, ent, t, flags);
     }
 }
 
@@ -96,13 +119,14 @@ __device__ __forceinline__ float team_max(float v) {
     return v;
 }
 
-template <int THREADS, int UNROLL, int LANES>
+template <int THREADS, int UNROLL, int LANES, int DEPTH>
 __global__ void __launch_bounds__(THREADS) token_stats_team(const acrl_bf16* __restrict__ logits, int64_t T, int V,
                                                             int64_t ld, const int32_t* __restrict__ ids,
                                                             const uint8_t* __restrict__ mask, float* __restrict__ lse,
                                                             float* __restrict__ logp, float* __restrict__ ent,
                                                             int32_t* flags) {
     constexpr int NW = THREADS / 32, RPW = 32 / LANES;
+    extern __shared__ uint4 ring[];
     static_assert(LANES >= 2 && LANES <= 32 && (LANES & (LANES - 1)) == 0, "lanes per row");
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, tl = lane % LANES;
     for (int64_t base = (int64_t(blockIdx.x) * NW + wid) * RPW; base < T; base += int64_t(gridDim.x) * NW * RPW) {
@@ -110,18 +134,55 @@ __global__ void __launch_bounds__(THREADS) token_stats_team(const acrl_bf16* __r
         const bool in = t < T;
         const bool live = in && !(mask && mask[t] == 0);
         const acrl_bf16* row = logits + (in ? t : 0) * ld;
+        RowTarget tgt{0.f, false};
+        if (tl == 0 && live) tgt = row_target(row, V, ids[t]);
         LseAcc acc = lse_empty();
         float mx = -INFINITY;
-        if (live) acc = row_partial<LANES, UNROLL>(row, V, tl, mx);
+        if (live) acc = team_partial<LANES, UNROLL, THREADS, DEPTH>(row, V, tl, mx, ring);
         acc = team_lse<LANES>(acc);
         mx = team_max<LANES>(mx);
         if (tl == 0 && in) {
             if (live)
-                row_outputs(acc, mx, row, V, ids[t], lse, logp, ent, t, flags);
+                row_outputs(acc, mx, tgt, lse, logp, ent, t, flags);
             else
                 lse[t] = logp[t] = ent[t] = 0.f;
         }
     }
+}
+
+// Rows up to this many columns (8 KB) are shared by eight lanes each, up to
+// kWarpRowMaxV by a warp, up to kMidRowMaxV (128 KB) by two warps (2 % faster
+// than four at V = 32,000), longer ones by four: many independent rows in
+// flight per SM and a short end-of-row merge (measured best of teams of 8 to
+// 1,024 threads).
+constexpr int64_t kTeamRowMaxV = 4096, kMidRowMaxV = 65536;
+constexpr int kUnroll = 4;
+
+// Steps of the ring: with few rows per SM, one step of loads per thread leaves
+// the memory system idle between steps (V = 151,936, T = 64: 30 us in
+// registers, 19 / 14.4 / 13.8 us with rings of 2 / 3 / 4 steps; T = 408: 34
+// against 26 / 23 / 23; V = 4,096, T = 1,024: 15 against 6.6 / 6.5 / 6.3).
+constexpr int kDepth = 3;
+
+// Ring or registers?  The line is drawn in 128-thread teams per SM (q: tenths).
+// - Few teams per SM: the ring, up to 2.3 x (above).
+// - 5.2 to 10.4 per SM: all of them fit in one wave of the register path (48
+//   registers), not in one of the ring's (64); V = 151,936, T = 1,216: 59 us in
+//   registers against 64, T = 1,600 (past the wave): 93 against 82.  A warp per
+//   row: only up to 7.5 (V = 16,384, T = 4,096: 25.8 against 26.5).
+// - Many: the ring for rows of a warp or less (V = 16,384, T = 65,536: 296 us
+//   against 317; V = 8,192: 153 against 162; V = 4,096: 82 against 88), the
+//   same for four warps a row; registers for two warps a row (V = 20,011,
+//   T = 65,536: 389 against 402; 49,152, T = 40,000: 548 against 553), except
+//   just past one wave (V = 32,000, T = 3,500: 45 against 40).
+bool use_ring(int64_t T, int team) {
+    constexpr int64_t kSms = 152;
+    const int64_t q = T >= (int64_t(1) << 40) ? INT64_MAX : T * team * 10 / (128 * kSms);
+    if (team == 8) return true;
+    if (q < 52) return true;
+    if (team == 32) return q > 75;
+    if (team == 64) return q > 104 && q < 140;
+    return q > 104;
 }
 
 }  // namespace
@@ -129,12 +190,6 @@ __global__ void __launch_bounds__(THREADS) token_stats_team(const acrl_bf16* __r
 }  // namespace acrl
 
 using namespace acrl;
-
-// Rows up to this many columns (8 KB) are shared by eight lanes each.
-constexpr int64_t kTeamRowMaxV = 4096;
-
-// Rows up to this many columns (128 KB) use two warps each.
-constexpr int64_t kMidRowMaxV = 65536;
 
 extern "C" acrl_status acrl_token_stats(const acrl_bf16* logits, int64_t T, int64_t V, int64_t ld,
                                         const int32_t* ids, const uint8_t* mask, float* lse, float* logp,
@@ -145,25 +200,21 @@ extern "C" acrl_status acrl_token_stats(const acrl_bf16* logits, int64_t T, int6
     if (!aligned16(logits)) return ACRL_ERR_INVALID_ARG;
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     const int v = int(V);
-    if (V <= kTeamRowMaxV) {
-        constexpr int THREADS = 256, LANES = 8;
-        token_stats_team<THREADS, 4, LANES><<<unsigned(grid_for(THREADS / LANES, T)), THREADS, 0, s>>>(
+    // `depth` steps of kUnroll 16-byte slots per thread of dynamic shared memory (at most 24 KB)
+    auto launch = [&](auto kernel, int threads, int depth, int64_t rows_per_cta) {
+        kernel<<<unsigned(grid_for(rows_per_cta, T)), threads, size_t(threads) * kUnroll * depth * 16, s>>>(
             logits, T, v, ld, ids, mask, lse, logp, entropy, dev_flags);
-    } else if (V <= kWarpRowMaxV) {
-        constexpr int THREADS = 256;
-        token_stats_warp<THREADS, 4><<<unsigned(grid_for(THREADS / 32, T)), THREADS, 0, s>>>(
-            logits, T, v, ld, ids, mask, lse, logp, entropy, dev_flags);
-    } else if (V <= kMidRowMaxV) {
-        // rows of up to 128 KB: two warps per row (measured 2 % faster than four at V = 32,000)
-        constexpr int THREADS = 64;
-        token_stats_cta<THREADS, 4><<<unsigned(grid_for(1, T)), THREADS, 0, s>>>(
-            logits, T, v, ld, ids, mask, lse, logp, entropy, dev_flags);
-    } else {
-        // 128 threads per row: many independent rows in flight per SM and a short
-        // end-of-row merge (measured best of 64/128/256/512/1024 and a warp per row)
-        constexpr int THREADS = 128;
-        token_stats_cta<THREADS, 4><<<unsigned(grid_for(1, T)), THREADS, 0, s>>>(
-            logits, T, v, ld, ids, mask, lse, logp, entropy, dev_flags);
-    }
-    return launch_status();
+        return launch_status();
+    };
+    const int team = V <= kTeamRowMaxV ? 8 : V <= kWarpRowMaxV ? 32 : V <= kMidRowMaxV ? 64 : 128;
+    const bool ring = use_ring(T, team);
+    if (team == 8) return launch(token_stats_team<64, kUnroll, 8, kDepth>, 64, kDepth, 8);
+    if (team == 32)
+        return ring ? launch(token_stats_warp<64, kUnroll, kDepth>, 64, kDepth, 2)
+                    : launch(token_stats_warp<256, kUnroll, 0>, 256, 0, 8);
+    if (team == 64)
+        return ring ? launch(token_stats_cta<64, kUnroll, kDepth>, 64, kDepth, 1)
+                    : launch(token_stats_cta<64, kUnroll, 0>, 64, 0, 1);
+    return ring ? launch(token_stats_cta<128, kUnroll, kDepth>, 128, kDepth, 1)
+                : launch(token_stats_cta<128, kUnroll, 0>, 128, 0, 1);
 }

@@ -1,0 +1,72 @@
+"""acrl_token_stats where its load path or its row team changes: a call of few
+rows (ring of loads in shared memory) and a call of many rows that takes the
+register path give the same rows the same bits, at row lengths around a whole
+step of the team's loads, around whole rings and around whole vectors; and
+both agree with a float64 log-softmax."""
+
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+from paper_2607_24062_gb300 import api  # noqa: E402
+
+DEV = "cuda"
+
+# team of 8: steps of 256 columns; 32: 1,024; 64: 2,048; 128: 4,096
+_WIDTHS = [1, 8, 63, 64, 255, 256, 257, 767, 768, 769, 1024, 4095, 4096, 4097, 5119, 5120, 5121, 7168, 16383, 16384, 16385,
+           18431, 18432, 18441, 20011, 32000, 65535, 65536, 65537, 65544, 69632, 69640, 100003, 151936]
+
+
+def _many(V):
+    """Rows that put the call on the register path (teams per SM between 5.2 and 7.5)."""
+    team = 8 if V <= 4096 else 32 if V <= 16384 else 64 if V <= 65536 else 128
+    return 6 * 128 * 152 // team if team > 8 else 4096
+
+
+@pytest.mark.parametrize("V", _WIDTHS)
+def test_few_and_many_rows_agree(V):
+    gen = torch.Generator(device=DEV).manual_seed(V)
+    R, ld = 5, (V + 7) // 8 * 8
+    base = torch.full((R, ld), float("nan"), dtype=torch.bfloat16, device=DEV)   # columns past V are never read
+    base[:, :V] = torch.randn((R, V), generator=gen, device=DEV) * 3
+    base[1, V // 2] = 40.0
+    base[2, :V] = -3.0
+    ids = torch.randint(0, V, (R,), generator=gen, device=DEV, dtype=torch.int32)
+    mask = torch.tensor([1, 1, 1, 0, 1], dtype=torch.uint8, device=DEV)
+    flags = api.new_flags()
+    few = api.token_stats(base, ids, mask, V=V, flags=flags)
+    T = _many(V)
+    pick = torch.arange(T, device=DEV) % R
+    many = api.token_stats(base[pick], ids[pick], mask[pick], V=V, flags=flags)
+    assert api.read_flags(flags) == 0
+    for a, b in zip(few, many):
+        assert torch.equal(a[pick].view(torch.int32), b.view(torch.int32))
+    z = base[:, :V].double()
+    lse = z.logsumexp(dim=1)
+    lp = z - lse[:, None]
+    want = (lse, lp.gather(1, ids.long()[:, None])[:, 0], -(lp.exp() * lp).sum(dim=1))
+    live = mask.bool()
+    for got, ref in zip(few, want):
+        assert float((got.double() - ref)[live].abs().max()) <= 2e-5 * max(1.0, float(ref[live].abs().max()))
+        assert float(got[3]) == 0.0
+
+
+@pytest.mark.parametrize("V", [256, 5000, 20011, 100003])
+def test_undefined_rows_and_bad_ids(V):
+    """NaN and infinities anywhere in the row, ids outside the vocabulary, on the ring path."""
+    ld = (V + 7) // 8 * 8
+    spots = [0, V // 3, V - 1]
+    rows = torch.zeros((3 * len(spots) + 2, ld), dtype=torch.bfloat16, device=DEV)
+    for k, bad in enumerate((float("nan"), float("inf"), float("-inf"))):
+        for j, c in enumerate(spots):
+            rows[k * len(spots) + j, c] = bad
+    T = rows.shape[0]
+    ids = torch.zeros(T, dtype=torch.int32, device=DEV)
+    ids[-2], ids[-1] = V, -1
+    flags = api.new_flags()
+    lse, logp, ent = api.token_stats(rows, ids, None, V=V, flags=flags)
+    assert api.read_flags(flags) == 0x3       # BAD_ID and NONFINITE
+    for x in (lse, logp, ent):
+        assert bool(x[:-2].isnan().all()) and not bool(x[-2:].isnan().any())
+    assert float(logp[-2]) == 0.0 and float(logp[-1]) == 0.0

@@ -422,48 +422,81 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     }
 }
 
-// Merge of the per-tile states of each row: lse, logp and entropy.  Eight
-// lanes per row, lane j folding tiles j, j+8, ... in order, then a fixed
-// butterfly over the eight (deterministic); partials are [n_tiles][M].
-constexpr int kMergeLanes = 8;
+// Merge of the per-tile states of each row: lse, logp and entropy; partials
+// are [n_tiles][M].  A CTA takes eight rows with 32 lanes each: lane j of a row
+// folds tiles j, j + 32, ... in order, kMergeLoads states in flight, then a
+// fixed tree over the 32 (the order depends on N alone).  Eight rows of states
+// are one 128-byte line of `partials`.  Latency bounds it at small M (a serial
+// chain of loads: eight lanes a row, one load at a time, took 46 us for 48 rows
+// of 594 tiles, now 8.6), the states' 16 bytes per row and tile at large M (4,096
+// rows: 50 -> 12 us).
+constexpr int kMergeRows = 8, kMergeLanes = 32, kMergeThreads = kMergeRows * kMergeLanes, kMergeLoads = 5;
 
-__global__ void lmhead_merge_kernel(const float4* __restrict__ partials, const acrl_bf16* __restrict__ logits, int M,
-                                    int N, int64_t ldl, int n_tiles, const int32_t* __restrict__ ids,
-                                    const uint8_t* __restrict__ mask, float* __restrict__ lse, float* __restrict__ logp,
-                                    float* __restrict__ ent, int32_t* flags) {
-    const int64_t g = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-    const int row = int(g / kMergeLanes), sub = int(g % kMergeLanes);
-    if (row >= M) return;  // the row's eight lanes leave together
-    if (mask && mask[row] == 0) {
-        if (sub == 0) lse[row] = logp[row] = ent[row] = 0.f;
-        return;
-    }
+__global__ void __launch_bounds__(kMergeThreads)
+    lmhead_merge_kernel(const float4* __restrict__ partials, const acrl_bf16* __restrict__ logits, int M, int N,
+                        int64_t ldl, int n_tiles, const int32_t* __restrict__ ids, const uint8_t* __restrict__ mask,
+                        float* __restrict__ lse, float* __restrict__ logp, float* __restrict__ ent, int32_t* flags) {
+    constexpr int NW = kMergeThreads / 32;
+    __shared__ float4 part[NW * kMergeRows];   // (U, s0, s1, max) per warp and row
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int r = lane % kMergeRows, j = wid * (32 / kMergeRows) + lane / kMergeRows;
+    const int64_t row = int64_t(blockIdx.x) * kMergeRows + r;
+    const bool in = row < M;
+    const bool live = in && !(mask && mask[row] == 0);
+    RowTarget tgt{0.f, false};
+    if (live && j == 0) tgt = row_target(logits + row * ldl, N, ids[row]);
     LseAcc acc = lse_empty();
     float mx = -INFINITY;
-#pragma unroll 1  // tiles
-    for (int n = sub; n < n_tiles; n += kMergeLanes) {
-        const float4 p = partials[int64_t(n) * M + row];
-        acc = lse_merge(acc, LseAcc{p.y, p.z, p.w});
-        mx = fmaxf(mx, p.x);
-    }
-    static_assert(kMergeLanes >= 2 && kMergeLanes <= 16 && (kMergeLanes & (kMergeLanes - 1)) == 0, "lanes per row");
-    const unsigned group = ((1u << kMergeLanes) - 1u) << (threadIdx.x & 31 & ~(kMergeLanes - 1));
+    if (live) {
+        const float4* p = partials + row;
+        for (int n = j; n < n_tiles; n += kMergeLoads * kMergeLanes) {
+            float4 f[kMergeLoads];
 #pragma unroll
-    for (int m = kMergeLanes / 2; m >= 1; m >>= 1) {
-        const LseAcc o{__shfl_xor_sync(group, acc.U, m), __shfl_xor_sync(group, acc.s0, m),
-                       __shfl_xor_sync(group, acc.s1, m)};
-        acc = lse_merge(acc, o);
-        mx = fmaxf(mx, __shfl_xor_sync(group, mx, m));
+            for (int k = 0; k < kMergeLoads; ++k) {
+                const int nk = n + k * kMergeLanes;
+                f[k] = nk < n_tiles ? __ldcs(p + int64_t(nk) * M) : make_float4(-INFINITY, -INFINITY, 0.f, 0.f);
+            }
+#pragma unroll
+            for (int k = 0; k < kMergeLoads; ++k) {
+                if (n + k * kMergeLanes >= n_tiles) break;
+                acc = lse_merge(acc, LseAcc{f[k].y, f[k].z, f[k].w});
+                mx = fmaxf(mx, f[k].x);
+            }
+        }
     }
-    if (sub == 0)
-        row_outputs(acc, mx, row_target(logits + int64_t(row) * ldl, N, ids[row]), lse, logp, ent, row, flags);
+#pragma unroll
+    for (int m = kMergeRows; m < 32; m <<= 1) {  // the warp's lanes of one row
+        acc = lse_merge(acc, shfl_xor(acc, m));
+        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, m));
+    }
+    if (lane < kMergeRows) part[wid * kMergeRows + lane] = make_float4(acc.U, acc.s0, acc.s1, mx);
+    __syncthreads();
+    if (wid != 0) return;
+    // warp 0: lane (j, r) takes warps j and j + 4, then the four lanes of a row meet
+    static_assert(NW == 8 && kMergeRows == 8, "two warps' states per lane");
+    float4 f = part[j * kMergeRows + r];
+    acc = LseAcc{f.x, f.y, f.z};
+    mx = f.w;
+    f = part[(j + 4) * kMergeRows + r];
+    acc = lse_merge(acc, LseAcc{f.x, f.y, f.z});
+    mx = fmaxf(mx, f.w);
+#pragma unroll
+    for (int m = kMergeRows; m < 32; m <<= 1) {
+        acc = lse_merge(acc, shfl_xor(acc, m));
+        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, m));
+    }
+    if (j == 0 && in) {
+        if (live)
+            row_outputs(acc, mx, tgt, lse, logp, ent, row, flags);
+        else
+            lse[row] = logp[row] = ent[row] = 0.f;
+    }
 }
 
 acrl_status launch_merge(const float4* partials, const acrl_bf16* logits, int64_t M, int64_t N, int64_t ldl,
                          const int32_t* ids, const uint8_t* mask, float* lse, float* logp, float* entropy,
                          int32_t* flags, cudaStream_t s) {
-    const int threads = 256, rows_per_block = threads / kMergeLanes;
-    lmhead_merge_kernel<<<unsigned((M + rows_per_block - 1) / rows_per_block), threads, 0, s>>>(
+    lmhead_merge_kernel<<<unsigned((M + kMergeRows - 1) / kMergeRows), kMergeThreads, 0, s>>>(
         partials, logits, int(M), int(N), ldl, int((N + kBN - 1) / kBN), ids, mask, lse, logp, entropy, flags);
     return launch_status();
 }

@@ -25,11 +25,31 @@ inline acrl_status launch_status() {
     return cudaGetLastError() == cudaSuccess ? ACRL_OK : ACRL_ERR_CUDA;
 }
 
-// Status of a launch call that returned an error (which is cleared, as
-// launch_status does).
-inline acrl_status launch_failed() {
-    (void)cudaGetLastError();
-    return ACRL_ERR_CUDA;
+// Every kernel of the path is launched here, with programmatic dependent launch: it may
+// start while the previous kernel of the stream is still running, and every
+// kernel therefore begins with grid_begin(), which lets the next one start and
+// then waits until everything before it has completed.  That hides most of the
+// launch latency between the path's short kernels; against a predecessor that
+// is no kernel of this library it is an ordinary launch.  `cluster` CTAs form a
+// cluster (0: as the kernel declares).  An error is cleared as launch_status does.
+template <typename... P, typename... A>
+acrl_status launch(void (*kernel)(P...), int64_t grid, int threads, size_t smem, int cluster, cudaStream_t s,
+                   const A&... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(unsigned(grid), 1, 1);
+    cfg.blockDim = dim3(unsigned(threads), 1, 1);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = unsigned(cluster);
+    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = cluster > 1 ? 2 : 1;
+    (void)cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+    return launch_status();
 }
 
 inline bool params_ok(const acrl_params* p) {

@@ -394,6 +394,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmB)) : "memory");
         asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmC)) : "memory");
     }
+    grid_begin();
     if (warp == 2) {  // one warp of each CTA of the pair allocates, together
         asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&bars->tmem_base)),
                      "r"(kTmemCols)
@@ -441,6 +442,7 @@ __global__ void __launch_bounds__(kMergeThreads)
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int r = lane % kMergeRows, j = wid * (32 / kMergeRows) + lane / kMergeRows;
     const int64_t row = int64_t(blockIdx.x) * kMergeRows + r;
+    grid_begin();
     const bool in = row < M;
     const bool live = in && !(mask && mask[row] == 0);
     RowTarget tgt{0.f, false};
@@ -496,9 +498,8 @@ __global__ void __launch_bounds__(kMergeThreads)
 acrl_status launch_merge(const float4* partials, const acrl_bf16* logits, int64_t M, int64_t N, int64_t ldl,
                          const int32_t* ids, const uint8_t* mask, float* lse, float* logp, float* entropy,
                          int32_t* flags, cudaStream_t s) {
-    lmhead_merge_kernel<<<unsigned((M + kMergeRows - 1) / kMergeRows), kMergeThreads, 0, s>>>(
-        partials, logits, int(M), int(N), ldl, int((N + kBN - 1) / kBN), ids, mask, lse, logp, entropy, flags);
-    return launch_status();
+    return launch(lmhead_merge_kernel, (M + kMergeRows - 1) / kMergeRows, kMergeThreads, 0, 0, s, partials, logits, int(M),
+                  int(N), ldl, int((N + kBN - 1) / kBN), ids, mask, lse, logp, entropy, flags);
 }
 
 bool encode_map(CUtensorMap* map, const void* ptr, uint64_t rows, uint64_t cols, uint64_t ld, uint32_t box_rows,
@@ -543,8 +544,7 @@ acrl_status launch_lmhead(const acrl_bf16* hidden, int64_t M, int64_t K, int64_t
     if (cudaOccupancyMaxActiveClusters(&clusters, lmhead_kernel, &cfg) != cudaSuccess || clusters < 1)
         return ACRL_ERR_CUDA;
     const int grid = int(2 * (total < clusters ? total : clusters));
-    lmhead_kernel<<<grid, kThreads, kSmemBytes, s>>>(tmA, tmB, tmC, int(M), int(N), int(K), partials, flags);
-    return launch_status();
+    return launch(lmhead_kernel, grid, kThreads, kSmemBytes, 0, s, tmA, tmB, tmC, int(M), int(N), int(K), partials, flags);
 }
 
 // True when every pointer is device memory of the current device: not managed

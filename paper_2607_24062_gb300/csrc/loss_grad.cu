@@ -464,6 +464,7 @@ __global__ void __launch_bounds__(THREADS) loss_grad_cta(
     const int warp = threadIdx.x >> 5;
     static_assert(!TM || (RECOMPUTE && THREADS == kCtaThreads && UNROLL == kCtaUnroll), "tensor-memory layout");
     RowKeep kp{keep, 0, 0u, 0, &keep_bar};
+    grid_begin();
     if (RECOMPUTE) {
         const int nvec = V >> 3;
         kp.s = min(kKeepOf<THREADS>, nvec);
@@ -522,6 +523,7 @@ __global__ void __launch_bounds__(THREADS) loss_grad_warp(
     constexpr int NW = THREADS / 32;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     int par = 0;
+    grid_begin();
     for (int64_t t = int64_t(blockIdx.x) * NW + wid; t < T; t += int64_t(gridDim.x) * NW)
         grad_row<32, UNROLL, RECOMPUTE, ENT, false>(logits, t, V, ld, ids, mask, lse, old_logp, coef, entropy, ent_coef, eps,
                                              grad, token_loss, flags, lane, nullptr, nullptr, par,
@@ -548,6 +550,7 @@ __global__ void __launch_bounds__(kSumThreads) loss_sum_kernel(const float* __re
     __shared__ double cta_sum;
     const int64_t c = blockIdx.x, ctas = gridDim.x;   // the launch is one cluster: the block index is the rank
     double s0 = 0.0, s1 = 0.0;
+    grid_begin();
     if ((reinterpret_cast<uintptr_t>(tl) & 15u) == 0) {
         const int64_t n4 = T / 4;
         const int64_t per = (n4 + ctas - 1) / ctas;
@@ -590,20 +593,8 @@ __global__ void __launch_bounds__(kSumThreads) loss_sum_kernel(const float* __re
 }
 
 acrl_status launch_loss_sum(const float* token_loss, int64_t T, float* loss, cudaStream_t s) {
-    const unsigned ctas = T <= kSumOneCta ? 1 : kSumCtas;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(ctas, 1, 1);
-    cfg.blockDim = dim3(kSumThreads, 1, 1);
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = ctas;
-    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = ctas > 1 ? 1 : 0;
-    if (cudaLaunchKernelEx(&cfg, loss_sum_kernel, token_loss, T, loss) != cudaSuccess)
-        return launch_failed();
-    return launch_status();
+    const int ctas = T <= kSumOneCta ? 1 : kSumCtas;
+    return launch(loss_sum_kernel, ctas, kSumThreads, 0, ctas, s, token_loss, T, loss);
 }
 
 template <bool RECOMPUTE, bool ENT>
@@ -611,49 +602,27 @@ acrl_status launch_loss_grad(const acrl_bf16* logits, int64_t T, int V, int64_t 
                              const uint8_t* mask, const float* lse, const float* old_logp, const float* coef,
                              const float* entropy, const float* ent_coef, float eps, acrl_bf16* grad,
                              float* token_loss, int32_t* flags, cudaStream_t s) {
-    if (V <= (RECOMPUTE ? kRecomputeWarpMaxV : kWarpRowMaxV)) {
-        constexpr int THREADS = 256;
-        loss_grad_warp<THREADS, 4, RECOMPUTE, ENT><<<unsigned(grid_for(THREADS / 32, T)), THREADS, 0, s>>>(
-            logits, T, V, ld, ids, mask, lse, old_logp, coef, entropy, ent_coef, eps, grad, token_loss, flags);
-    } else if (!RECOMPUTE && V >= kWideRowMinV) {
-        loss_grad_cta<kWideThreads, kCtaUnroll, false, ENT><<<unsigned(grid_for(1, T)), kWideThreads, 0, s>>>(
-            logits, T, V, ld, ids, mask, lse, old_logp, coef, entropy, ent_coef, eps, grad, token_loss, flags);
-    } else if (RECOMPUTE && (V >> 3) <= kTinyMaxVecs) {
-        if constexpr (RECOMPUTE) {
-            auto kernel = loss_grad_cta<kTinyThreads, kCtaUnroll, true, ENT>;
-            const int smem = 16 * min(V >> 3, kTinyKeepVecs);
-            if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
-                return ACRL_ERR_CUDA;
-            kernel<<<unsigned(grid_for(1, T)), kTinyThreads, smem, s>>>(
-                logits, T, V, ld, ids, mask, lse, old_logp, coef, entropy, ent_coef, eps, grad, token_loss, flags);
-        }
-    } else if (RECOMPUTE && (V >> 3) <= kSmallMaxVecs) {
-        if constexpr (RECOMPUTE) {
-            auto kernel = loss_grad_cta<kSmallThreads, kCtaUnroll, true, ENT>;
-            const int smem = 16 * min(V >> 3, kSmallKeepVecs);
-            if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
-                return ACRL_ERR_CUDA;
-            kernel<<<unsigned(grid_for(1, T)), kSmallThreads, smem, s>>>(
-                logits, T, V, ld, ids, mask, lse, old_logp, coef, entropy, ent_coef, eps, grad, token_loss, flags);
-        }
-    } else if (RECOMPUTE && (V >> 3) >= kTmemMinVecs) {
-        if constexpr (RECOMPUTE) {
-            auto kernel = loss_grad_cta<kCtaThreads, kCtaUnroll, true, ENT, true>;
-            const int smem = 16 * kKeepVecs;
-            if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
-                return ACRL_ERR_CUDA;
-            kernel<<<unsigned(grid_for(1, T)), kCtaThreads, smem, s>>>(
-                logits, T, V, ld, ids, mask, lse, old_logp, coef, entropy, ent_coef, eps, grad, token_loss, flags);
-        }
-    } else {
-        auto kernel = loss_grad_cta<kCtaThreads, kCtaUnroll, RECOMPUTE, ENT>;
-        const int smem = RECOMPUTE ? 16 * (V >> 3 < kKeepVecs ? V >> 3 : kKeepVecs) : 0;
+    auto run = [&](auto kernel, int64_t rows_per_cta, int threads, int keep_vecs) {
+        const int smem = 16 * min(V >> 3, keep_vecs);
         if (smem > 0 && cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
             return ACRL_ERR_CUDA;
-        kernel<<<unsigned(grid_for(1, T)), kCtaThreads, smem, s>>>(logits, T, V, ld, ids, mask, lse, old_logp, coef,
-                                                                   entropy, ent_coef, eps, grad, token_loss, flags);
+        return launch(kernel, grid_for(rows_per_cta, T), threads, size_t(smem), 0, s, logits, T, V, ld, ids, mask, lse,
+                      old_logp, coef, entropy, ent_coef, eps, grad, token_loss, flags);
+    };
+    constexpr int U = kCtaUnroll;
+    if constexpr (RECOMPUTE) {
+        const int nvec = V >> 3;
+        if (V <= kRecomputeWarpMaxV) return run(loss_grad_warp<256, U, true, ENT>, 8, 256, 0);
+        if (nvec <= kTinyMaxVecs) return run(loss_grad_cta<kTinyThreads, U, true, ENT>, 1, kTinyThreads, kTinyKeepVecs);
+        if (nvec <= kSmallMaxVecs)
+            return run(loss_grad_cta<kSmallThreads, U, true, ENT>, 1, kSmallThreads, kSmallKeepVecs);
+        if (nvec >= kTmemMinVecs) return run(loss_grad_cta<kCtaThreads, U, true, ENT, true>, 1, kCtaThreads, kKeepVecs);
+        return run(loss_grad_cta<kCtaThreads, U, true, ENT>, 1, kCtaThreads, kKeepVecs);
+    } else {
+        if (V <= kWarpRowMaxV) return run(loss_grad_warp<256, U, false, ENT>, 8, 256, 0);
+        if (V >= kWideRowMinV) return run(loss_grad_cta<kWideThreads, U, false, ENT>, 1, kWideThreads, 0);
+        return run(loss_grad_cta<kCtaThreads, U, false, ENT>, 1, kCtaThreads, 0);
     }
-    return ACRL_OK;
 }
 
 }  // namespace

@@ -83,6 +83,7 @@ __global__ void __launch_bounds__(kSeqThreads + 32) seq_stats_kernel(
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int nct = int(cluster_size()), rank = int(cluster_rank());
     const int i = int(blockIdx.x) / nct;
+    grid_begin();
     if (wid == NW) {
         if (rank == 0) {
             const int g = group_of(goff, Gn, i);
@@ -206,6 +207,7 @@ __global__ void __launch_bounds__(kFinThreads) seq_finalize_kernel(
     __shared__ float sh_max[NW];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const bool keep = S <= kFinSeqs;
+    grid_begin();
     bool bad = false;
     long long N = 0;
     int sv = 0;
@@ -327,6 +329,7 @@ __global__ void grpo_kernel(const float* __restrict__ R, const int32_t* __restri
     const int64_t tid = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
     const int64_t g = tid / LANES;
     const int sub = int(tid % LANES);
+    grid_begin();
     if (g >= Gn) return;  // the prompt's lanes leave together
     const unsigned team = LANES == 1 ? 0u : ((1u << LANES) - 1u) << (threadIdx.x & 31 & ~(LANES - 1));
     const int b = goff[g], e = goff[g + 1];
@@ -376,6 +379,7 @@ __global__ void grpo_kernel(const float* __restrict__ R, const int32_t* __restri
 }
 
 __global__ void controller_init_kernel(acrl_controller_state* st, double X_init) {
+    grid_begin();
     acrl_controller_state s;
     s.X = X_init > 0.0 ? X_init : 0.0;
     s.calib_sum = 0.0;
@@ -440,6 +444,7 @@ __global__ void __launch_bounds__(kSeqThreads) controller_weights_kernel(
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int nct = int(cluster_size()), rank = int(cluster_rank());
     const int i = int(blockIdx.x) / nct;
+    grid_begin();
     int64_t lo, hi;
     if (!seq_range(so, i, T, lo, hi)) lo = hi = 0;
     const float logC = logf(p.C);
@@ -591,6 +596,7 @@ __global__ void __launch_bounds__(kFinThreads) controller_finalize_kernel(acrl_c
     __shared__ long long sh_nt[NW];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int used = min(NW, (S + 31) / 32);  // warps with responses of their own
+    grid_begin();
     if (wid < used) {
         long long nt = 0;
         double sw = 0.0, sa = 0.0;
@@ -650,22 +656,6 @@ int ctas_per_response(int32_t S, int64_t T) {
     return c;
 }
 
-// Launch over S responses with a cluster of c CTAs each.
-template <typename... P, typename... A>
-cudaError_t launch_per_response(void (*kernel)(P...), int32_t S, int c, int threads, cudaStream_t s, A... args) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(unsigned(int64_t(S) * c), 1, 1);
-    cfg.blockDim = dim3(unsigned(threads), 1, 1);
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = unsigned(c);
-    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = c > 1 ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
-}
-
 }  // namespace
 }  // namespace acrl
 
@@ -681,12 +671,14 @@ extern "C" acrl_status acrl_seq_discrepancy(const float* logp_pi, const float* l
     if (T > 0 && (!logp_pi || !logp_mu || !lr || !d)) return ACRL_ERR_INVALID_ARG;
     if ((S > 0 && !seq) || (Gn > 0 && !grp)) return ACRL_ERR_INVALID_ARG;
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-    if (S > 0 && launch_per_response(seq_stats_kernel, S, ctas_per_response(S, T), kSeqThreads + 32, s, logp_pi, logp_mu,
-                                     mask, T, seq_offsets, S, group_offsets, Gn, entropy, lr, d, seq,
-                                     dev_flags) != cudaSuccess)
-        return launch_failed();
-    seq_finalize_kernel<<<1, kFinThreads, 0, s>>>(T, seq_offsets, S, group_offsets, Gn, seq, grp, batch, dev_flags);
-    return launch_status();
+    const int c = ctas_per_response(S, T);
+    acrl_status st = ACRL_OK;
+    if (S > 0)
+        st = launch(seq_stats_kernel, int64_t(S) * c, kSeqThreads + 32, 0, c, s, logp_pi, logp_mu, mask, T, seq_offsets, S,
+                    group_offsets, Gn, entropy, lr, d, seq, dev_flags);
+    if (st != ACRL_OK) return st;
+    return launch(seq_finalize_kernel, 1, kFinThreads, 0, 0, s, T, seq_offsets, S, group_offsets, Gn, seq, grp, batch,
+                  dev_flags);
 }
 
 extern "C" acrl_status acrl_grpo_advantage(const float* rewards, const int32_t* group_offsets, int32_t Gn, int32_t S,
@@ -696,22 +688,16 @@ extern "C" acrl_status acrl_grpo_advantage(const float* rewards, const int32_t* 
     if (Gn == 0) return ACRL_OK;
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     const int threads = 128;
-    auto launch = [&](auto kernel, int lanes) {
-        const int64_t grid = (int64_t(Gn) * lanes + threads - 1) / threads;
-        kernel<<<unsigned(grid), threads, 0, s>>>(rewards, group_offsets, Gn, S, p->adv_eps, p->adv_ddof,
-                                                  p->singleton_rule, adv, dev_flags);
+    auto run = [&](auto kernel, int lanes) {
+        return launch(kernel, (int64_t(Gn) * lanes + threads - 1) / threads, threads, 0, 0, s, rewards, group_offsets, Gn,
+                      S, p->adv_eps, p->adv_ddof, p->singleton_rule, adv, dev_flags);
     };
-    if (Gn <= kGrpoTeamPrompts)
-        launch(grpo_kernel<8>, 8);
-    else
-        launch(grpo_kernel<1>, 1);
-    return launch_status();
+    return Gn <= kGrpoTeamPrompts ? run(grpo_kernel<8>, 8) : run(grpo_kernel<1>, 1);
 }
 
 extern "C" acrl_status acrl_controller_init(acrl_controller_state* state, const acrl_params* p, acrl_stream stream) {
     if (!state || !params_ok(p)) return ACRL_ERR_INVALID_ARG;
-    controller_init_kernel<<<1, 1, 0, reinterpret_cast<cudaStream_t>(stream)>>>(state, p->X_init);
-    return launch_status();
+    return launch(controller_init_kernel, 1, 1, 0, 0, reinterpret_cast<cudaStream_t>(stream), state, p->X_init);
 }
 
 extern "C" acrl_status acrl_controller_save(const acrl_controller_state* state, acrl_controller_state* host_state,
@@ -743,12 +729,13 @@ extern "C" acrl_status acrl_controller_step(acrl_controller_state* state, const 
     if (T > 0 && (!lr || !weight || !coef)) return ACRL_ERR_INVALID_ARG;
     if ((S > 0 && (!seq || !adv)) || (Gn > 0 && !grp)) return ACRL_ERR_INVALID_ARG;
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-    if (S > 0 && launch_per_response(controller_weights_kernel, S, ctas_per_response(S, T), kSeqThreads, s, state, *p, lr,
-                                     mask, T, seq_offsets, Gn, seq, grp, batch, adv, weight, coef, alpha,
-                                     ent_coef) != cudaSuccess)
-        return launch_failed();
-    controller_finalize_kernel<<<1, kFinThreads, 0, s>>>(state, *p, S, seq, batch, dev_flags);
-    return launch_status();
+    const int c = ctas_per_response(S, T);
+    acrl_status st = ACRL_OK;
+    if (S > 0)
+        st = launch(controller_weights_kernel, int64_t(S) * c, kSeqThreads, 0, c, s, state, *p, lr, mask, T, seq_offsets, Gn,
+                    seq, grp, batch, adv, weight, coef, alpha, ent_coef);
+    if (st != ACRL_OK) return st;
+    return launch(controller_finalize_kernel, 1, kFinThreads, 0, 0, s, state, *p, S, seq, batch, dev_flags);
 }
 
 extern "C" acrl_status acrl_read_flags(const int32_t* dev_flags, int32_t* host_flags, acrl_stream stream) {

@@ -43,6 +43,7 @@ __global__ void __launch_bounds__(THREADS, kMinCtas<THREADS, DEPTH>)
     __shared__ float pmax[NW];
     extern __shared__ uint4 ring[];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    grid_begin();
     for (int64_t t = blockIdx.x; t < T; t += gridDim.x) {
         if (mask && mask[t] == 0) {
             if (threadIdx.x == 0) lse[t] = logp[t] = ent[t] = 0.f;
@@ -84,6 +85,7 @@ __global__ void __launch_bounds__(THREADS) token_stats_warp(const acrl_bf16* __r
     constexpr int NW = THREADS / 32;
     extern __shared__ uint4 ring[];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    grid_begin();
     for (int64_t t = int64_t(blockIdx.x) * NW + wid; t < T; t += int64_t(gridDim.x) * NW) {
         if (mask && mask[t] == 0) {
             if (lane == 0) lse[t] = logp[t] = ent[t] = 0.f;
@@ -129,6 +131,7 @@ __global__ void __launch_bounds__(THREADS) token_stats_team(const acrl_bf16* __r
     extern __shared__ uint4 ring[];
     static_assert(LANES >= 2 && LANES <= 32 && (LANES & (LANES - 1)) == 0, "lanes per row");
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, tl = lane % LANES;
+    grid_begin();
     for (int64_t base = (int64_t(blockIdx.x) * NW + wid) * RPW; base < T; base += int64_t(gridDim.x) * NW * RPW) {
         const int64_t t = base + lane / LANES;
         const bool in = t < T;
@@ -201,20 +204,19 @@ extern "C" acrl_status acrl_token_stats(const acrl_bf16* logits, int64_t T, int6
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     const int v = int(V);
     // `depth` steps of kUnroll 16-byte slots per thread of dynamic shared memory (at most 24 KB)
-    auto launch = [&](auto kernel, int threads, int depth, int64_t rows_per_cta) {
-        kernel<<<unsigned(grid_for(rows_per_cta, T)), threads, size_t(threads) * kUnroll * depth * 16, s>>>(
-            logits, T, v, ld, ids, mask, lse, logp, entropy, dev_flags);
-        return launch_status();
+    auto run = [&](auto kernel, int threads, int depth, int64_t rows_per_cta) {
+        return launch(kernel, grid_for(rows_per_cta, T), threads, size_t(threads) * kUnroll * depth * 16, 0, s, logits, T,
+                      v, ld, ids, mask, lse, logp, entropy, dev_flags);
     };
     const int team = V <= kTeamRowMaxV ? 8 : V <= kWarpRowMaxV ? 32 : V <= kMidRowMaxV ? 64 : 128;
     const bool ring = use_ring(T, team);
-    if (team == 8) return launch(token_stats_team<64, kUnroll, 8, kDepth>, 64, kDepth, 8);
+    if (team == 8) return run(token_stats_team<64, kUnroll, 8, kDepth>, 64, kDepth, 8);
     if (team == 32)
-        return ring ? launch(token_stats_warp<64, kUnroll, kDepth>, 64, kDepth, 2)
-                    : launch(token_stats_warp<256, kUnroll, 0>, 256, 0, 8);
+        return ring ? run(token_stats_warp<64, kUnroll, kDepth>, 64, kDepth, 2)
+                    : run(token_stats_warp<256, kUnroll, 0>, 256, 0, 8);
     if (team == 64)
-        return ring ? launch(token_stats_cta<64, kUnroll, kDepth>, 64, kDepth, 1)
-                    : launch(token_stats_cta<64, kUnroll, 0>, 64, 0, 1);
-    return ring ? launch(token_stats_cta<128, kUnroll, kDepth>, 128, kDepth, 1)
-                : launch(token_stats_cta<128, kUnroll, 0>, 128, 0, 1);
+        return ring ? run(token_stats_cta<64, kUnroll, kDepth>, 64, kDepth, 1)
+                    : run(token_stats_cta<64, kUnroll, 0>, 64, 0, 1);
+    return ring ? run(token_stats_cta<128, kUnroll, kDepth>, 128, kDepth, 1)
+                : run(token_stats_cta<128, kUnroll, 0>, 128, 0, 1);
 }

@@ -376,6 +376,20 @@ acrl_status acrl_loss_grad_logits(const acrl_bf16* logits, int64_t T, int64_t V,
 acrl_status acrl_reduce_loss(const float* token_loss, int64_t T, float* loss, acrl_stream stream);
 
 /*
+ * acrl_scale_grad -- out[t, j] = grad[t, j] * s for j < V, s being *scale
+ * rounded to bf16, the product rounded to bf16: the gradient of a loss that the
+ * caller scaled (gradient accumulation, mixed-precision loss scaling).  Where
+ * *scale is exactly 1 nothing is written: the caller uses `grad` as it is.
+ *   grad   device bf16 [T, ld], as acrl_loss_grad_logits writes it.
+ *   scale  device float [1].
+ *   out    device bf16 [T, ldo] output, no overlap with grad; ldo >= V, a
+ *          multiple of 8.  The columns from V up to the next multiple of 8 are
+ *          written too (scaled like the rest, from grad's).
+ */
+acrl_status acrl_scale_grad(const acrl_bf16* grad, int64_t T, int64_t V, int64_t ld, const float* scale,
+                            acrl_bf16* out, int64_t ldo, acrl_stream stream);
+
+/*
  * Host-buffer pipeline -- the whole on-policy pass (token statistics,
  * discrepancy, advantages, controller, gradient: the calls above, each citing
  * its passage) for a batch whose inputs and outputs live in host memory, e.g.

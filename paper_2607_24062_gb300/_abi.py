@@ -73,6 +73,7 @@ SIGNATURES = {
     "acrl_loss_grad_logits": (c_i32, [c_p, c_i64, c_i64, c_i64, c_p, c_p, c_p, c_p, c_p, c_p, c_p, c_f32, c_p, c_p,
                                       c_p, c_p, c_p]),
     "acrl_reduce_loss": (c_i32, [c_p, c_i64, c_p, c_p]),
+    "acrl_scale_grad": (c_i32, [c_p, c_i64, c_i64, c_i64, c_p, c_p, c_i64, c_p]),
     "acrl_host_pipeline_workspace_bytes": (c_i64, [c_i64, c_i64, c_i32, c_i32, c_i32]),
     "acrl_host_pipeline_create": (c_i32, [ctypes.POINTER(c_p), c_i64, c_i64, c_i64, c_i32, c_i32, c_i32, c_p,
                                           c_i64]),

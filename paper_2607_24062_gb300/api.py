@@ -266,6 +266,25 @@ def reduce_loss(token_loss, *, loss=None, stream=None):
     return loss
 
 
+def scale_grad(grad, scale, *, V=None, out=None, stream=None):
+    """acrl_scale_grad: grad (bf16 [T, ld]) times the float32 scalar on the device.  Returns bf16 [T, ldo], ldo = V
+    rounded up to a multiple of eight; its contents are undefined where the scalar is exactly 1."""
+    T, ld = _rows(grad, "grad")
+    V = grad.shape[1] if V is None else V
+    if V > ld:
+        raise AcrlError(f"V = {V} is more than the row stride {ld}")
+    _need(scale, torch.float32, 1, "scale")
+    ldo = (V + 7) // 8 * 8
+    if out is None:
+        out = torch.empty((T, ldo), dtype=torch.bfloat16, device=grad.device)
+    else:
+        To, ldo = _rows(out, "out")
+        if To < T or out.shape[1] < V:
+            raise AcrlError(f"out: shape {tuple(out.shape)}, needs {(T, V)}")
+    _call("acrl_scale_grad", (grad, scale, out), stream, _ptr(grad), T, V, ld, _ptr(scale), _ptr(out), ldo)
+    return out
+
+
 def lmhead_workspace_bytes(M: int, N: int) -> int:
     return int(lib().acrl_lmhead_workspace_bytes(M, N))
 
@@ -442,7 +461,7 @@ def check_flags(flags, stream=None) -> None:
 
 
 __all__ = ["Params", "AcrlError", "token_stats", "seq_discrepancy", "grpo_advantage", "controller_init",
-           "controller_step", "loss_grad_logits", "reduce_loss", "read_flags", "check_flags", "read_state", "Discrepancy",
+           "controller_step", "loss_grad_logits", "reduce_loss", "scale_grad", "read_flags", "check_flags", "read_state", "Discrepancy",
            "lmhead_logits_stats", "lmhead_merge", "lmhead_workspace_bytes", "lmhead_stats_noalloc", "save_state",
            "load_state", "controller_save", "controller_load", "selftest_wait_timeout",
            "host_pipeline_workspace_bytes", "host_pipeline_create", "host_pipeline_step", "host_pipeline_begin",

@@ -6,8 +6,8 @@
 The forward runs the whole pass of `AcrlStep` (statistics, discrepancy,
 advantages, controller, then the gradient kernel, which writes dL/dlogits in
 bf16 while it computes the loss), so the backward needs no second pass over
-the logits: it hands back that buffer, scaled by the incoming gradient when
-that is not 1.  The gradient is the one of Eq. ACRL on the on-policy step
+the logits: it hands back that buffer, or a copy scaled by the incoming
+gradient when that is not 1.  The gradient is the one of Eq. ACRL on the on-policy step
 (theta = theta_old, so r = 1), with the importance weights treated as
 constants, as the paper's rho is built from theta_old.
 
@@ -21,6 +21,7 @@ from typing import Callable
 
 import torch
 
+from . import api
 from .pipeline import AcrlStep
 
 
@@ -36,7 +37,10 @@ class _AcrlLoss(torch.autograd.Function):
     def backward(ctx, grad_out):
         g = ctx.step.grad[: ctx.rows, : ctx.cols]
         if float(grad_out) != 1.0:  # one scalar read; the common loss.backward() passes 1
-            g = g * grad_out.to(g.dtype)
+            if torch.is_grad_enabled() or grad_out.dtype != torch.float32 or grad_out.device != g.device:
+                g = g * grad_out.to(g.dtype)  # a graph of the backward itself, or no scalar the kernel reads
+            else:
+                g = api.scale_grad(g, grad_out)[:, : ctx.cols]
         return g, None, None, None, None, None, None, None, None
 
 

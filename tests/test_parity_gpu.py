@@ -801,3 +801,40 @@ def test_loss_sum_blocks_tails_and_alignment(offset):
         ref = math.fsum(host(x).astype(np.float64).tolist())
         bound = 1e-6 * float(host(x).astype(np.float64).__abs__().sum()) + 1e-6
         assert abs(float(a) - ref) <= bound, (T, float(a), ref)
+
+
+@pytest.mark.parametrize("T,V,ld", [(1, 1, 8), (300, 7, 8), (5, 8, 16), (3, 2047, 2048), (2, 8193, 8208), (131, 20011, 20016),
+                                    (1000, 264, 264)])
+def test_scale_grad_is_the_bf16_product(T, V, ld):
+    """acrl_scale_grad against torch's bf16 product, bit for bit: rows shorter and longer than a block's step, padded
+    row strides, infinities; a scale of exactly 1 writes nothing."""
+    gen = torch.Generator(device=DEV).manual_seed(T + V)
+    g = torch.randn((T, ld), generator=gen, device=DEV).to(torch.bfloat16)
+    g[0, 0] = float("inf")
+    for f in (0.25, -3.7, 0.0, 1.0 + 2.0 ** -12):   # the last rounds to a bf16 of 1, and is a copy
+        s = torch.tensor(f, device=DEV)
+        out = torch.full((T, (V + 7) // 8 * 8 + 8), 5.0, dtype=torch.bfloat16, device=DEV)
+        acrl.api.scale_grad(g, s, V=V, out=out)
+        ref = g[:, :V] * s.to(torch.bfloat16)
+        same = (out[:, :V].view(torch.int16) == ref.contiguous().view(torch.int16)) | (out[:, :V].isnan() & ref.isnan())
+        assert bool(same.all())
+        assert bool((out[:, (V + 7) // 8 * 8:] == 5.0).all())
+    out = torch.full((T, (V + 7) // 8 * 8), 5.0, dtype=torch.bfloat16, device=DEV)
+    acrl.api.scale_grad(g, torch.ones((), device=DEV), V=V, out=out)
+    assert bool((out == 5.0).all())
+
+
+def test_autograd_backward_of_the_backward():
+    """The gradient stays a function of the incoming scale where a graph of the backward is asked for."""
+    spec = W.small_variant(W.GRPO, name="autograd2", n_prompts=2, group_size=4, len_lo=5, len_hi=20, V=1003)
+    b = _gen(spec, seed=3)
+    step = acrl.AcrlStep.for_batch(b, acrl.Params())
+    x = b.logits[:, :b.V].detach().requires_grad_(True)
+    s = torch.tensor(0.5, device=DEV, requires_grad=True)
+    loss = acrl.acrl_loss(step, x, b.ids, b.mask, b.logp_mu, b.rewards, b.seq_offsets, b.group_offsets)
+    g, = torch.autograd.grad(loss * s, x, create_graph=True)
+    v = torch.randn(g.shape, device=DEV).to(g.dtype)
+    ds, = torch.autograd.grad((g.float() * v.float()).sum(), s)
+    ref = (step.grad[:, :b.V].float() * v.float()).sum()
+    # bf16 rounding of the products' sum on torch's side: 2^-8 of the terms' magnitude
+    assert abs(float(ds - ref)) <= 2.0 ** -8 * float((step.grad[:, :b.V].float() * v.float()).abs().sum())

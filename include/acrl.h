@@ -319,6 +319,22 @@ acrl_status acrl_controller_step(acrl_controller_state* state, const acrl_params
                                  int32_t* dev_flags, acrl_stream stream);
 
 /*
+ * acrl_importance_weights -- acrl_seq_discrepancy, acrl_grpo_advantage and
+ * acrl_controller_step in order, for callers that do nothing between them: the
+ * weights of a batch from per-token log-probs (the call whose cost Sec. 5.4
+ * reports).  Same arguments, outputs and flags, the same bits; batches of up to
+ * 32 responses and prompts whose tokens one cluster can take are done by one
+ * kernel.
+ */
+acrl_status acrl_importance_weights(acrl_controller_state* state, const acrl_params* p,
+                                    const float* logp_pi, const float* logp_mu, const uint8_t* mask,
+                                    int64_t T, const float* rewards, const int64_t* seq_offsets, int32_t S,
+                                    const int32_t* group_offsets, int32_t Gn, const float* entropy,
+                                    float* lr, float* d, acrl_seq_stats* seq, acrl_group_stats* grp,
+                                    acrl_batch_stats* batch, float* adv, float* weight, float* coef,
+                                    float* alpha, float* ent_coef, int32_t* dev_flags, acrl_stream stream);
+
+/*
  * acrl_loss_grad_logits -- loss of Eq. ACRL and its gradient w.r.t. the logits.
  * With r_t = exp(logp_t - old_logp_t) (exactly 1 when old_logp is NULL, the
  * one-update-per-rollout setting of App. A) and g_t = 1 on the unclipped

@@ -70,6 +70,8 @@ SIGNATURES = {
     "acrl_controller_load": (c_i32, [c_p, c_p, c_p]),
     "acrl_controller_step": (c_i32, [c_p, ctypes.POINTER(Params), c_p, c_p, c_i64, c_p, c_i32, c_p, c_i32, c_p, c_p,
                                      c_p, c_p, c_p, c_p, c_p, c_p, c_p, c_p]),
+    "acrl_importance_weights": (c_i32, [c_p, ctypes.POINTER(Params), c_p, c_p, c_p, c_i64, c_p, c_p, c_i32, c_p, c_i32]
+                                + [c_p] * 13),
     "acrl_loss_grad_logits": (c_i32, [c_p, c_i64, c_i64, c_i64, c_p, c_p, c_p, c_p, c_p, c_p, c_p, c_f32, c_p, c_p,
                                       c_p, c_p, c_p]),
     "acrl_reduce_loss": (c_i32, [c_p, c_i64, c_p, c_p]),

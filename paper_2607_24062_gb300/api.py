@@ -226,6 +226,40 @@ def controller_step(state, params: Params, disc: Discrepancy, mask, seq_offsets,
     return weight, coef, alpha
 
 
+def importance_weights(state, params: Params, logp_pi, logp_mu, mask, rewards, seq_offsets, group_offsets,
+                       entropy=None, *, out: Discrepancy, adv, weight, coef, alpha=None, ent_coef=None, flags,
+                       stream=None) -> None:
+    """acrl_importance_weights: seq_discrepancy, grpo_advantage and controller_step in one call, into the caller's
+    buffers."""
+    T, S, Gn = logp_pi.numel(), seq_offsets.numel() - 1, group_offsets.numel() - 1
+    f32 = torch.float32
+    _need(state, torch.uint8, STATE_DTYPE.itemsize, "state")
+    _need(logp_pi, f32, T, "logp_pi")
+    _need(logp_mu, f32, T, "logp_mu")
+    _opt(mask, torch.uint8, T, "mask")
+    _need(rewards, f32, S, "rewards")
+    _need(seq_offsets, torch.int64, S + 1, "seq_offsets")
+    _need(group_offsets, torch.int32, Gn + 1, "group_offsets")
+    _opt(entropy, f32, T, "entropy")
+    _need(out.lr, f32, T, "lr")
+    _need(out.d, f32, T, "d")
+    _need(out.seq, torch.uint8, S * SEQ_DTYPE.itemsize, "seq")
+    _need(out.grp, torch.uint8, Gn * GRP_DTYPE.itemsize, "grp")
+    _need(out.batch, torch.uint8, BATCH_DTYPE.itemsize, "batch")
+    _need(adv, f32, S, "adv")
+    _need(weight, f32, T, "weight")
+    _need(coef, f32, T, "coef")
+    _opt(alpha, f32, S, "alpha")
+    _opt(ent_coef, f32, T, "ent_coef")
+    _need(flags, torch.int32, 1, "flags")
+    _call("acrl_importance_weights",
+          (state, logp_pi, logp_mu, mask, rewards, seq_offsets, group_offsets, entropy, out.lr, out.d, out.seq, out.grp,
+           out.batch, adv, weight, coef, alpha, ent_coef, flags), stream,
+          _ptr(state), ctypes.byref(params), _ptr(logp_pi), _ptr(logp_mu), _ptr(mask), T, _ptr(rewards),
+          _ptr(seq_offsets), S, _ptr(group_offsets), Gn, _ptr(entropy), _ptr(out.lr), _ptr(out.d), _ptr(out.seq),
+          _ptr(out.grp), _ptr(out.batch), _ptr(adv), _ptr(weight), _ptr(coef), _ptr(alpha), _ptr(ent_coef), _ptr(flags))
+
+
 def loss_grad_logits(logits, ids, mask, lse, old_logp, coef, clip_eps: float, *, V=None, entropy=None, ent_coef=None,
                      grad=None, token_loss=None, loss=None, flags=None, stream=None):
     """acrl_loss_grad_logits.  Returns (grad bf16 [T, ld], token_loss [T], loss [1]).

@@ -158,6 +158,55 @@ __device__ __forceinline__ T warp_max(T v) {
 
 __device__ __forceinline__ double shfl_xor_f64(double v, int m) { return __shfl_xor_sync(0xffffffffu, v, m); }
 
+// Reciprocal, quotient and square root in fp64 with short dependent chains: from
+// one fp64 operation to the next that needs it takes some 80 cycles here, and the
+// compiler's division and root are a dozen of them.  Newton-Raphson from the fp32
+// approximation (23 bits): one step on the reciprocal (46 bits), then the
+// residual of the quotient, which brings the error down to the rounding of the
+// last operation; likewise for the root.  `recip64` and `quot64` want
+// 2^-100 <= |b| < 2^100, so that the approximation and every product stay normal
+// (counts always are); `div64` and `sqrt64` take other operands to the ordinary
+// operation.
+__device__ __forceinline__ bool exp_within(double v, int lim) {  // 2^-lim <= |v| < 2^lim
+    const int e = ((__double2hiint(v) >> 20) & 0x7ff) - 1023;
+    return e >= -lim && e < lim;
+}
+
+__device__ __forceinline__ double recip64(double b) {
+    float x;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(x) : "f"(float(b)));
+    const double r = double(x);
+    return fma(fma(-b, r, 1.0), r, r);
+}
+
+// a / b, r = recip64(b).
+__device__ __forceinline__ double quot64(double a, double b, double r) {
+    const double q = a * r;
+    const double c = fma(fma(-b, q, a), r, q);
+    return (__double2hiint(q) & 0x7ff00000) == 0x7ff00000 ? q : c;  // an infinite a has no residual
+}
+
+__device__ __forceinline__ double div64(double a, double b) {
+    return exp_within(b, 100) ? quot64(a, b, recip64(b)) : a / b;
+}
+
+__device__ __forceinline__ double sqrt64(double v) {
+    if (!exp_within(v, 100) || v < 0.0) return sqrt(v);
+    const double r = double(rsqrtf(float(v)));
+    double g = v * r, h = 0.5 * r;
+    const double e = fma(-h, g, 0.5);
+    g = fma(g, e, g);
+    h = fma(h, e, h);
+    return fma(fma(-g, g, v), h, g);
+}
+
+// Sum of 32 non-negative counts below 2^31.
+__device__ __forceinline__ long long warp_count(int n) {
+    const unsigned lo = __reduce_add_sync(0xffffffffu, unsigned(n) & 0xffffu);
+    const unsigned hi = __reduce_add_sync(0xffffffffu, unsigned(n) >> 16);
+    return (long long)(lo) + ((long long)(hi) << 16);
+}
+
 // Four sums: lane l ends with the total of value l / 8.
 __device__ __forceinline__ double warp_sum4(double a0, double a1, double a2, double a3) {
     const int lane = threadIdx.x & 31;

@@ -15,7 +15,7 @@ from parity import assert_close_abs, assert_close_rel, compare_batch, compare_gr
 pytestmark = pytest.mark.gpu
 
 import paper_2607_24062_gb300 as acrl  # noqa: E402
-from paper_2607_24062_gb300 import api  # noqa: E402
+from paper_2607_24062_gb300 import _abi, api  # noqa: E402
 
 DEV = "cuda"
 
@@ -89,3 +89,67 @@ def test_loss_sum_sizes(T):
         bound = 4 * 2.0 ** -24 * float(x.double().abs().sum()) + 1e-30
         assert abs(float(api.reduce_loss(x)) - want) <= bound
         assert torch.equal(api.reduce_loss(x), api.reduce_loss(x))
+
+
+def _three_calls_and_one(p, steps, pi, mu, mask, so, go, R, H, ent):
+    """Every output byte of the three calls and of the one that does all, after `steps` steps of one controller."""
+    outs = []
+    for one in (False, True):
+        T, S, Gn = pi.numel(), so.numel() - 1, go.numel() - 1
+        state, flags = api.controller_init(p), api.new_flags()
+        f = lambda n: torch.full((n,), 7.0, device=DEV)  # noqa: E731
+        disc = api.Discrepancy(f(T), f(T), api.struct_buffer(_abi.SEQ_DTYPE, S), api.struct_buffer(_abi.GRP_DTYPE, Gn),
+                               api.struct_buffer(_abi.BATCH_DTYPE, 1), S, Gn)
+        adv, w, coef, alpha, ec = f(S), f(T), f(T), f(S), (f(T) if ent else None)
+        for _ in range(steps):
+            if one:
+                api.importance_weights(state, p, pi, mu, mask, R, so, go, H, out=disc, adv=adv, weight=w, coef=coef,
+                                       alpha=alpha, ent_coef=ec, flags=flags)
+            else:
+                api.seq_discrepancy(pi, mu, mask, so, go, H, out=disc, flags=flags)
+                api.grpo_advantage(R, go, p, adv=adv, flags=flags)
+                api.controller_step(state, p, disc, mask, so, go, adv, weight=w, coef=coef, alpha=alpha, ent_coef=ec,
+                                    flags=flags)
+        outs.append([host(x.view(torch.uint8)) for x in
+                     (state, flags, disc.lr, disc.d, disc.seq, disc.grp, disc.batch, adv, w, coef, alpha) +
+                     ((ec,) if ent else ())])
+    return outs
+
+
+def _assert_same_bytes(a, b):
+    names = "state flags lr d seq grp batch adv weight coef alpha ent_coef".split()
+    assert not [(nm, np.flatnonzero(x != y)[:8].tolist()) for nm, x, y in zip(names, a, b) if not np.array_equal(x, y)]
+
+
+# one part and one prompt; two and four CTAs a response; parts that fill both groups and both passes of eight CTAs;
+# more than a round of tokens a thread; empty responses; the largest counts it takes and the next
+_ONE_SHAPES = [(1, 1, 1, 1), (1, 1, 9000, 9000), (4, 1, 256, 256), (2, 4, 64, 1100), (1, 9, 0, 700), (4, 4, 100, 520),
+               (8, 4, 0, 260), (32, 1, 1, 200), (33, 1, 1, 9), (1, 33, 1, 9), (3, 1, 300, 12000)]
+
+
+@pytest.mark.parametrize("Q,G,lo,hi", _ONE_SHAPES)
+@pytest.mark.parametrize("kw", [dict(), dict(y_gran=acrl.Y_BATCH, agg=acrl.AGG_TOKEN_MEAN, calib_steps=2),
+                                dict(mode=acrl.MODE_MIS, C=1.1), dict(mode=acrl.MODE_ACRL_FALLBACK, X_init=0.01, x_ema=0.3),
+                                dict(y_gran=acrl.Y_SEQUENCE, entropy_coeff=0.01, adv_ddof=0)])
+def test_one_call_has_the_bits_of_the_three(Q, G, lo, hi, kw):
+    pi, mu, mask, so, go, R, H = _tokens(Q, G, lo, hi, seed=Q * 77 + G)
+    p = acrl.Params(**kw)
+    ent = p.entropy_coeff > 0
+    a, b = _three_calls_and_one(p, 3, pi, mu, mask, so, go, R, H if ent else None, ent)
+    _assert_same_bytes(a, b)
+    a, b = _three_calls_and_one(p, 1, pi, mu, None, so, go, R, H, ent)
+    _assert_same_bytes(a, b)
+
+
+def test_one_call_on_uneven_prompts_and_bad_offsets():
+    pi, mu, mask, so, go, R, H = _tokens(6, 2, 1, 300, seed=5)
+    p = acrl.Params()
+    uneven = torch.tensor([0, 0, 1, 1, 5, 12, 12], dtype=torch.int32, device=DEV)   # empty prompts, one of one
+    broken_go = torch.tensor([0, 3, 2, 7, 9, 11, 13], dtype=torch.int32, device=DEV)
+    broken_so = so.clone()
+    broken_so[4] = so[-1] + 5
+    nan = pi.clone()
+    nan[3] = float("nan")
+    for args in ((pi, so, uneven), (pi, so, broken_go), (pi, broken_so, go), (nan, so, go)):
+        a, b = _three_calls_and_one(p, 2, args[0], mu, mask, args[1], args[2], R, H, False)
+        _assert_same_bytes(a, b)

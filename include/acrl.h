@@ -383,6 +383,22 @@ acrl_status acrl_loss_grad_logits(const acrl_bf16* logits, int64_t T, int64_t V,
                                   int32_t* dev_flags, acrl_stream stream);
 
 /*
+ * acrl_step -- one on-policy pass: acrl_token_stats, acrl_importance_weights
+ * (with the pass's own log-probs and entropies) and acrl_loss_grad_logits (with
+ * its lse, r = 1, and the entropy bonus when ent_coef is given), in one call.
+ * Arguments, outputs and flags are those of the three.
+ */
+acrl_status acrl_step(acrl_controller_state* state, const acrl_params* p,
+                      const acrl_bf16* logits, int64_t T, int64_t V, int64_t ld,
+                      const int32_t* ids, const uint8_t* mask, const float* logp_mu, const float* rewards,
+                      const int64_t* seq_offsets, int32_t S, const int32_t* group_offsets, int32_t Gn,
+                      float* lse, float* logp, float* entropy, float* lr, float* d,
+                      acrl_seq_stats* seq, acrl_group_stats* grp, acrl_batch_stats* batch, float* adv,
+                      float* weight, float* coef, float* alpha, float* ent_coef,
+                      acrl_bf16* grad, float* token_loss, float* loss,
+                      int32_t* dev_flags, acrl_stream stream);
+
+/*
  * acrl_reduce_loss -- *loss = sum_t token_loss[t] over T entries, in the same
  * fixed order and fp64 accumulation as acrl_loss_grad_logits.  Gives the
  * batch loss when the gradient was produced chunk by chunk (Eq. ACRL's outer

@@ -74,6 +74,8 @@ SIGNATURES = {
                                 + [c_p] * 13),
     "acrl_loss_grad_logits": (c_i32, [c_p, c_i64, c_i64, c_i64, c_p, c_p, c_p, c_p, c_p, c_p, c_p, c_f32, c_p, c_p,
                                       c_p, c_p, c_p]),
+    "acrl_step": (c_i32, [c_p, ctypes.POINTER(Params), c_p, c_i64, c_i64, c_i64, c_p, c_p, c_p, c_p, c_p, c_i32, c_p,
+                          c_i32] + [c_p] * 18),
     "acrl_reduce_loss": (c_i32, [c_p, c_i64, c_p, c_p]),
     "acrl_scale_grad": (c_i32, [c_p, c_i64, c_i64, c_i64, c_p, c_p, c_i64, c_p]),
     "acrl_host_pipeline_workspace_bytes": (c_i64, [c_i64, c_i64, c_i32, c_i32, c_i32]),

@@ -290,6 +290,41 @@ def loss_grad_logits(logits, ids, mask, lse, old_logp, coef, clip_eps: float, *,
     return grad, token_loss, loss
 
 
+def step(state, params: Params, logits, ids, mask, logp_mu, rewards, seq_offsets, group_offsets, *, V, lse, logp,
+         entropy, out: Discrepancy, adv, weight, coef, alpha=None, ent_coef=None, grad, token_loss, loss, flags,
+         stream=None) -> None:
+    """acrl_step: token_stats, importance_weights and loss_grad_logits in one call, into the caller's buffers."""
+    T, ld = _rows(logits, "logits")
+    S, Gn = seq_offsets.numel() - 1, group_offsets.numel() - 1
+    f32 = torch.float32
+    _need(state, torch.uint8, STATE_DTYPE.itemsize, "state")
+    _need(ids, torch.int32, T, "ids")
+    _opt(mask, torch.uint8, T, "mask")
+    _need(logp_mu, f32, T, "logp_mu")
+    _need(rewards, f32, S, "rewards")
+    _need(seq_offsets, torch.int64, S + 1, "seq_offsets")
+    _need(group_offsets, torch.int32, Gn + 1, "group_offsets")
+    for name, t in (("lse", lse), ("logp", logp), ("entropy", entropy), ("lr", out.lr), ("d", out.d),
+                    ("weight", weight), ("coef", coef), ("token_loss", token_loss)):
+        _need(t, f32, T, name)
+    _need(out.seq, torch.uint8, S * SEQ_DTYPE.itemsize, "seq")
+    _need(out.grp, torch.uint8, Gn * GRP_DTYPE.itemsize, "grp")
+    _need(out.batch, torch.uint8, BATCH_DTYPE.itemsize, "batch")
+    _need(adv, f32, S, "adv")
+    _opt(alpha, f32, S, "alpha")
+    _opt(ent_coef, f32, T, "ent_coef")
+    if grad.dtype != torch.bfloat16 or grad.dim() != 2 or grad.stride(0) != ld or grad.stride(1) != 1 or \
+            grad.shape[0] < T:
+        raise AcrlError("grad: expected a bf16 [T, ld] tensor with the logits' row stride")
+    _need(loss, f32, 1, "loss")
+    _need(flags, torch.int32, 1, "flags")
+    bufs = (lse, logp, entropy, out.lr, out.d, out.seq, out.grp, out.batch, adv, weight, coef, alpha, ent_coef, grad,
+            token_loss, loss, flags)
+    _call("acrl_step", (state, logits, ids, mask, logp_mu, rewards, seq_offsets, group_offsets) + bufs, stream,
+          _ptr(state), ctypes.byref(params), _ptr(logits), T, V, ld, _ptr(ids), _ptr(mask), _ptr(logp_mu),
+          _ptr(rewards), _ptr(seq_offsets), S, _ptr(group_offsets), Gn, *[_ptr(t) for t in bufs])
+
+
 def reduce_loss(token_loss, *, loss=None, stream=None):
     """acrl_reduce_loss."""
     T = token_loss.numel()

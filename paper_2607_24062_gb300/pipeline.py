@@ -1,8 +1,11 @@
-"""One on-policy ACRL pass over a batch: the five C-ABI calls in order on one
+"""One on-policy ACRL pass over a batch: the C-ABI calls in order on one
 stream, with every buffer allocated once per batch shape.
 
     token_stats -> seq_discrepancy -> grpo_advantage -> controller_step
                 -> loss_grad_logits
+
+Where nothing comes between them (no exchange between ranks, no chunks) the five
+are made as one call, with the same results.
 
 The weights need Y_g, which needs every row of the prompt, so the gradient
 pass can only start after the statistics pass has seen the whole batch: the
@@ -96,9 +99,22 @@ class AcrlStep:
 
     def run(self, logits, ids, mask, logp_mu, rewards, seq_offsets, group_offsets, stream=None, exchange=None,
             **grad_kw):
+        if exchange is None and not grad_kw and self._whole(logits, seq_offsets, group_offsets):
+            api.step(self.state, self.params, logits, ids, mask, logp_mu, rewards, seq_offsets, group_offsets, V=self.V,
+                     lse=self.lse, logp=self.logp, entropy=self.entropy, out=self.disc, adv=self.adv,
+                     weight=self.weight, coef=self.coef, alpha=self.alpha, ent_coef=self.ent_coef, grad=self.grad,
+                     token_loss=self.token_loss, loss=self.loss, flags=self.flags, stream=stream)
+            return
         self.statistics(logits, ids, mask, logp_mu, rewards, seq_offsets, group_offsets, stream=stream,
                         exchange=exchange)
         self.gradient(logits, ids, mask, stream=stream, **grad_kw)
+
+    def _whole(self, logits, seq_offsets, group_offsets) -> bool:
+        """The batch is the one this object was built for, and its two halves are the ones below: one call does both."""
+        cls = type(self)
+        return (logits.shape[0] == self.T == self.logp.numel() and seq_offsets.numel() == self.S + 1 and
+                group_offsets.numel() == self.Gn + 1 and self.disc.S == self.S and self.disc.Gn == self.Gn and
+                cls.statistics is AcrlStep.statistics and cls.gradient is AcrlStep.gradient)
 
     @classmethod
     def for_batch(cls, batch, params: Params, device="cuda", grad_rows=None):
@@ -141,6 +157,11 @@ class AcrlStep:
         return api.read_state(self.state)
 
 
+def _struct_out(dtype, n: int, dev) -> torch.Tensor:
+    """Bytes for n ABI structs, every one of which the call writes."""
+    return torch.empty(n * dtype.itemsize, dtype=torch.uint8, device=dev) if n > 0 else api.struct_buffer(dtype, n, dev)
+
+
 @dataclass
 class Weights:
     weight: torch.Tensor      # float32 [T] importance weight per token (0 where masked)
@@ -161,9 +182,18 @@ def importance_weights(state, params: Params, logp_old, logp_mu, mask, rewards, 
     the batch-statistics bytes before the controller, as in
     AcrlStep.statistics."""
     flags = api.new_flags(logp_old.device) if flags is None else flags
+    if exchange is None:
+        dev, T, S, Gn = logp_old.device, logp_old.numel(), seq_offsets.numel() - 1, group_offsets.numel() - 1
+        f32 = dict(dtype=torch.float32, device=dev)
+        lr, d, weight, coef = (torch.empty(T, **f32) for _ in range(4))
+        adv, alpha = torch.empty(rewards.numel(), **f32), torch.empty(S, **f32)
+        disc = api.Discrepancy(lr, d, _struct_out(SEQ_DTYPE, S, dev), _struct_out(GRP_DTYPE, Gn, dev),
+                               _struct_out(BATCH_DTYPE, 1, dev), S, Gn)
+        api.importance_weights(state, params, logp_old, logp_mu, mask, rewards, seq_offsets, group_offsets, out=disc,
+                               adv=adv, weight=weight, coef=coef, alpha=alpha, flags=flags, stream=stream)
+        return Weights(weight, coef, adv, alpha, disc, flags)
     disc = api.seq_discrepancy(logp_old, logp_mu, mask, seq_offsets, group_offsets, flags=flags, stream=stream)
-    if exchange is not None:
-        exchange(disc.batch)
+    exchange(disc.batch)
     adv = api.grpo_advantage(rewards, group_offsets, params, flags=flags, stream=stream)
     weight, coef, alpha = api.controller_step(state, params, disc, mask, seq_offsets, group_offsets, adv, flags=flags,
                                               stream=stream)

@@ -13,7 +13,7 @@
 // CTA's TMEM.  Per SM a K slab is 32 KB (A 128 x 64 + B 128 x 64), so six
 // stages fit and the weight half is never staged twice in a pair.
 //   warp 0     in each CTA, one thread issues the TMA loads (128B-swizzled)
-//              of the CTA's A and B into a 6-stage ring, counted on the even
+//              of the CTA's A and B into a ring of stages, counted on the even
 //              CTA's stage barrier;
 //   warp 1     in the even CTA, one thread issues tcgen05.mma (M=256, N=256,
 //              K=16, kind::f16) into one of two 256-column accumulators and
@@ -49,11 +49,26 @@ namespace {
 
 constexpr int kBM = 128, kBN = 256;   // rows of H per CTA, columns (weight rows) per tile
 constexpr int kBK = 64;               // K slab: 64 bf16 = one 128-byte row under the 128-byte swizzle
-constexpr int kStages = 6;
 constexpr int kHalfBN = kBN / 2;      // weight rows staged by each CTA of a pair
-constexpr int kABytes = kBM * kBK * 2;
 constexpr int kBBytes = kHalfBN * kBK * 2;
-constexpr int kStageBytes = kABytes + kBBytes;   // per CTA; the pair's stage barrier counts twice this
+// The ring: STAGES stages of B and of AROWS rows of A per CTA.  Up to 16 rows of
+// H in all, a stage holds and loads only those (the MMA reads the 128 rows that its
+// shape has; what the others hold lands in accumulator rows that nothing reads):
+// a copy whose box of 128 rows has eight or fewer in the tensor is slow, and the
+// freed memory makes more stages for the weight's stream from HBM.  K = 4,096,
+// N = 151,936 with the merge, M = 1 / 4 / 8 / 16: 380 / 331 / 306 / 211 us with
+// boxes of 128 rows and six stages, 195 / 199 / 199 / 203 with the short ring (the
+// weight's bytes take 186).  Rings of 32 rows (10 stages) and 64 rows (8) gain
+// nothing over the full one: 214 us each for 32 rows, 220 against 217 for 48.
+template <int STAGES, int AROWS>
+struct Ring {
+    static constexpr int kStages = STAGES, kARows = AROWS;
+    static constexpr int kABytes = AROWS * kBK * 2;
+    static constexpr int kBytes = STAGES * (kABytes + kBBytes);
+};
+using RingFull = Ring<6, kBM>;
+using Ring16 = Ring<11, 16>;
+constexpr int kMaxStages = 11;
 constexpr int kThreads = 192;
 constexpr uint32_t kTmemCols = 512;
 constexpr int kBandM = 32;            // row tiles per band (16 pairs)
@@ -72,20 +87,20 @@ constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | (uint32_t(kBN >
 //   tfull[b]   each CTA: accumulator b is complete
 //   tempty[b]  even CTA: the eight epilogue warps of the pair drained accumulator b
 struct Barriers {
-    uint64_t full[kStages];
-    uint64_t empty[kStages];
+    uint64_t full[kMaxStages];
+    uint64_t empty[kMaxStages];
     uint64_t tfull[2];
     uint64_t tempty[2];
     uint64_t mma_done;
     uint32_t tmem_base;
     int32_t abort;
 };
-// The B stages come first, then the A stages, the output staging blocks and
-// the barriers, with a margin behind them (every descriptor read stays inside
-// the allocation).
-constexpr int kMargin = 8192;
-constexpr int kSmemBytes = 1024 + kStages * kStageBytes + kOutBytes + int(sizeof(Barriers)) + kMargin;
-static_assert(kSmemBytes <= 227 * 1024, "shared memory per CTA");
+// The A stages come first, then the B stages, the output staging blocks and the
+// barriers: what the MMA reads beyond a short A stage stays inside the allocation.
+template <class R>
+constexpr int kSmemBytes = 1024 + R::kBytes + kOutBytes + int(sizeof(Barriers));
+static_assert(kSmemBytes<RingFull> <= 227 * 1024 && kSmemBytes<Ring16> <= 227 * 1024, "shared memory per CTA");
+static_assert(kBBytes >= kBM * kBK * 2, "the MMA's reads beyond the last A stage stay inside the B stages");
 
 // ---------------------------------------------------------------------------
 // PTX wrappers
@@ -191,8 +206,10 @@ __device__ __forceinline__ void give_up(volatile int32_t* abort, int32_t* flags)
 // roles
 // ---------------------------------------------------------------------------
 
+template <class R>
 __device__ void producer(const CUtensorMap* tmA, const CUtensorMap* tmB, uint8_t* sA, uint8_t* sB, Barriers* bars,
-                         uint32_t rank, int m_pairs, int n_tiles, int total, int k_iters, int32_t* flags) {
+                         uint32_t rank, int m_pairs, int n_tiles, int total, int k_iters, int a_bytes, int32_t* flags) {
+    constexpr int kStages = R::kStages;
     volatile int32_t* abort = &bars->abort;
     const int cl = int(blockIdx.x >> 1), ncl = int(gridDim.x >> 1);
     int stage = 0;
@@ -210,10 +227,10 @@ __device__ void producer(const CUtensorMap* tmA, const CUtensorMap* tmB, uint8_t
                 ok = false;
                 break;
             }
-            // the even CTA's barrier counts both CTAs' bytes of this stage
-            if (rank == 0) mbar_expect_tx(&bars->full[stage], 2 * kStageBytes);
+            // the even CTA's barrier counts both CTAs' bytes of this stage; with a short ring only the even CTA has rows
+            if (rank == 0) mbar_expect_tx(&bars->full[stage], 2 * kBBytes + (R::kARows < kBM ? 1 : 2) * a_bytes);
             const uint32_t full0 = peer_addr(&bars->full[stage], 0);
-            tma_load_pair(sA + stage * kABytes, tmA, full0, kk * kBK, m * kBM);
+            if (R::kARows == kBM || rank == 0) tma_load_pair(sA + stage * R::kABytes, tmA, full0, kk * kBK, m * kBM);
             tma_load_pair(sB + stage * kBBytes, tmB, full0, kk * kBK, n * kBN + int(rank) * kHalfBN);
             ++issued;
             if (++stage == kStages) {
@@ -237,8 +254,10 @@ __device__ void producer(const CUtensorMap* tmA, const CUtensorMap* tmB, uint8_t
 }
 
 // The even CTA's MMA thread.
+template <class R>
 __device__ void mma_issuer(uint8_t* sA, uint8_t* sB, Barriers* bars, uint32_t tmem, int total, int k_iters,
                            int32_t* flags) {
+    constexpr int kStages = R::kStages;
     volatile int32_t* abort = &bars->abort;
     const int cl = int(blockIdx.x >> 1), ncl = int(gridDim.x >> 1);
     // descriptors of stage 0; a descriptor advances by (address offset) / 16
@@ -263,7 +282,7 @@ __device__ void mma_issuer(uint8_t* sA, uint8_t* sB, Barriers* bars, uint32_t tm
                 break;
             }
             tc_fence_after();
-            const uint64_t ad = adesc0 + uint64_t((stage * kABytes) >> 4);
+            const uint64_t ad = adesc0 + uint64_t((stage * R::kABytes) >> 4);
             const uint64_t bd = bdesc0 + uint64_t((stage * kBBytes) >> 4);
 #pragma unroll
             for (int k16 = 0; k16 < kBK / 16; ++k16)  // 16 columns = 32 bytes = 2 descriptor units
@@ -361,15 +380,16 @@ __device__ void epilogue(Barriers* bars, uint32_t tmem, uint32_t rank, const CUt
     __syncwarp();
 }
 
+template <class R>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     lmhead_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
-                  const __grid_constant__ CUtensorMap tmC, int M, int N, int K, float4* __restrict__ partials,
+                  const __grid_constant__ CUtensorMap tmC, int M, int N, int K, int a_bytes, float4* __restrict__ partials,
                   int32_t* flags) {
     extern __shared__ uint8_t smem_raw[];
     uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    uint8_t* sB = base;
-    uint8_t* sA = base + kStages * kBBytes;
-    uint8_t* sOut = base + kStages * kStageBytes;
+    uint8_t* sA = base;
+    uint8_t* sB = base + R::kStages * R::kABytes;
+    uint8_t* sOut = base + R::kBytes;
     Barriers* bars = reinterpret_cast<Barriers*>(sOut + kOutBytes);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t rank = cluster_rank();
@@ -379,7 +399,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     const int k_iters = (K + kBK - 1) / kBK;
 
     if (threadIdx.x == 0) {
-        for (int s = 0; s < kStages; ++s) {
+        for (int s = 0; s < R::kStages; ++s) {
             mbar_init(&bars->full[s], 1);
             mbar_init(&bars->empty[s], 1);
         }
@@ -408,9 +428,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     const uint32_t tmem = bars->tmem_base;
 
     if (warp == 0) {
-        if (lane == 0) producer(&tmA, &tmB, sA, sB, bars, rank, m_pairs, n_tiles, total, k_iters, flags);
+        if (lane == 0) producer<R>(&tmA, &tmB, sA, sB, bars, rank, m_pairs, n_tiles, total, k_iters, a_bytes, flags);
     } else if (warp == 1) {
-        if (lane == 0 && rank == 0) mma_issuer(sA, sB, bars, tmem, total, k_iters, flags);
+        if (lane == 0 && rank == 0) mma_issuer<R>(sA, sB, bars, tmem, total, k_iters, flags);
     } else {
         epilogue(bars, tmem, rank, &tmC, sOut, M, N, m_pairs, n_tiles, total, partials, flags);
     }
@@ -522,15 +542,19 @@ bool encode_map(CUtensorMap* map, const void* ptr, uint64_t rows, uint64_t cols,
 // Tensor maps, shared-memory opt-in and the persistent launch (clusters of two
 // CTAs, one CTA per SM, fewer if there are fewer tiles).  Arguments, including
 // where the operands live, are checked by the callers.
-acrl_status launch_lmhead(const acrl_bf16* hidden, int64_t M, int64_t K, int64_t ldh, const acrl_bf16* weight,
-                          int64_t N, int64_t ldw, acrl_bf16* logits, int64_t ldl, float4* partials, int32_t* flags,
-                          cudaStream_t s) {
+template <class R>
+acrl_status launch_ring(const acrl_bf16* hidden, int64_t M, int64_t K, int64_t ldh, const acrl_bf16* weight, int64_t N,
+                        int64_t ldw, acrl_bf16* logits, int64_t ldl, float4* partials, int32_t* flags, cudaStream_t s) {
+    // the short ring's boxes have the tensor's rows, in eights
+    const int a_rows = R::kARows == kBM ? kBM : int((M + 7) / 8 * 8);
     CUtensorMap tmA, tmB, tmC;
-    if (!encode_map(&tmA, hidden, uint64_t(M), uint64_t(K), uint64_t(ldh), kBM, kBK, CU_TENSOR_MAP_SWIZZLE_128B) ||
+    if (!encode_map(&tmA, hidden, uint64_t(M), uint64_t(K), uint64_t(ldh), a_rows, kBK, CU_TENSOR_MAP_SWIZZLE_128B) ||
         !encode_map(&tmB, weight, uint64_t(N), uint64_t(K), uint64_t(ldw), kHalfBN, kBK, CU_TENSOR_MAP_SWIZZLE_128B) ||
         !encode_map(&tmC, logits, uint64_t(M), uint64_t(N), uint64_t(ldl), 32, 32, CU_TENSOR_MAP_SWIZZLE_64B))
         return ACRL_ERR_CUDA;
-    if (cudaFuncSetAttribute(lmhead_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes) != cudaSuccess)
+    auto* kernel = lmhead_kernel<R>;
+    constexpr int smem = kSmemBytes<R>;
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
         return ACRL_ERR_CUDA;
     // 256 x 256 tiles; as many clusters as can be resident at once
     const int64_t total = (((M + kBM - 1) / kBM + 1) / 2) * ((N + kBN - 1) / kBN);
@@ -538,13 +562,19 @@ acrl_status launch_lmhead(const acrl_bf16* hidden, int64_t M, int64_t K, int64_t
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(2 * 1024, 1, 1);
     cfg.blockDim = dim3(kThreads, 1, 1);
-    cfg.dynamicSmemBytes = kSmemBytes;
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     int clusters = 0;
-    if (cudaOccupancyMaxActiveClusters(&clusters, lmhead_kernel, &cfg) != cudaSuccess || clusters < 1)
-        return ACRL_ERR_CUDA;
+    if (cudaOccupancyMaxActiveClusters(&clusters, kernel, &cfg) != cudaSuccess || clusters < 1) return ACRL_ERR_CUDA;
     const int grid = int(2 * (total < clusters ? total : clusters));
-    return launch(lmhead_kernel, grid, kThreads, kSmemBytes, 0, s, tmA, tmB, tmC, int(M), int(N), int(K), partials, flags);
+    return launch(kernel, grid, kThreads, smem, 0, s, tmA, tmB, tmC, int(M), int(N), int(K), a_rows * kBK * 2, partials,
+                  flags);
+}
+
+acrl_status launch_lmhead(const acrl_bf16* hidden, int64_t M, int64_t K, int64_t ldh, const acrl_bf16* weight, int64_t N,
+                          int64_t ldw, acrl_bf16* logits, int64_t ldl, float4* partials, int32_t* flags, cudaStream_t s) {
+    auto* run = M <= Ring16::kARows ? launch_ring<Ring16> : launch_ring<RingFull>;
+    return run(hidden, M, K, ldh, weight, N, ldw, logits, ldl, partials, flags, s);
 }
 
 // True when every pointer is device memory of the current device: not managed

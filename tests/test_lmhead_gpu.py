@@ -77,6 +77,14 @@ def test_lmhead_small_shapes(M, N, K):
     assert_close_rel(host(ent), oH, floor=1e-5, what="entropy")
 
 
+# the ring for up to 16 rows at its ends, with boxes of one and two eights of rows; more K slabs than stages, so
+# that it wraps, with K on and off the slab
+@pytest.mark.parametrize("M,N,K", [(1, 513, 1000), (8, 700, 1032), (9, 300, 64), (16, 1000, 2048), (17, 513, 1000)])
+def test_lmhead_few_rows(M, N, K):
+    test_lmhead_small_shapes(M, N, K)
+
+
+
 def test_lmhead_matches_token_stats_on_same_logits():
     """The fused statistics equal acrl_token_stats run on the logits the GEMM wrote."""
     M, N, K = 256, 32000, 512

@@ -28,14 +28,23 @@ namespace {
 
 constexpr uint32_t kSignPair = 0x80008000u;
 
-// CTA kernel: 512 threads, four 16-byte vectors per thread and step.  Its
-// recompute path keeps kKeepVecs vectors of a row in shared memory between the
-// sweeps (96 KB, three whole sweep chunks; two 512-thread CTAs per SM).
+// CTA kernel: four 16-byte vectors per thread and step.  The recompute path of
+// long rows takes 512 threads and keeps kKeepVecs vectors of a row in shared memory
+// between the sweeps (96 KB, three whole sweep chunks; two 512-thread CTAs per SM).
 constexpr int kCtaThreads = 512, kCtaUnroll = 4;
-// The streaming path (lse given) takes 768-thread CTAs for rows of more than
-// 65,536 columns: 1.02-1.04 of the copy rate there against 0.99-1.02 with 512
-// threads (whose last step over such a row is more ragged); 512 stay best for
-// shorter rows.
+// The streaming path (lse given) takes a CTA per row, of the most threads that the
+// row keeps busy for one whole step (the smallest for a row of 2,048 columns is 64
+// threads; 512 from 16,384 columns), and below that a warp per row.  Fewer threads
+// leave the row's later steps to wait for memory one after the other, more leave
+// threads idle or the last step ragged.  Kernel with its loss sum, us, warp per row
+// (what rows of up to 16,384 columns took before) and now: 1,000 x 2,048 5.3 / 5.0;
+// 8,000 x 2,600 21.1 / 19.2; 8,000 x 4,096 27.9 / 24.5; 1,000 x 5,003 11.7 / 8.4;
+// 8,000 x 5,003 38.1 / 30.7; 300 x 8,192 8.8 / 4.6; 30,000 x 8,192 150.8 / 144.7;
+// 8,000 x 10,007 68.3 / 52.1; 20,000 x 14,001 179.4 / 168.5; 600 x 16,384 18.4 /
+// 10.2; 20,000 x 16,384 208 / 189 (a copy of the bytes: 196).  Rows of more than
+// 65,536 columns: 768 threads, 1.02-1.04 of the copy rate there against 0.99-1.02
+// with 512 (whose last step over such a row is more ragged).
+constexpr int kStreamStep = 8 * kCtaUnroll;   // columns of one thread's step
 constexpr int kWideThreads = 768;
 constexpr int64_t kWideRowMinV = 65537;
 constexpr int kChunk = kCtaThreads * kCtaUnroll;   // vectors one sweep step of the CTA covers
@@ -662,9 +671,13 @@ acrl_status launch_loss_grad(const acrl_bf16* logits, int64_t T, int V, int64_t 
         if (nvec >= kTmemMinVecs) return run(loss_grad_cta<kCtaThreads, U, true, ENT, true>, 1, kCtaThreads, kKeepVecs);
         return run(loss_grad_cta<kCtaThreads, U, true, ENT>, 1, kCtaThreads, kKeepVecs);
     } else {
-        if (V <= kWarpRowMaxV) return run(loss_grad_warp<256, U, false, ENT>, 8, 256, 0);
         if (V >= kWideRowMinV) return run(loss_grad_cta<kWideThreads, U, false, ENT>, 1, kWideThreads, 0);
-        return run(loss_grad_cta<kCtaThreads, U, false, ENT>, 1, kCtaThreads, 0);
+        if (V >= 512 * kStreamStep) return run(loss_grad_cta<512, U, false, ENT>, 1, 512, 0);
+        if (V >= 384 * kStreamStep) return run(loss_grad_cta<384, U, false, ENT>, 1, 384, 0);
+        if (V >= 256 * kStreamStep) return run(loss_grad_cta<256, U, false, ENT>, 1, 256, 0);
+        if (V >= 128 * kStreamStep) return run(loss_grad_cta<128, U, false, ENT>, 1, 128, 0);
+        if (V >= 64 * kStreamStep) return run(loss_grad_cta<64, U, false, ENT>, 1, 64, 0);
+        return run(loss_grad_warp<256, U, false, ENT>, 8, 256, 0);
     }
 }
 

@@ -2,7 +2,7 @@
 // giving the log-sum-exp, the sampled token's log-prob and the entropy.
 //
 // Each row is read exactly once from HBM in 16-byte loads that L1 does not keep.
-// A team of threads (eight lanes for rows of up to 4,096 columns, a warp for
+// A team of threads (eight or sixteen lanes for the shortest rows, a warp for
 // other short rows, the whole CTA for vocabulary-size rows) owns a row; every
 // thread keeps an online base-2 state (max, sum 2^(u-U), sum 2^(u-U)(u-U))
 // over its strided share of the row, and the team merges the states with a
@@ -102,11 +102,11 @@ __global__ void __launch_bounds__(THREADS) token_stats_warp(const acrl_bf16* __r
     }
 }
 
-// Short rows (V <= kTeamRowMaxV): LANES lanes per row, 32 / LANES rows per warp
-// at a time.  The team merges its states over log2(LANES) shuffle levels
-// instead of five, which matters where the merges' exponentials are a large
-// share of the row's (V = 2,048: 0.75 -> 0.94 of the copy rate with 8 lanes).
-// Every lane takes part in the shuffles, whether its row is masked or not.
+// The shortest rows: LANES lanes per row, 32 / LANES rows per warp at a time.
+// The team merges its states over log2(LANES) shuffle levels instead of five,
+// which matters where the merges' exponentials are a large share of the row's
+// (V = 2,048: 0.75 -> 0.94 of the copy rate with 8 lanes).  Every lane takes part
+// in the shuffles, whether its row is masked or not.
 template <int LANES>
 __device__ __forceinline__ LseAcc team_lse(LseAcc a) {
 #pragma unroll
@@ -153,12 +153,18 @@ __global__ void __launch_bounds__(THREADS) token_stats_team(const acrl_bf16* __r
     }
 }
 
-// Rows up to this many columns (8 KB) are shared by eight lanes each, up to
-// kWarpRowMaxV by a warp, up to kMidRowMaxV (128 KB) by two warps (2 % faster
-// than four at V = 32,000), longer ones by four: many independent rows in
-// flight per SM and a short end-of-row merge (measured best of teams of 8 to
-// 1,024 threads).
-constexpr int64_t kTeamRowMaxV = 4096, kMidRowMaxV = 65536;
+// Rows up to kTeamRowMaxV columns are shared by eight lanes each, up to
+// kTeam16RowMaxV by sixteen, up to kWarpRowMaxV by a warp, up to kMidRowMaxV
+// (80 KB) by two warps, longer ones by four: many independent rows in flight per SM
+// and a short end-of-row merge (measured best of teams of 8 to 1,024 threads).  The
+// line depends on V alone, so that a row's result does not depend on the batch it
+// is in.  Where they lie, us: V = 4,096, T = 1,024 / 8,000 / 30,000: eight lanes
+// 6.0 / 14.2 / 43.1, sixteen 3.9 / 14.1 / 40.8, a warp 3.3 / 15.3 / 43.8; V = 3,333:
+// eight 5.9 / 12.9 / 35.7, sixteen 3.9 / 13.9 / 36.4; V = 5,003: sixteen 5.2 / 18.9 /
+// 51.9, a warp 4.4 / 19.3 / 56.9.  V = 49,152, T = 300 / 1,340 / 4,000 / 16,000: two
+// warps 10.2 / 24.7 / 63.8 / 225, four 8.3 / 22.0 / 60.3 / 219; V = 40,000, T = 400 /
+// 3,000 / 10,000: two 10.8 / 39.3 / 123, four 8.9 / 40.8 / 119.
+constexpr int64_t kTeamRowMaxV = 3584, kTeam16RowMaxV = 4608, kMidRowMaxV = 40960;
 constexpr int kUnroll = 4;
 
 // Steps of the ring: with few rows per SM, one step of loads per thread leaves
@@ -175,16 +181,19 @@ constexpr int kDepth = 3;
 //   row: only up to 7.5 (V = 16,384, T = 4,096: 25.8 against 26.5).
 // - Many: the ring for rows of a warp or less (V = 16,384, T = 65,536: 296 us
 //   against 317; V = 8,192: 153 against 162; V = 4,096: 82 against 88), the
-//   same for four warps a row; registers for two warps a row (V = 20,011,
-//   T = 65,536: 389 against 402; 49,152, T = 40,000: 548 against 553), except
-//   just past one wave (V = 32,000, T = 3,500: 45 against 40).
-bool use_ring(int64_t T, int team) {
+//   same for four warps a row.  Two warps a row: registers where the row's last
+//   step is a large part of it (V = 20,011: a step of 12,000 rows 254 us against
+//   257, of 40,000 750 against 762) and up to some 2.5 waves (V = 32,000, 5,000
+//   rows: 174 against 181), except just past one wave (V = 32,000, T = 3,500: 45
+//   against 40); else the ring (V = 32,000, steps of 16,000 and 38,000 rows: 485
+//   and 1,084 against 480 and 1,072).
+bool use_ring(int64_t T, int team, int V) {
     constexpr int64_t kSms = 152;
     const int64_t q = T >= (int64_t(1) << 40) ? INT64_MAX : T * team * 10 / (128 * kSms);
-    if (team == 8) return true;
+    if (team <= 16) return true;
     if (q < 52) return true;
     if (team == 32) return q > 75;
-    if (team == 64) return q > 104 && q < 140;
+    if (team == 64) return V >= 28672 ? q > 400 || (q > 104 && q < 140) : q > 104 && q < 140;
     return q > 104;
 }
 
@@ -208,9 +217,14 @@ extern "C" acrl_status acrl_token_stats(const acrl_bf16* logits, int64_t T, int6
         return launch(kernel, grid_for(rows_per_cta, T), threads, size_t(threads) * kUnroll * depth * 16, 0, s, logits, T,
                       v, ld, ids, mask, lse, logp, entropy, dev_flags);
     };
-    const int team = V <= kTeamRowMaxV ? 8 : V <= kWarpRowMaxV ? 32 : V <= kMidRowMaxV ? 64 : 128;
-    const bool ring = use_ring(T, team);
+    const int team = V <= kTeamRowMaxV     ? 8
+                     : V <= kTeam16RowMaxV ? 16
+                     : V <= kWarpRowMaxV   ? 32
+                     : V <= kMidRowMaxV    ? 64
+                                           : 128;
+    const bool ring = use_ring(T, team, v);
     if (team == 8) return run(token_stats_team<64, kUnroll, 8, kDepth>, 64, kDepth, 8);
+    if (team == 16) return run(token_stats_team<64, kUnroll, 16, kDepth>, 64, kDepth, 4);
     if (team == 32)
         return ring ? run(token_stats_warp<64, kUnroll, kDepth>, 64, kDepth, 2)
                     : run(token_stats_warp<256, kUnroll, 0>, 256, 0, 8);

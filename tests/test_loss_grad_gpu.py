@@ -1,0 +1,51 @@
+"""acrl_loss_grad_logits with the lse given, where the CTA that a row gets changes
+size: rows one column short of, at and past the lines, rows shorter than a
+step, with one to seven columns beyond whole vectors, against float64."""
+
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+from paper_2607_24062_gb300 import api  # noqa: E402
+
+DEV = "cuda"
+
+
+@pytest.mark.parametrize("V", [1, 7, 257, 2047, 2048, 2049, 3333, 4095, 4096, 4097, 6145, 8191, 8192, 8193, 12287, 12288, 12289,
+                               16383, 16384, 16385, 20011, 65536, 65537, 100003])
+@pytest.mark.parametrize("bonus", [False, True])
+def test_streaming_gradient_by_row_length(V, bonus):
+    gen = torch.Generator(device=DEV).manual_seed(V)
+    T, ld = 37, (V + 7) // 8 * 8
+    x = torch.full((T, ld), float("nan"), dtype=torch.bfloat16, device=DEV)   # columns past V are never used
+    x[:, :V] = torch.randn((T, V), generator=gen, device=DEV) * 2
+    ids = torch.randint(0, V, (T,), generator=gen, device=DEV, dtype=torch.int32)
+    mask = (torch.arange(T, device=DEV) % 5 != 1).to(torch.uint8)
+    coef = torch.randn(T, generator=gen, device=DEV) * 1e-2
+    coef[3] = 0.0
+    z = x[:, :V].double()
+    lse = z.logsumexp(dim=1)
+    lp = z - lse[:, None]
+    H = -(lp.exp() * lp).sum(dim=1)
+    e = mask * 1e-3 if bonus else None
+    flags = api.new_flags()
+    grad = torch.full((T, ld), 5.0, dtype=torch.bfloat16, device=DEV)
+    g, tl, loss = api.loss_grad_logits(x, ids, mask, lse.float(), None, coef * mask, 0.2, V=V, grad=grad, flags=flags,
+                                       entropy=H.float() if bonus else None, ent_coef=e)
+    assert api.read_flags(flags) == 0
+    c = (coef * mask).double()
+    p = lp.exp()
+    want = p * c[:, None]
+    want.scatter_add_(1, ids.long()[:, None], -c[:, None])
+    if bonus:
+        want += e.double()[:, None] * p * (lp + H[:, None])
+    # bf16 rounding of the result, and the fp32 rounding of lse and of the exponent (2^-24 of some 30) on its terms
+    size = p * (c.abs()[:, None] + (e.double()[:, None] * (lp.abs() + H[:, None]) if bonus else 0.0))
+    size.scatter_add_(1, ids.long()[:, None], c.abs()[:, None])
+    assert bool(((g[:, :V].double() - want).abs() <= 2.0 ** -8 * want.abs() + 2.0 ** -17 * size + 1e-38).all())
+    assert bool((g[:, V:] == 5.0).all())
+    want_tl = -c - (e.double() * H if bonus else 0.0)
+    assert bool(((tl.double() - want_tl).abs() <= 2.0 ** -22 * (c.abs() + (e.double() * H if bonus else 0.0)) + 1e-30).all())
+    whole = tl.double().sum()
+    assert abs(float(loss) - float(whole)) <= 2.0 ** -21 * float(tl.double().abs().sum()) + 1e-30

@@ -13,14 +13,14 @@ from paper_2607_24062_gb300 import api  # noqa: E402
 
 DEV = "cuda"
 
-# team of 8: steps of 256 columns; 32: 1,024; 64: 2,048; 128: 4,096
-_WIDTHS = [1, 8, 63, 64, 255, 256, 257, 767, 768, 769, 1024, 4095, 4096, 4097, 5119, 5120, 5121, 7168, 16383, 16384, 16385,
-           18431, 18432, 18441, 20011, 32000, 65535, 65536, 65537, 65544, 69632, 69640, 100003, 151936]
+# team of 8: steps of 256 columns; 16: 512; 32: 1,024; 64: 2,048; 128: 4,096
+_WIDTHS = [1, 8, 63, 64, 255, 256, 257, 767, 768, 769, 1024, 4095, 4096, 4097, 5119, 5120, 5121, 3584, 3585, 4608, 4609, 7168, 16383, 16384, 16385,
+           18431, 18432, 18441, 20011, 32000, 40960, 40961, 65535, 65536, 65537, 65544, 69632, 69640, 100003, 151936]
 
 
 def _many(V):
     """Rows that put the call on the register path (teams per SM between 5.2 and 7.5)."""
-    team = 8 if V <= 4096 else 32 if V <= 16384 else 64 if V <= 65536 else 128
+    team = 8 if V <= 4608 else 32 if V <= 16384 else 64 if V <= 40960 else 128
     return 6 * 128 * 152 // team if team > 8 else 4096
 
 

@@ -13,7 +13,7 @@
 // coefficient and no bonus, clipped) are written as zeros without reading
 // their logits.  With lse == NULL the row's log-sum-exp is first recomputed
 // by a sweep over the same row; the first 16-byte vectors of the row (up to
-// 40, 72 or 96 KB, by the CTA's size) stay in the CTA's shared memory and, for
+// 20, 40, 72 or 96 KB, by the CTA's size) stay in the CTA's shared memory and, for
 // rows of 65,536 columns or more, the next up to kTmemVecs (128 KB) in its
 // tensor memory between the two sweeps, so that only the rest of the row is
 // read again, from L2.  The shared-memory part arrives by one bulk copy
@@ -67,30 +67,32 @@ static_assert(kCtaThreads == 512 && kCtaUnroll == 4, "column layout: 16 warps, 4
 // until it has given up its allocation permit: measured with ncu, 15.6 warps
 // resident per SM against 30.7 for the same work without tcgen05 code.
 constexpr int kTmemMinVecs = kKeepVecs + kChunk;
-// Longer rows of up to kSmallMaxVecs vectors (V <= 40,967) take 256-thread CTAs in
-// the recompute path, each keeping up to 72 KB of its row in shared memory so
-// that three fit on an SM (the rest of the row, at most 8 KB, is read again
-// from L2): 0.92-0.98 of the copy rate for V = 32,000-40,000 against 0.77-0.85
-// with two 512-thread CTAs per SM; from V = 44,000 the 512-thread CTAs, which
-// keep 96 KB, are ahead (0.87-0.93 against 0.82-0.87).
-constexpr int kSmallThreads = 256;
-constexpr int kSmallKeepVecs = 4608;
+// Shorter rows take smaller CTAs, so that several fit on an SM with what they keep:
+//   from kRecomputeCtaMinV columns  64 threads,  up to 20 KB: rows of up to 7,168
+//   up to kTinyKeepVecs vectors    128 threads,  up to 40 KB: V <= 20,487
+//   up to kSmallMaxVecs vectors    256 threads,  up to 72 KB: V <= 40,967 (of a row
+//                                  longer than 72 KB the rest, at most 8 KB, is read
+//                                  again from L2)
+// and those below a warp each, which reads its row again from L2.  Us, the call with
+// its loss sum: 30,000 x 5,003 126 with a warp, 102 with 64 threads, 131 with 128;
+// 8,000 x 6,200 45 / 37 / 44; 1,000 x 8,192 15.5 / 12.5 / 11.8; 16,000 x 14,001
+// 199 with 64, 137 with 128, 174 with 256; 10,000 x 24,000 219 with 128 (whose rest
+// of the row is a ragged step in each sweep), 151 with 256, 215 with 512; 2,000 x
+// 44,000 79 with 256, 68 with 512; 30,000 x 3,333 77 with a warp (in CTAs of two; 83
+// in CTAs of eight), 84 with 64 threads.
+constexpr int kRecomputeCtaMinV = 4096;
+constexpr int kLeastThreads = 64, kLeastKeepVecs = 1280;
+constexpr int kLeastMaxV = 7168;
+constexpr int kTinyThreads = 128, kTinyKeepVecs = 2560;
+constexpr int kSmallThreads = 256, kSmallKeepVecs = 4608;
 constexpr int kSmallMaxVecs = 5120;
-// Rows of up to kTinyMaxVecs vectors (V <= 24,583) take 128-thread CTAs that
-// keep up to 40 KB of the row (five or more CTAs per SM; the rest, at most
-// 8 KB, is read again from L2): 0.95-1.04 of the copy rate for V = 8,192-
-// 24,576, where one warp per row, reading the whole row again from L2, reached
-// 0.70-0.87 (32 rows of 32 KB in flight per SM no longer fit in L2 at
-// V = 16,384).  Rows of up to kRecomputeWarpMaxV columns keep one warp per
-// row (0.95 against 0.82 at V = 6,144).
-constexpr int kTinyThreads = 128;
-constexpr int kTinyKeepVecs = 2560;
-constexpr int kTinyMaxVecs = 3072;
-constexpr int kRecomputeWarpMaxV = 6144;
 
 // Vectors of a row that a recompute CTA of THREADS threads keeps in shared memory.
 template <int THREADS>
-constexpr int kKeepOf = THREADS == kTinyThreads ? kTinyKeepVecs : THREADS == kSmallThreads ? kSmallKeepVecs : kKeepVecs;
+constexpr int kKeepOf = THREADS == kLeastThreads   ? kLeastKeepVecs
+                        : THREADS == kTinyThreads  ? kTinyKeepVecs
+                        : THREADS == kSmallThreads ? kSmallKeepVecs
+                                                   : kKeepVecs;
 
 // Where the vectors of a row live between the two sweeps of the recompute
 // path: [0, s) in `smem` (filled by a bulk copy that completes on `bar`),
@@ -217,11 +219,15 @@ __device__ __forceinline__ LseAcc recompute_partial(const acrl_bf16* __restrict_
         for (int k = 0; k < UNROLL; ++k) buf[k] = ld_policy(vrow + v + k * TEAM, pol);
         fold_vectors<UNROLL>(acc, mx, buf);
     }
-    for (; v < nvec; v += TEAM) {
-        uint4 buf[1] = {ld_policy(vrow + v, pol)};
-        fold_vectors<1>(acc, mx, buf);
-    }
-    for (int j = (nvec << 3) + tid; j < V; j += TEAM) fold_scalar(acc, mx, bf16_to_float(row[j]));
+    const int j = (nvec << 3) + tid;   // at most one column per thread beyond the whole vectors
+    const float last = j < V ? bf16_to_float(row[j]) : 0.f;
+    rest_of_row<TEAM>(
+        v, nvec, [&](int i) { return ld_policy(vrow + i, pol); },
+        [&](const uint4& x, int) {
+            const uint4 buf[1] = {x};
+            fold_vectors<1>(acc, mx, buf);
+        });
+    if (j < V) fold_scalar(acc, mx, last);
     if (s > 0) {
         if (!wait_phase(kp.bar, parity, nullptr)) raise_flag(flags, ACRL_FLAG_TIMEOUT);
         for (v = tid; v + (UNROLL - 1) * TEAM < s; v += UNROLL * TEAM) {
@@ -264,7 +270,9 @@ __device__ __forceinline__ void stream_grad_row(const acrl_bf16* __restrict__ ro
                 st_stream(dst + vi, grad_vec<ENT>(buf[k], rp, rp.a - (vi << 3)));
             }
         }
-        for (; v < nvec; v += TEAM) st_stream(dst + v, grad_vec<ENT>(ld_policy(src + v, pol), rp, rp.a - (v << 3)));
+        rest_of_row<TEAM>(
+            v, nvec, [&](int i) { return ld_policy(src + i, pol); },
+            [&](const uint4& x, int i) { st_stream(dst + i, grad_vec<ENT>(x, rp, rp.a - (i << 3))); });
         for (int ch = 0; TM && ch < kp.tm_chunks; ++ch) {
             uint4 buf[UNROLL];
 #pragma unroll
@@ -664,8 +672,9 @@ acrl_status launch_loss_grad(const acrl_bf16* logits, int64_t T, int V, int64_t 
     constexpr int U = kCtaUnroll;
     if constexpr (RECOMPUTE) {
         const int nvec = V >> 3;
-        if (V <= kRecomputeWarpMaxV) return run(loss_grad_warp<256, U, true, ENT>, 8, 256, 0);
-        if (nvec <= kTinyMaxVecs) return run(loss_grad_cta<kTinyThreads, U, true, ENT>, 1, kTinyThreads, kTinyKeepVecs);
+        if (V < kRecomputeCtaMinV) return run(loss_grad_warp<64, U, true, ENT>, 2, 64, 0);
+        if (V <= kLeastMaxV) return run(loss_grad_cta<kLeastThreads, U, true, ENT>, 1, kLeastThreads, kLeastKeepVecs);
+        if (nvec <= kTinyKeepVecs) return run(loss_grad_cta<kTinyThreads, U, true, ENT>, 1, kTinyThreads, kTinyKeepVecs);
         if (nvec <= kSmallMaxVecs)
             return run(loss_grad_cta<kSmallThreads, U, true, ENT>, 1, kSmallThreads, kSmallKeepVecs);
         if (nvec >= kTmemMinVecs) return run(loss_grad_cta<kCtaThreads, U, true, ENT, true>, 1, kCtaThreads, kKeepVecs);
@@ -677,7 +686,7 @@ acrl_status launch_loss_grad(const acrl_bf16* logits, int64_t T, int V, int64_t 
         if (V >= 256 * kStreamStep) return run(loss_grad_cta<256, U, false, ENT>, 1, 256, 0);
         if (V >= 128 * kStreamStep) return run(loss_grad_cta<128, U, false, ENT>, 1, 128, 0);
         if (V >= 64 * kStreamStep) return run(loss_grad_cta<64, U, false, ENT>, 1, 64, 0);
-        return run(loss_grad_warp<256, U, false, ENT>, 8, 256, 0);
+        return run(loss_grad_warp<64, U, false, ENT>, 2, 64, 0);
     }
 }
 

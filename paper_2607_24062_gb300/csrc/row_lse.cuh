@@ -69,6 +69,24 @@ __device__ __forceinline__ void fold_scalar(LseAcc& acc, float& mx, float z) {
     acc.s1 = fmaf(e, y, acc.s1);
 }
 
+// The ragged last step of a sweep: vectors v, v + TEAM, ... below n, the next one
+// loaded before one is used (two loads in flight, and few registers).
+template <int TEAM, typename Load, typename Use>
+__device__ __forceinline__ void rest_of_row(int v, int n, Load load, Use use) {
+    if (v >= n) return;
+    uint4 cur = load(v);
+#pragma unroll 1
+    for (;;) {
+        const int w = v + TEAM;
+        uint4 next = cur;
+        if (w < n) next = load(w);
+        use(cur, v);
+        if (w >= n) return;
+        cur = next;
+        v = w;
+    }
+}
+
 // The thread's partial state over its share of one row (lane `tid` of a team of TEAM threads).
 template <int TEAM, int UNROLL>
 __device__ __forceinline__ LseAcc row_partial(const acrl_bf16* __restrict__ row, int V, int tid, float& mx) {

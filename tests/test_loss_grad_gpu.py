@@ -1,6 +1,7 @@
-"""acrl_loss_grad_logits with the lse given, where the CTA that a row gets changes
-size: rows one column short of, at and past the lines, rows shorter than a
-step, with one to seven columns beyond whole vectors, against float64."""
+"""acrl_loss_grad_logits where the CTA that a row gets changes size, with the lse
+given and recomputed: rows one column short of, at and past the lines, rows
+shorter than a step, with one to seven columns beyond whole vectors and with a
+ragged rest beyond what the CTA keeps on chip, against float64."""
 
 import pytest
 import torch
@@ -16,6 +17,17 @@ DEV = "cuda"
                                16383, 16384, 16385, 20011, 65536, 65537, 100003])
 @pytest.mark.parametrize("bonus", [False, True])
 def test_streaming_gradient_by_row_length(V, bonus):
+    _check(V, bonus, recompute=False)
+
+
+@pytest.mark.parametrize("V", [1, 7, 1025, 4095, 4096, 4097, 7168, 7169, 10240, 10243, 20480, 20487, 20488, 24007, 36864, 40001,
+                               40967, 40968, 49155, 61003, 65535, 65536, 70001])
+@pytest.mark.parametrize("bonus", [False, True])
+def test_recomputed_gradient_by_row_length(V, bonus):
+    _check(V, bonus, recompute=True)
+
+
+def _check(V, bonus, recompute):
     gen = torch.Generator(device=DEV).manual_seed(V)
     T, ld = 37, (V + 7) // 8 * 8
     x = torch.full((T, ld), float("nan"), dtype=torch.bfloat16, device=DEV)   # columns past V are never used
@@ -31,7 +43,7 @@ def test_streaming_gradient_by_row_length(V, bonus):
     e = mask * 1e-3 if bonus else None
     flags = api.new_flags()
     grad = torch.full((T, ld), 5.0, dtype=torch.bfloat16, device=DEV)
-    g, tl, loss = api.loss_grad_logits(x, ids, mask, lse.float(), None, coef * mask, 0.2, V=V, grad=grad, flags=flags,
+    g, tl, loss = api.loss_grad_logits(x, ids, mask, None if recompute else lse.float(), None, coef * mask, 0.2, V=V, grad=grad, flags=flags,
                                        entropy=H.float() if bonus else None, ent_coef=e)
     assert api.read_flags(flags) == 0
     c = (coef * mask).double()

@@ -41,12 +41,19 @@ constexpr int kCtaThreads = 512, kCtaUnroll = 4;
 // 8,000 x 2,600 21.1 / 19.2; 8,000 x 4,096 27.9 / 24.5; 1,000 x 5,003 11.7 / 8.4;
 // 8,000 x 5,003 38.1 / 30.7; 300 x 8,192 8.8 / 4.6; 30,000 x 8,192 150.8 / 144.7;
 // 8,000 x 10,007 68.3 / 52.1; 20,000 x 14,001 179.4 / 168.5; 600 x 16,384 18.4 /
-// 10.2; 20,000 x 16,384 208 / 189 (a copy of the bytes: 196).  Rows of more than
-// 65,536 columns: 768 threads, 1.02-1.04 of the copy rate there against 0.99-1.02
-// with 512 (whose last step over such a row is more ragged).
+// 10.2; 20,000 x 16,384 208 / 189 (a copy of the bytes: 196).
 constexpr int kStreamStep = 8 * kCtaUnroll;   // columns of one thread's step
+// Rows of more than 65,536 columns are split between CTAs of 256 threads, two whole
+// steps and a little more for each (nine for 151,936 columns): more of the row is in
+// flight when rows are few, the chip stays even when they are many, and a ragged
+// last step is short.  A CTA of 768 threads per row / split: 40 x 151,936 12.7 / 9.2
+// us, 408 x 151,936 42.4 / 41.2, 700 x 151,936 69.7 / 65.9, 3,000 x 151,936 268 / 262,
+// 3,000 x 65,544 123.5 / 117.8, 3,000 x 200,000 355 / 343; with 6 to 8 shares of
+// 151,936 columns 66.7, with 11 to 14 68.
+constexpr int kShareThreads = 256, kShareVecs = 2 * kShareThreads * kCtaUnroll;
+constexpr int64_t kShareRowMinV = 65537;
+// A call of so many rows that the shares would not fit a grid takes a CTA per row.
 constexpr int kWideThreads = 768;
-constexpr int64_t kWideRowMinV = 65537;
 constexpr int kChunk = kCtaThreads * kCtaUnroll;   // vectors one sweep step of the CTA covers
 constexpr int kKeepVecs = 3 * kChunk;
 static_assert(kKeepVecs * 16 <= 100 * 1024, "two CTAs per SM must fit");
@@ -130,6 +137,13 @@ __device__ __forceinline__ uint4 tmem_ld4(uint32_t taddr) {
 }
 __device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+
+// The vectors [begin, end) of a row that a CTA handles: all of them, or one of the
+// shares of a row that several CTAs split; the first share's CTA also writes what
+// there is one of per row.
+struct RowShare {
+    int begin, end;
+};
 
 // Per-row constants of the streaming pass.
 struct RowPlan {
@@ -251,9 +265,8 @@ __device__ __forceinline__ LseAcc recompute_partial(const acrl_bf16* __restrict_
 // then the vectors in shared memory.
 template <int TEAM, int UNROLL, bool ENT, bool LAST = false, bool TM = false>
 __device__ __forceinline__ void stream_grad_row(const acrl_bf16* __restrict__ row, acrl_bf16* __restrict__ grow, int V,
-                                                int tid, const RowPlan& rp,
-                                                const RowKeep& kp = RowKeep{nullptr, 0, 0u, 0, nullptr}) {
-    const int nvec = V >> 3;
+                                                int tid, const RowPlan& rp, const RowKeep& kp, const RowShare& sh) {
+    const int nvec = LAST ? V >> 3 : sh.end;
     const uint4* src = reinterpret_cast<const uint4*>(row);
     uint4* dst = reinterpret_cast<uint4*>(grow);
     if (LAST) {
@@ -287,7 +300,7 @@ __device__ __forceinline__ void stream_grad_row(const acrl_bf16* __restrict__ ro
         }
         for (int vi = tid; vi < kp.s; vi += TEAM) st_stream(dst + vi, grad_vec<ENT>(kp.smem[vi], rp, rp.a - (vi << 3)));
     } else {
-        int v = tid;
+        int v = sh.begin + tid;
         for (; v + (UNROLL - 1) * TEAM < nvec; v += UNROLL * TEAM) {
             uint4 buf[UNROLL];
 #pragma unroll
@@ -300,6 +313,7 @@ __device__ __forceinline__ void stream_grad_row(const acrl_bf16* __restrict__ ro
         }
         for (; v < nvec; v += TEAM) st_stream(dst + v, grad_vec<ENT>(ld_stream(src + v), rp, rp.a - (v << 3)));
     }
+    if (nvec != V >> 3) return;   // the columns beyond the whole vectors are the last share's
     for (int j = (nvec << 3) + tid; j < V; j += TEAM) {
         float val = grad_elem<ENT>(bf16_to_float(row[j]), rp);
         if (!ENT && rp.sgn) val = -val;
@@ -314,11 +328,12 @@ __device__ __forceinline__ void stream_grad_row(const acrl_bf16* __restrict__ ro
 constexpr uint32_t kZeroPair = 0u, kNaNPair = 0x7FC07FC0u;
 
 template <int TEAM>
-__device__ __forceinline__ void fill_row(acrl_bf16* __restrict__ grow, int V, int tid, uint32_t pair) {
-    const int nvec = V >> 3;
+__device__ __forceinline__ void fill_row(acrl_bf16* __restrict__ grow, int V, int tid, uint32_t pair, const RowShare& sh) {
+    const int nvec = sh.end;
     uint4* dst = reinterpret_cast<uint4*>(grow);
     const uint4 z = make_uint4(pair, pair, pair, pair);
-    for (int v = tid; v < nvec; v += TEAM) st_stream(dst + v, z);
+    for (int v = sh.begin + tid; v < nvec; v += TEAM) st_stream(dst + v, z);
+    if (nvec != V >> 3) return;
     for (int j = (nvec << 3) + tid; j < V; j += TEAM) grow[j] = static_cast<acrl_bf16>(pair & 0xffffu);
 }
 
@@ -385,7 +400,7 @@ __device__ __forceinline__ void grad_row(const acrl_bf16* __restrict__ logits, i
                                          const float* __restrict__ coef, const float* __restrict__ entropy,
                                          const float* __restrict__ ent_coef, float eps, acrl_bf16* __restrict__ grad,
                                          float* __restrict__ token_loss, int32_t* flags, int tid, LseAcc* part,
-                                         float* part_mx, int& par, const RowKeep& kp) {
+                                         float* part_mx, int& par, const RowKeep& kp, const RowShare& sh) {
     const acrl_bf16* row = logits + t * ld;
     acrl_bf16* grow = grad + t * ld;
     const bool m = mask ? mask[t] != 0 : true;
@@ -393,7 +408,8 @@ __device__ __forceinline__ void grad_row(const acrl_bf16* __restrict__ logits, i
     const float e = ENT ? ent_coef[t] : 0.f;
     const int a = ids[t];
     const bool bad_id = a < 0 || a >= V;
-    if (m && bad_id && tid == 0) raise_flag(flags, ACRL_FLAG_BAD_ID);
+    const bool lead = tid == 0 && sh.begin == 0;
+    if (m && bad_id && lead) raise_flag(flags, ACRL_FLAG_BAD_ID);
     const bool live = m && !bad_id && (c0 != 0.f || e != 0.f);
     float c = 0.f, loss = 0.f, L = 0.f, H = 0.f, za = 0.f, lp = 0.f;
     bool undefined = false;
@@ -445,7 +461,7 @@ __device__ __forceinline__ void grad_row(const acrl_bf16* __restrict__ logits, i
         // a row whose lse or log-prob is not finite (a NaN or an infinity among its logits), or whose old
         // log-prob is NaN, has no defined surrogate: NaN token loss and gradient row, and the flag
         undefined = !isfinite(L) || !isfinite(lp) || (old_logp != nullptr && isnan(old_logp[t]));
-        if (undefined && tid == 0) raise_flag(flags, ACRL_FLAG_NONFINITE);
+        if (undefined && lead) raise_flag(flags, ACRL_FLAG_NONFINITE);
         const RowCoef rc = row_coef(c0, lp, old_logp, t, eps);
         c = rc.c;
         loss = rc.loss;
@@ -454,25 +470,26 @@ __device__ __forceinline__ void grad_row(const acrl_bf16* __restrict__ logits, i
             loss -= e * H;
         }
     }
-    if (tid == 0) token_loss[t] = undefined ? __int_as_float(0x7fc00000) : loss;
+    if (lead) token_loss[t] = undefined ? __int_as_float(0x7fc00000) : loss;
     if (undefined) {
-        fill_row<TEAM>(grow, V, tid, kNaNPair);
+        fill_row<TEAM>(grow, V, tid, kNaNPair, sh);
     } else if (c == 0.f && e == 0.f) {
-        fill_row<TEAM>(grow, V, tid, kZeroPair);
+        fill_row<TEAM>(grow, V, tid, kZeroPair, sh);
     } else {
         stream_grad_row<TEAM, UNROLL, ENT, RECOMPUTE, TM>(row, grow, V, tid, make_plan<ENT>(c, e, L, H, za, lp, a),
-                                                          kp);
+                                                          kp, sh);
     }
 }
 
 // TM: the recompute instance whose CTAs keep whole chunks of a row in tensor
-// memory (512 threads, rows of at least kTmemMinVecs vectors).
-template <int THREADS, int UNROLL, bool RECOMPUTE, bool ENT, bool TM = false>
+// memory (512 threads, rows of at least kTmemMinVecs vectors).  SHARED_ROW: `shares`
+// CTAs per row, T x shares of them.
+template <int THREADS, int UNROLL, bool RECOMPUTE, bool ENT, bool TM = false, bool SHARED_ROW = false>
 __global__ void __launch_bounds__(THREADS) loss_grad_cta(
     const acrl_bf16* __restrict__ logits, int64_t T, int V, int64_t ld, const int32_t* __restrict__ ids,
     const uint8_t* __restrict__ mask, const float* __restrict__ lse, const float* __restrict__ old_logp,
     const float* __restrict__ coef, const float* __restrict__ entropy, const float* __restrict__ ent_coef, float eps,
-    acrl_bf16* __restrict__ grad, float* __restrict__ token_loss, int32_t* flags) {
+    acrl_bf16* __restrict__ grad, float* __restrict__ token_loss, int32_t* flags, int shares) {
     __shared__ LseAcc part[2 * (THREADS / 32)];
     __shared__ float part_mx[2 * (THREADS / 32)];
     __shared__ uint32_t tmem_base;
@@ -510,12 +527,21 @@ __global__ void __launch_bounds__(THREADS) loss_grad_cta(
         }
     }
     int par = 0;
-    for (int64_t t = blockIdx.x; t < T; t += gridDim.x) {
+    for (int64_t i = blockIdx.x; i < (SHARED_ROW ? T * shares : T); i += gridDim.x) {
         // a CTA with a further row refills its shared-memory part only once every thread has read the last one
-        if (RECOMPUTE && t != blockIdx.x) __syncthreads();
+        if (RECOMPUTE && i != blockIdx.x) __syncthreads();
+        int64_t t = i;
+        RowShare sh{0, V >> 3};
+        if (SHARED_ROW) {   // few rows: T x shares fits an int
+            t = int(i) / shares;
+            const int share = int(i) - int(t) * shares;
+            const int per = (((V >> 3) + shares - 1) / shares + 7) & ~7;   // shares begin on 128-byte lines of the row
+            sh.begin = min(sh.end, share * per);
+            sh.end = share == shares - 1 ? sh.end : min(sh.end, share * per + per);
+        }
         grad_row<THREADS, UNROLL, RECOMPUTE, ENT, TM>(logits, t, V, ld, ids, mask, lse, old_logp, coef, entropy,
                                                       ent_coef, eps, grad, token_loss, flags, threadIdx.x, part, part_mx,
-                                                      par, kp);
+                                                      par, kp, sh);
     }
     if constexpr (TM) {
         if (kp.tm_chunks > 0) {   // every tensor-memory read has completed (tmem_wait_ld)
@@ -536,7 +562,7 @@ __global__ void __launch_bounds__(THREADS) loss_grad_warp(
     const acrl_bf16* __restrict__ logits, int64_t T, int V, int64_t ld, const int32_t* __restrict__ ids,
     const uint8_t* __restrict__ mask, const float* __restrict__ lse, const float* __restrict__ old_logp,
     const float* __restrict__ coef, const float* __restrict__ entropy, const float* __restrict__ ent_coef, float eps,
-    acrl_bf16* __restrict__ grad, float* __restrict__ token_loss, int32_t* flags) {
+    acrl_bf16* __restrict__ grad, float* __restrict__ token_loss, int32_t* flags, int) {
     constexpr int NW = THREADS / 32;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     int par = 0;
@@ -544,7 +570,7 @@ __global__ void __launch_bounds__(THREADS) loss_grad_warp(
     for (int64_t t = int64_t(blockIdx.x) * NW + wid; t < T; t += int64_t(gridDim.x) * NW)
         grad_row<32, UNROLL, RECOMPUTE, ENT, false>(logits, t, V, ld, ids, mask, lse, old_logp, coef, entropy, ent_coef, eps,
                                              grad, token_loss, flags, lane, nullptr, nullptr, par,
-                                             RowKeep{nullptr, 0, 0u, 0, nullptr});
+                                             RowKeep{nullptr, 0, 0u, 0, nullptr}, RowShare{0, V >> 3});
 }
 
 // Scalar loss: sum of token losses in a fixed order, by one cluster of CTAs
@@ -662,12 +688,12 @@ acrl_status launch_loss_grad(const acrl_bf16* logits, int64_t T, int V, int64_t 
                              const uint8_t* mask, const float* lse, const float* old_logp, const float* coef,
                              const float* entropy, const float* ent_coef, float eps, acrl_bf16* grad,
                              float* token_loss, int32_t* flags, cudaStream_t s) {
-    auto run = [&](auto kernel, int64_t rows_per_cta, int threads, int keep_vecs) {
+    auto run = [&](auto kernel, int64_t rows_per_cta, int threads, int keep_vecs, int shares = 1) {
         const int smem = 16 * min(V >> 3, keep_vecs);
         if (smem > 0 && cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
             return ACRL_ERR_CUDA;
-        return launch(kernel, grid_for(rows_per_cta, T), threads, size_t(smem), 0, s, logits, T, V, ld, ids, mask, lse,
-                      old_logp, coef, entropy, ent_coef, eps, grad, token_loss, flags);
+        return launch(kernel, grid_for(rows_per_cta, T * shares), threads, size_t(smem), 0, s, logits, T, V, ld, ids, mask,
+                      lse, old_logp, coef, entropy, ent_coef, eps, grad, token_loss, flags, shares);
     };
     constexpr int U = kCtaUnroll;
     if constexpr (RECOMPUTE) {
@@ -680,7 +706,12 @@ acrl_status launch_loss_grad(const acrl_bf16* logits, int64_t T, int V, int64_t 
         if (nvec >= kTmemMinVecs) return run(loss_grad_cta<kCtaThreads, U, true, ENT, true>, 1, kCtaThreads, kKeepVecs);
         return run(loss_grad_cta<kCtaThreads, U, true, ENT>, 1, kCtaThreads, kKeepVecs);
     } else {
-        if (V >= kWideRowMinV) return run(loss_grad_cta<kWideThreads, U, false, ENT>, 1, kWideThreads, 0);
+        if (V >= kShareRowMinV) {
+            const int shares = (V >> 3) / kShareVecs;
+            if (T <= kMaxGrid / shares)
+                return run(loss_grad_cta<kShareThreads, U, false, ENT, false, true>, 1, kShareThreads, 0, shares);
+            return run(loss_grad_cta<kWideThreads, U, false, ENT>, 1, kWideThreads, 0);
+        }
         if (V >= 512 * kStreamStep) return run(loss_grad_cta<512, U, false, ENT>, 1, 512, 0);
         if (V >= 384 * kStreamStep) return run(loss_grad_cta<384, U, false, ENT>, 1, 384, 0);
         if (V >= 256 * kStreamStep) return run(loss_grad_cta<256, U, false, ENT>, 1, 256, 0);

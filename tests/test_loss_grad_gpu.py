@@ -14,7 +14,7 @@ DEV = "cuda"
 
 
 @pytest.mark.parametrize("V", [1, 7, 257, 2047, 2048, 2049, 3333, 4095, 4096, 4097, 6145, 8191, 8192, 8193, 12287, 12288, 12289,
-                               16383, 16384, 16385, 20011, 65536, 65537, 100003])
+                               16383, 16384, 16385, 20011, 65536, 65537, 65543, 65544, 81921, 100003, 151936, 200001])
 @pytest.mark.parametrize("bonus", [False, True])
 def test_streaming_gradient_by_row_length(V, bonus):
     _check(V, bonus, recompute=False)

@@ -25,6 +25,7 @@ constexpr int kSeqThreads = 256;
 constexpr int kSeqUnroll = 4;    // tokens per thread in flight
 constexpr int kFinThreads = 512;
 constexpr int kSeqCtas = 304, kSeqTokens = 256;  // see ctas_per_response
+constexpr int kGrpoThreads = 128;
 constexpr int kGrpoTeamPrompts = 1024;  // up to this many prompts are shared by eight lanes each
 constexpr int kFinSeqs = 2048;   // responses whose mean distance the batch kernel keeps in shared memory
 
@@ -258,10 +259,11 @@ __device__ __forceinline__ void write_batch(double s, long long N, int sv, int q
     }
 }
 
-// K2b: prompt statistics and batch statistics; also checks the offsets.
-__global__ void __launch_bounds__(kFinThreads) seq_finalize_kernel(
-    int64_t T, const int64_t* __restrict__ so, int S, const int32_t* __restrict__ goff, int Gn,
-    const acrl_seq_stats* __restrict__ seq, acrl_group_stats* grp, acrl_batch_stats* batch, int32_t* flags) {
+// K2b: prompt statistics and batch statistics; also checks the offsets.  One CTA.
+__device__ __forceinline__ void finalize_seqs(int64_t T, const int64_t* __restrict__ so, int S,
+                                              const int32_t* __restrict__ goff, int Gn,
+                                              const acrl_seq_stats* __restrict__ seq, acrl_group_stats* grp,
+                                              acrl_batch_stats* batch, int32_t* flags) {
     constexpr int NW = kFinThreads / 32;
     __shared__ double sh_D[kFinSeqs];  // D_i, and the valid tokens of response i
     __shared__ int sh_n[kFinSeqs];
@@ -271,7 +273,6 @@ __global__ void __launch_bounds__(kFinThreads) seq_finalize_kernel(
     __shared__ float sh_max[NW];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const bool keep = S <= kFinSeqs;
-    grid_begin();
     bool bad = false;
     long long N = 0;
     int sv = 0;
@@ -356,6 +357,13 @@ __global__ void __launch_bounds__(kFinThreads) seq_finalize_kernel(
     }
 }
 
+__global__ void __launch_bounds__(kFinThreads) seq_finalize_kernel(
+    int64_t T, const int64_t* __restrict__ so, int S, const int32_t* __restrict__ goff, int Gn,
+    const acrl_seq_stats* __restrict__ seq, acrl_group_stats* grp, acrl_batch_stats* batch, int32_t* flags) {
+    grid_begin();
+    finalize_seqs(T, so, S, goff, Gn, seq, grp, batch, flags);
+}
+
 // K3: GRPO advantages.  LANES lanes share a prompt: a thread per prompt ran
 // G dependent loads and G fp64 divisions one after the other (12.2 us for 64
 // prompts of 8; 5.7 us with eight lanes).  LANES = 1 is for batches of so many
@@ -421,6 +429,23 @@ __global__ void grpo_kernel(const float* __restrict__ R, const int32_t* __restri
     grid_begin();
     grpo_prompt<LANES>(int64_t(blockIdx.x) * blockDim.x + threadIdx.x, R, goff, Gn, S, adv_eps, ddof, singleton_rule, adv,
                        flags);
+}
+
+// K2b and K3 at once, for a caller that wants both: CTA 0 finalises, the others
+// make the advantages meanwhile, kGrpoThreads of theirs each (with all 512 the fp64
+// work of 64 prompts on one SM took longer than the launch it saves).  The three
+// calls, 64 / 128 / 256 / 512 responses: 22.7 / 26.1 / 30.5 / 44.5 us with a launch of
+// its own, 19.1 / 22.3 / 28.5 / 42.1 so.
+__global__ void __launch_bounds__(kFinThreads) seq_finalize_grpo_kernel(
+    int64_t T, const int64_t* __restrict__ so, int S, const int32_t* __restrict__ goff, int Gn,
+    const acrl_seq_stats* __restrict__ seq, acrl_group_stats* grp, acrl_batch_stats* batch, const float* __restrict__ R,
+    float adv_eps, int ddof, int singleton_rule, float* __restrict__ adv, int32_t* flags) {
+    grid_begin();
+    if (blockIdx.x == 0)
+        finalize_seqs(T, so, S, goff, Gn, seq, grp, batch, flags);
+    else if (threadIdx.x < kGrpoThreads)
+        grpo_prompt<8>(int64_t(blockIdx.x - 1) * kGrpoThreads + threadIdx.x, R, goff, Gn, S, adv_eps, ddof, singleton_rule,
+                       adv, flags);
 }
 
 __global__ void controller_init_kernel(acrl_controller_state* st, double X_init) {
@@ -1045,6 +1070,15 @@ int ctas_per_response(int32_t S, int64_t T) {
     return c;
 }
 
+acrl_status launch_seq_stats(const float* logp_pi, const float* logp_mu, const uint8_t* mask, int64_t T,
+                             const int64_t* seq_offsets, int32_t S, const int32_t* group_offsets, int32_t Gn,
+                             const float* entropy, float* lr, float* d, acrl_seq_stats* seq, int32_t* flags,
+                             cudaStream_t s) {
+    const int c = ctas_per_response(S, T);
+    return launch(seq_stats_kernel, int64_t(S) * c, kSeqThreads + 32, 0, c, s, logp_pi, logp_mu, mask, T, seq_offsets, S,
+                  group_offsets, Gn, entropy, lr, d, seq, flags);
+}
+
 }  // namespace
 }  // namespace acrl
 
@@ -1060,11 +1094,9 @@ extern "C" acrl_status acrl_seq_discrepancy(const float* logp_pi, const float* l
     if (T > 0 && (!logp_pi || !logp_mu || !lr || !d)) return ACRL_ERR_INVALID_ARG;
     if ((S > 0 && !seq) || (Gn > 0 && !grp)) return ACRL_ERR_INVALID_ARG;
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-    const int c = ctas_per_response(S, T);
     acrl_status st = ACRL_OK;
     if (S > 0)
-        st = launch(seq_stats_kernel, int64_t(S) * c, kSeqThreads + 32, 0, c, s, logp_pi, logp_mu, mask, T, seq_offsets, S,
-                    group_offsets, Gn, entropy, lr, d, seq, dev_flags);
+        st = launch_seq_stats(logp_pi, logp_mu, mask, T, seq_offsets, S, group_offsets, Gn, entropy, lr, d, seq, dev_flags, s);
     if (st != ACRL_OK) return st;
     return launch(seq_finalize_kernel, 1, kFinThreads, 0, 0, s, T, seq_offsets, S, group_offsets, Gn, seq, grp, batch,
                   dev_flags);
@@ -1076,7 +1108,7 @@ extern "C" acrl_status acrl_grpo_advantage(const float* rewards, const int32_t* 
     if (S > 0 && (!rewards || !adv)) return ACRL_ERR_INVALID_ARG;
     if (Gn == 0) return ACRL_OK;
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-    const int threads = 128;
+    const int threads = kGrpoThreads;
     auto run = [&](auto kernel, int lanes) {
         return launch(kernel, (int64_t(Gn) * lanes + threads - 1) / threads, threads, 0, 0, s, rewards, group_offsets, Gn,
                       S, p->adv_eps, p->adv_ddof, p->singleton_rule, adv, dev_flags);
@@ -1145,9 +1177,19 @@ extern "C" acrl_status acrl_importance_weights(acrl_controller_state* state, con
         return launch(weights_cluster_kernel, ctas, kOneThreads, 0, ctas, reinterpret_cast<cudaStream_t>(stream), state, *p,
                       logp_pi, logp_mu, mask, T, rewards, seq_offsets, S, group_offsets, Gn, entropy, lr, d, seq, grp, batch,
                       adv, weight, coef, alpha, ent_coef, nct, dev_flags);
-    acrl_status st = acrl_seq_discrepancy(logp_pi, logp_mu, mask, T, seq_offsets, S, group_offsets, Gn, entropy, lr, d, seq,
-                                          grp, batch, dev_flags, stream);
-    if (st == ACRL_OK) st = acrl_grpo_advantage(rewards, group_offsets, Gn, S, p, adv, dev_flags, stream);
+    acrl_status st;
+    if (S > 0 && Gn > 0 && Gn <= kGrpoTeamPrompts) {
+        cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
+        st = launch_seq_stats(logp_pi, logp_mu, mask, T, seq_offsets, S, group_offsets, Gn, entropy, lr, d, seq, dev_flags, s);
+        if (st == ACRL_OK)
+            st = launch(seq_finalize_grpo_kernel, 1 + (int64_t(Gn) * 8 + kGrpoThreads - 1) / kGrpoThreads, kFinThreads, 0, 0, s, T,
+                        seq_offsets, S, group_offsets, Gn, seq, grp, batch, rewards, p->adv_eps, p->adv_ddof,
+                        p->singleton_rule, adv, dev_flags);
+    } else {
+        st = acrl_seq_discrepancy(logp_pi, logp_mu, mask, T, seq_offsets, S, group_offsets, Gn, entropy, lr, d, seq, grp,
+                                  batch, dev_flags, stream);
+        if (st == ACRL_OK) st = acrl_grpo_advantage(rewards, group_offsets, Gn, S, p, adv, dev_flags, stream);
+    }
     if (st != ACRL_OK) return st;
     return acrl_controller_step(state, p, lr, mask, T, seq_offsets, S, group_offsets, Gn, seq, grp, batch, adv, weight, coef,
                                 alpha, ent_coef, dev_flags, stream);

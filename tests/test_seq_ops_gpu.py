@@ -124,7 +124,9 @@ def _assert_same_bytes(a, b):
 # one part and one prompt; two and four CTAs a response; parts that fill both groups and both passes of eight CTAs;
 # more than a round of tokens a thread; empty responses; the largest counts it takes and the next
 _ONE_SHAPES = [(1, 1, 1, 1), (1, 1, 9000, 9000), (4, 1, 256, 256), (2, 4, 64, 1100), (1, 9, 0, 700), (4, 4, 100, 520),
-               (8, 4, 0, 260), (32, 1, 1, 200), (33, 1, 1, 9), (1, 33, 1, 9), (3, 1, 300, 12000)]
+               (8, 4, 0, 260), (32, 1, 1, 200), (33, 1, 1, 9), (1, 33, 1, 9), (3, 1, 300, 12000),
+               # beyond it: advantages beside the batch statistics, in one, in several and (too many prompts) in no CTAs there
+               (17, 3, 0, 40), (64, 8, 0, 30), (1024, 1, 0, 3), (1025, 1, 0, 3)]
 
 
 @pytest.mark.parametrize("Q,G,lo,hi", _ONE_SHAPES)

@@ -375,10 +375,32 @@ __device__ __forceinline__ RowPlan make_plan(float c, float e, float L, float H,
     return rp;
 }
 
+// The online state without the entropy's sum, and its merge (lse_merge's).
+struct LseSum {
+    float U, s0;
+};
+
+__device__ __forceinline__ LseSum sum_exp_merge(const LseSum& a, const LseSum& b) {
+    const float U = fmaxf(a.U, b.U);
+    const float fa = a.s0 > 0.f ? ex2(a.U - U) : 0.f;
+    const float fb = b.s0 > 0.f ? ex2(b.U - U) : 0.f;
+    return LseSum{U, fa * a.s0 + fb * b.s0};
+}
+
+__device__ __forceinline__ LseSum shfl_xor(const LseSum& a, int m) {
+    return LseSum{__shfl_xor_sync(0xffffffffu, a.U, m), __shfl_xor_sync(0xffffffffu, a.s0, m)};
+}
+
+__device__ __forceinline__ LseSum warp_sum_exp(LseSum a) {
+#pragma unroll
+    for (int m = 16; m >= 1; m >>= 1) a = sum_exp_merge(a, shfl_xor(a, m));
+    return a;
+}
+
 // lse and logp = z_a - lse of a row from its merged state and maximum, in the
 // same form as the statistics kernel (the rounding of max*log2(e) corrected
 // exactly through an FMA).
-__device__ __forceinline__ void lse_logp(const LseAcc& acc, float mx, float za, float& L, float& lp) {
+__device__ __forceinline__ void lse_logp(const LseSum& acc, float mx, float za, float& L, float& lp) {
     const float l2s0 = log2f(acc.s0);
     const float c = fmaf(mx, kLog2e, -acc.U);
     L = fmaf(kLn2, l2s0 - c, mx);
@@ -399,7 +421,7 @@ __device__ __forceinline__ void grad_row(const acrl_bf16* __restrict__ logits, i
                                          const float* __restrict__ lse, const float* __restrict__ old_logp,
                                          const float* __restrict__ coef, const float* __restrict__ entropy,
                                          const float* __restrict__ ent_coef, float eps, acrl_bf16* __restrict__ grad,
-                                         float* __restrict__ token_loss, int32_t* flags, int tid, LseAcc* part,
+                                         float* __restrict__ token_loss, int32_t* flags, int tid, LseSum* part,
                                          float* part_mx, int& par, const RowKeep& kp, const RowShare& sh) {
     const acrl_bf16* row = logits + t * ld;
     acrl_bf16* grow = grad + t * ld;
@@ -423,7 +445,8 @@ __device__ __forceinline__ void grad_row(const acrl_bf16* __restrict__ logits, i
         za = bf16_to_float(row[a]);
         if (RECOMPUTE) {
             float mx;
-            LseAcc acc = warp_lse(recompute_partial<TEAM, UNROLL, TM>(row, V, tid, mx, kp, uint32_t(par), flags));
+            const LseAcc mine = recompute_partial<TEAM, UNROLL, TM>(row, V, tid, mx, kp, uint32_t(par), flags);
+            LseSum acc = warp_sum_exp(LseSum{mine.U, mine.s0});   // the entropy's sum is not wanted: the compiler drops it
             if (TM && kp.tm_chunks > 0)
                 tmem_wait_st();   // before the barrier: the row's tensor-memory part is written
             mx = warp_max(mx);
@@ -434,22 +457,21 @@ __device__ __forceinline__ void grad_row(const acrl_bf16* __restrict__ logits, i
                 constexpr int NW = TEAM / 32;
                 static_assert(!RECOMPUTE || (NW <= 32 && (NW & (NW - 1)) == 0), "warps per team");
                 const int lane = tid & 31;
-                LseAcc* pp = part + par * NW;
+                LseSum* pp = part + par * NW;
                 float* pm = part_mx + par * NW;
                 if (lane == 0) {
                     pp[tid >> 5] = acc;
                     pm[tid >> 5] = mx;
                 }
                 __syncthreads();
-                acc = lane < NW ? pp[lane] : lse_empty();
+                acc = lane < NW ? pp[lane] : LseSum{-INFINITY, 0.f};
                 mx = lane < NW ? pm[lane] : -INFINITY;
 #pragma unroll
                 for (int o = NW / 2; o >= 1; o >>= 1) {
-                    acc = lse_merge(acc, shfl_xor(acc, o));
+                    acc = sum_exp_merge(acc, shfl_xor(acc, o));
                     mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
                 }
-                acc = LseAcc{__shfl_sync(0xffffffffu, acc.U, 0), __shfl_sync(0xffffffffu, acc.s0, 0),
-                             __shfl_sync(0xffffffffu, acc.s1, 0)};
+                acc = LseSum{__shfl_sync(0xffffffffu, acc.U, 0), __shfl_sync(0xffffffffu, acc.s0, 0)};
                 mx = __shfl_sync(0xffffffffu, mx, 0);
                 par ^= 1;
             }
@@ -490,7 +512,7 @@ __global__ void __launch_bounds__(THREADS) loss_grad_cta(
     const uint8_t* __restrict__ mask, const float* __restrict__ lse, const float* __restrict__ old_logp,
     const float* __restrict__ coef, const float* __restrict__ entropy, const float* __restrict__ ent_coef, float eps,
     acrl_bf16* __restrict__ grad, float* __restrict__ token_loss, int32_t* flags, int shares) {
-    __shared__ LseAcc part[2 * (THREADS / 32)];
+    __shared__ LseSum part[2 * (THREADS / 32)];
     __shared__ float part_mx[2 * (THREADS / 32)];
     __shared__ uint32_t tmem_base;
     __shared__ __align__(8) uint64_t keep_bar;

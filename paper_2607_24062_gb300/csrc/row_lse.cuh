@@ -6,6 +6,13 @@
 
 namespace acrl {
 
+// Element-wise maximum of two bf16 pairs (a NaN gives way to a number, as in fmaxf).
+__device__ __forceinline__ uint32_t max_bf16x2(uint32_t a, uint32_t b) {
+    uint32_t r;
+    asm("max.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
+    return r;
+}
+
 // Fold UNROLL 8-element vectors into the thread's running state.
 template <int UNROLL>
 __device__ __forceinline__ void fold_vectors(LseAcc& acc, float& mx, const uint4 (&v)[UNROLL]) {
@@ -17,11 +24,12 @@ __device__ __forceinline__ void fold_vectors(LseAcc& acc, float& mx, const uint4
         f[k][4] = bf16_lo(v[k].z); f[k][5] = bf16_hi(v[k].z);
         f[k][6] = bf16_lo(v[k].w); f[k][7] = bf16_hi(v[k].w);
     }
-    float vm = f[0][0];
+    // the maximum in bf16 pairs: half the instructions of 32-bit maxima, the same value
+    uint32_t pm = max_bf16x2(max_bf16x2(v[0].x, v[0].y), max_bf16x2(v[0].z, v[0].w));
 #pragma unroll
-    for (int k = 0; k < UNROLL; ++k)
-#pragma unroll
-        for (int j = 0; j < 8; ++j) vm = fmaxf(vm, f[k][j]);
+    for (int k = 1; k < UNROLL; ++k)
+        pm = max_bf16x2(pm, max_bf16x2(max_bf16x2(v[k].x, v[k].y), max_bf16x2(v[k].z, v[k].w)));
+    const float vm = fmaxf(bf16_lo(pm), bf16_hi(pm));
     if (vm > mx) {  // new running maximum: rescale the partial sums
         const float Un = vm * kLog2e;
         if (acc.s0 > 0.f) {

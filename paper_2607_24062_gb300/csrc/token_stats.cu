@@ -176,9 +176,10 @@ constexpr int kDepth = 3;
 // Ring or registers?  The line is drawn in 128-thread teams per SM (q: tenths).
 // - Few teams per SM: the ring, up to 2.3 x (above).
 // - 5.2 to 10.4 per SM: all of them fit in one wave of the register path (48
-//   registers), not in one of the ring's (64); V = 151,936, T = 1,216: 59 us in
-//   registers against 64, T = 1,600 (past the wave): 93 against 82.  A warp per
-//   row: only up to 7.5 (V = 16,384, T = 4,096: 25.8 against 26.5).
+//   registers), not in one of the ring's (80); V = 151,936, T = 1,216: 58 us in
+//   registers against 67, T = 1,600 (past the wave): 92 against 77; V = 49,152,
+//   T = 1,000: 17.4 against 22.8; a warp per row, V = 16,384, T = 6,000: 34.1
+//   against 37.9.
 // - Many: the ring for rows of a warp or less (V = 16,384, T = 65,536: 296 us
 //   against 317; V = 8,192: 153 against 162; V = 4,096: 82 against 88), the
 //   same for four warps a row.  Two warps a row: registers where the row's last
@@ -192,7 +193,6 @@ bool use_ring(int64_t T, int team, int V) {
     const int64_t q = T >= (int64_t(1) << 40) ? INT64_MAX : T * team * 10 / (128 * kSms);
     if (team <= 16) return true;
     if (q < 52) return true;
-    if (team == 32) return q > 75;
     if (team == 64) return V >= 28672 ? q > 400 || (q > 104 && q < 140) : q > 104 && q < 140;
     return q > 104;
 }

@@ -5,36 +5,35 @@
 // lse, the sampled token's log-prob and the entropy without reading the logits
 // again.
 //
-// Blackwell path: a persistent kernel of CTA pairs (clusters of one pair, or of
-// two that share loads by multicast; tcgen05 cta_group::2), one CTA per SM,
-// warp-specialised.  A pair computes a 256 x 256 tile of the logits: each CTA
-// stages its own 128 rows of H and its 128-row half of the weight tile, and the
-// MMAs of the even CTA read both CTAs' shared memory and write each CTA's 128
-// accumulator rows into that CTA's TMEM.  Per SM a K slab is 32 KB (A 128 x 64 +
-// B 128 x 64), so six stages fit and the weight half is never staged twice in a
-// pair.
+// Blackwell path: a persistent kernel of CTA pairs (clusters of two CTAs,
+// tcgen05 cta_group::2), one CTA per SM, warp-specialised.  A pair computes a
+// 256 x 256 tile of the logits: each CTA stages its own 128 rows of H and its
+// 128-row half of the weight tile, and the MMAs of the even CTA read both
+// CTAs' shared memory and write each CTA's 128 accumulator rows into that
+// CTA's TMEM.  Per SM a K slab is 32 KB (A 128 x 64 + B 128 x 64), so six
+// stages fit and the weight half is never staged twice in a pair.
 //   warp 0     in each CTA, one thread issues the TMA loads (128B-swizzled)
 //              of the CTA's A and B into a ring of stages, counted on the even
 //              CTA's stage barrier;
 //   warp 1     in the even CTA, one thread issues tcgen05.mma (M=256, N=256,
 //              K=16, kind::f16) into one of two 256-column accumulators and
-//              releases each stage to the producers of the cluster's CTAs, one
-//              commit per CTA;
+//              releases each stage to the producers of both CTAs, one commit
+//              per CTA;
 //   warps 2-5  in each CTA, the epilogue: tcgen05.ld of its accumulator rows
 //              (each thread one row), round to bf16, fold the statistics, and
 //              write the logits through shared memory with TMA bulk tensor
 //              stores (32 x 32 blocks, two staging buffers per warp).
 // Tiles are visited in bands of 32 row tiles (16 pairs) so that the weight
 // tiles in flight are shared through L2 by the pairs working on the same band.
-// Every CTA loads only from this GPU's memory into its cluster's shared memory (the
+// Every CTA loads only from this GPU's memory into its own shared memory (the
 // tensor maps are encoded over pointers that the entry points have checked to
 // be device memory of the current device), and each load fills that CTA's
-// shared memory, or with two pairs also that of the CTA at its place in the other.
+// shared memory alone.
 // Every wait on an mbarrier is bounded in time; on expiry the kernel raises
 // ACRL_FLAG_TIMEOUT, lets the copies it issued land, and exits after freeing
-// its TMEM.  The cluster's CTAs meet at a barrier after initialising their
-// mbarriers and again before any frees its TMEM or exits, so none touches a peer
-// that has gone.
+// its TMEM.  The two CTAs meet at a cluster barrier after initialising their
+// barriers and again before either frees its TMEM or exits, so neither touches
+// a peer that has gone.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
@@ -61,23 +60,14 @@ constexpr int kBBytes = kHalfBN * kBK * 2;
 // boxes of 128 rows and six stages, 195 / 199 / 199 / 203 with the short ring (the
 // weight's bytes take 186).  Rings of 32 rows (10 stages) and 64 rows (8) gain
 // nothing over the full one: 214 us each for 32 rows, 220 against 217 for 48.
-template <int STAGES, int AROWS, int PAIRS = 1>
+template <int STAGES, int AROWS>
 struct Ring {
-    static constexpr int kStages = STAGES, kARows = AROWS, kPairs = PAIRS, kCluster = 2 * PAIRS;
+    static constexpr int kStages = STAGES, kARows = AROWS;
     static constexpr int kABytes = AROWS * kBK * 2;
     static constexpr int kBytes = STAGES * (kABytes + kBBytes);
 };
 using RingFull = Ring<6, kBM>;
 using Ring16 = Ring<11, 16>;
-// Two pairs in a cluster of four, on neighbouring column tiles of the same rows: each
-// pair loads half of the rows into both, so that a CTA takes 24 KB per K slab from L2
-// instead of 32 (a pair's loads at the full MMA rate ask more of L2 than it gives:
-// with half of the MMAs left out 1,003 x 2,048 x 32,001 took 76 us against 95-105).
-// 144 of the 152 SMs fit clusters of four; all the same, with the merge, pairs / fours:
-// 1,003 x 2,048 x 32,001 99.0 / 96.0 us, 600 x 4,096 x 16,000 73.8 / 70.7, 2,048 x
-// 1,024 x 151,936 473 / 464, 4,096 x 4,096 x 151,936 3,113 / 3,045; where the rounds
-// come out unevenly, 768 x 4,096 x 32,000, 137 / 141.
-using RingWide = Ring<6, kBM, 2>;
 constexpr int kMaxStages = 11;
 constexpr int kThreads = 192;
 constexpr uint32_t kTmemCols = 512;
@@ -93,7 +83,7 @@ constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | (uint32_t(kBN >
                             (uint32_t((2 * kBM) >> 4) << 24);
 // Barriers:
 //   full[s]    even CTA: both CTAs' copies of stage s landed
-//   empty[s]   each CTA: the MMAs reading stage s are done (of both pairs, where there are two)
+//   empty[s]   each CTA: the MMAs reading stage s are done
 //   tfull[b]   each CTA: accumulator b is complete
 //   tempty[b]  even CTA: the eight epilogue warps of the pair drained accumulator b
 struct Barriers {
@@ -130,18 +120,6 @@ __device__ __forceinline__ void tma_load_pair(void* dst, const CUtensorMap* map,
         : "memory");
 }
 
-// The same into every CTA of `mask`, at the same place; each copy is counted on
-// the barrier at that place in the even CTA of its destination's pair (`bar` is in
-// an even CTA).
-__device__ __forceinline__ void tma_load_multicast(void* dst, const CUtensorMap* map, uint32_t bar, int x, int y,
-                                                   uint16_t mask) {
-    asm volatile(
-        "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes.multicast::cluster "
-        "[%0], [%1, {%2, %3}], [%4], %5;" ::"r"(smem_u32(dst)),
-        "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(bar), "h"(mask)
-        : "memory");
-}
-
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
@@ -166,14 +144,6 @@ __device__ __forceinline__ void mma_pair(uint32_t tmem_d, uint64_t adesc, uint64
 // thread's MMAs so far have completed.
 __device__ __forceinline__ void mma_commit(uint32_t bar) {
     asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
-}
-
-// The same on the barrier at the place of `bar` (in this CTA) in every CTA of `mask`.
-__device__ __forceinline__ void mma_commit_multicast(uint32_t bar, uint16_t mask) {
-    asm volatile(
-        "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(bar),
-        "h"(mask)
-        : "memory");
 }
 
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
@@ -241,8 +211,7 @@ __device__ void producer(const CUtensorMap* tmA, const CUtensorMap* tmB, uint8_t
                          uint32_t rank, int m_pairs, int n_tiles, int total, int k_iters, int a_bytes, int32_t* flags) {
     constexpr int kStages = R::kStages;
     volatile int32_t* abort = &bars->abort;
-    const int cl = int(blockIdx.x) / R::kCluster, ncl = int(gridDim.x) / R::kCluster;
-    const int pair = int(rank) / 2, side = int(rank) & 1;
+    const int cl = int(blockIdx.x >> 1), ncl = int(gridDim.x >> 1);
     int stage = 0;
     uint32_t phase = 0;
     long issued = 0;
@@ -250,8 +219,7 @@ __device__ void producer(const CUtensorMap* tmA, const CUtensorMap* tmB, uint8_t
     for (int t = cl; t < total && ok; t += ncl) {
         int mp, n;
         tile_coords(t, m_pairs, n_tiles, mp, n);
-        n = n * R::kPairs + pair;
-        const int m = 2 * mp + side;
+        const int m = 2 * mp + int(rank);
         for (int kk = 0; kk < k_iters; ++kk) {
             if (!mbar_try_wait(&bars->empty[stage], phase ^ 1u) &&
                 !wait_phase(&bars->empty[stage], phase ^ 1u, abort)) {
@@ -260,14 +228,10 @@ __device__ void producer(const CUtensorMap* tmA, const CUtensorMap* tmB, uint8_t
                 break;
             }
             // the even CTA's barrier counts both CTAs' bytes of this stage; with a short ring only the even CTA has rows
-            if (side == 0) mbar_expect_tx(&bars->full[stage], 2 * kBBytes + (R::kARows < kBM ? 1 : 2) * a_bytes);
-            const uint32_t full0 = peer_addr(&bars->full[stage], 2 * pair);
-            if constexpr (R::kPairs == 2)   // this pair's half of the rows that both pairs' CTAs of this side need
-                tma_load_multicast(sA + stage * R::kABytes + pair * (R::kABytes / 2), tmA, full0, kk * kBK,
-                                   m * kBM + pair * (kBM / 2), uint16_t(5u << side));
-            else if (R::kARows == kBM || rank == 0)
-                tma_load_pair(sA + stage * R::kABytes, tmA, full0, kk * kBK, m * kBM);
-            tma_load_pair(sB + stage * kBBytes, tmB, full0, kk * kBK, n * kBN + side * kHalfBN);
+            if (rank == 0) mbar_expect_tx(&bars->full[stage], 2 * kBBytes + (R::kARows < kBM ? 1 : 2) * a_bytes);
+            const uint32_t full0 = peer_addr(&bars->full[stage], 0);
+            if (R::kARows == kBM || rank == 0) tma_load_pair(sA + stage * R::kABytes, tmA, full0, kk * kBK, m * kBM);
+            tma_load_pair(sB + stage * kBBytes, tmB, full0, kk * kBK, n * kBN + int(rank) * kHalfBN);
             ++issued;
             if (++stage == kStages) {
                 stage = 0;
@@ -278,7 +242,7 @@ __device__ void producer(const CUtensorMap* tmA, const CUtensorMap* tmB, uint8_t
     if (!ok) {
         // let the copies this thread started land before the CTA can exit: the even CTA waits for its
         // barriers (they count both CTAs' copies), the odd one gives its copies time to land
-        if (side == 0) {
+        if (rank == 0) {
             for (long j = issued - 1; j >= 0 && j >= issued - kStages; --j)
                 wait_phase(&bars->full[j % kStages], uint32_t((j / kStages) & 1), nullptr);
         } else {
@@ -291,11 +255,11 @@ __device__ void producer(const CUtensorMap* tmA, const CUtensorMap* tmB, uint8_t
 
 // The even CTA's MMA thread.
 template <class R>
-__device__ void mma_issuer(uint8_t* sA, uint8_t* sB, Barriers* bars, uint32_t rank, uint32_t tmem, int total,
-                           int k_iters, int32_t* flags) {
+__device__ void mma_issuer(uint8_t* sA, uint8_t* sB, Barriers* bars, uint32_t tmem, int total, int k_iters,
+                           int32_t* flags) {
     constexpr int kStages = R::kStages;
     volatile int32_t* abort = &bars->abort;
-    const int cl = int(blockIdx.x) / R::kCluster, ncl = int(gridDim.x) / R::kCluster;
+    const int cl = int(blockIdx.x >> 1), ncl = int(gridDim.x >> 1);
     // descriptors of stage 0; a descriptor advances by (address offset) / 16
     const uint64_t adesc0 = smem_desc(smem_u32(sA)), bdesc0 = smem_desc(smem_u32(sB));
     int stage = 0;
@@ -323,30 +287,25 @@ __device__ void mma_issuer(uint8_t* sA, uint8_t* sB, Barriers* bars, uint32_t ra
 #pragma unroll
             for (int k16 = 0; k16 < kBK / 16; ++k16)  // 16 columns = 32 bytes = 2 descriptor units
                 mma_pair(d, ad + uint64_t(2 * k16), bd + uint64_t(2 * k16), (kk | k16) != 0);
-            // release the stage to the producers: one commit for each CTA's barrier
-            if constexpr (R::kPairs == 2) {
-                mma_commit_multicast(smem_u32(&bars->empty[stage]), 0xF);
-            } else {
-                mma_commit(peer_addr(&bars->empty[stage], 0));
-                mma_commit(peer_addr(&bars->empty[stage], 1));
-            }
+            // release the stage to both producers: one commit for each CTA's barrier
+            mma_commit(peer_addr(&bars->empty[stage], 0));
+            mma_commit(peer_addr(&bars->empty[stage], 1));
             if (++stage == kStages) {
                 stage = 0;
                 phase ^= 1u;
             }
         }
         if (!ok) break;
-        mma_commit(peer_addr(&bars->tfull[acc], rank));
-        mma_commit(peer_addr(&bars->tfull[acc], rank + 1));
+        mma_commit(peer_addr(&bars->tfull[acc], 0));
+        mma_commit(peer_addr(&bars->tfull[acc], 1));
         acc ^= 1;
         if (acc == 0) acc_phase ^= 1u;
     }
     // every MMA this thread issued has finished before the pair moves on
-    mma_commit(peer_addr(&bars->mma_done, rank));
+    mma_commit(peer_addr(&bars->mma_done, 0));
     wait_phase(&bars->mma_done, 0, nullptr);
 }
 
-template <class R>
 __device__ void epilogue(Barriers* bars, uint32_t tmem, uint32_t rank, const CUtensorMap* tmC, uint8_t* sOut, int M,
                          int N, int m_pairs, int n_tiles, int total, float4* __restrict__ partials, int32_t* flags) {
     volatile int32_t* abort = &bars->abort;
@@ -357,16 +316,14 @@ __device__ void epilogue(Barriers* bars, uint32_t tmem, uint32_t rank, const CUt
     // pieces permuted by the 64-byte swizzle the output tensor map applies
     const uint32_t out0 = smem_u32(sOut + (warp - 2) * 2 * kOutBlockBytes) + uint32_t(lane * 64);
     const uint32_t swz = uint32_t((lane >> 1) & 3);
-    const int cl = int(blockIdx.x) / R::kCluster, ncl = int(gridDim.x) / R::kCluster;
-    const int pair = int(rank) / 2, side = int(rank) & 1;
+    const int cl = int(blockIdx.x >> 1), ncl = int(gridDim.x >> 1);
     int buf = 0;
     int acc = 0;
     uint32_t acc_phase = 0;
     for (int t = cl; t < total; t += ncl) {
         int mp, n;
         tile_coords(t, m_pairs, n_tiles, mp, n);
-        n = n * R::kPairs + pair;
-        const int m = 2 * mp + side;
+        const int m = 2 * mp + int(rank);
         const bool ready = wait_phase(&bars->tfull[acc], acc_phase, abort);
         if (!__all_sync(0xffffffffu, ready)) {
             give_up(abort, flags);
@@ -385,7 +342,7 @@ __device__ void epilogue(Barriers* bars, uint32_t tmem, uint32_t rank, const CUt
             if (c == kBN / 32 - 1) {  // this CTA's rows are read out: tell the even CTA's MMA thread
                 tc_fence_before();
                 __syncwarp();
-                if (lane == 0) remote_arrive(peer_addr(&bars->tempty[acc], 2 * pair));
+                if (lane == 0) remote_arrive(peer_addr(&bars->tempty[acc], 0));
             }
             const int col0 = n * kBN + c * 32;
             if (col0 >= N) continue;  // the same for the whole warp
@@ -414,7 +371,7 @@ __device__ void epilogue(Barriers* bars, uint32_t tmem, uint32_t rank, const CUt
                 tma_store_2d(tmC, sOut + (warp - 2) * 2 * kOutBlockBytes + buf * kOutBlockBytes, col0, row0);
             buf ^= 1;
         }
-        if (row < M && (R::kPairs == 1 || n * kBN < N)) partials[int64_t(n) * M + row] = make_float4(mx, st.U, st.s0, st.s1);
+        if (row < M) partials[int64_t(n) * M + row] = make_float4(mx, st.U, st.s0, st.s1);
         __syncwarp();
         acc ^= 1;
         if (acc == 0) acc_phase ^= 1u;
@@ -424,7 +381,7 @@ __device__ void epilogue(Barriers* bars, uint32_t tmem, uint32_t rank, const CUt
 }
 
 template <class R>
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     lmhead_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                   const __grid_constant__ CUtensorMap tmC, int M, int N, int K, int a_bytes, float4* __restrict__ partials,
                   int32_t* flags) {
@@ -438,14 +395,13 @@ __global__ void __launch_bounds__(kThreads, 1)
     const uint32_t rank = cluster_rank();
     const int m_tiles = (M + kBM - 1) / kBM, n_tiles = (N + kBN - 1) / kBN;
     const int m_pairs = (m_tiles + 1) / 2;
-    const int n_groups = (n_tiles + R::kPairs - 1) / R::kPairs;
-    const int total = m_pairs * n_groups;  // a pair of row tiles x one column tile for each pair of CTAs
+    const int total = m_pairs * n_tiles;  // tiles of 256 x 256 (a pair of row tiles x one column tile)
     const int k_iters = (K + kBK - 1) / kBK;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < R::kStages; ++s) {
             mbar_init(&bars->full[s], 1);
-            mbar_init(&bars->empty[s], R::kPairs);
+            mbar_init(&bars->empty[s], 1);
         }
         for (int b = 0; b < 2; ++b) {
             mbar_init(&bars->tfull[b], 1);
@@ -472,11 +428,11 @@ __global__ void __launch_bounds__(kThreads, 1)
     const uint32_t tmem = bars->tmem_base;
 
     if (warp == 0) {
-        if (lane == 0) producer<R>(&tmA, &tmB, sA, sB, bars, rank, m_pairs, n_groups, total, k_iters, a_bytes, flags);
+        if (lane == 0) producer<R>(&tmA, &tmB, sA, sB, bars, rank, m_pairs, n_tiles, total, k_iters, a_bytes, flags);
     } else if (warp == 1) {
-        if (lane == 0 && (rank & 1) == 0) mma_issuer<R>(sA, sB, bars, rank, tmem, total, k_iters, flags);
+        if (lane == 0 && rank == 0) mma_issuer<R>(sA, sB, bars, tmem, total, k_iters, flags);
     } else {
-        epilogue<R>(bars, tmem, rank, &tmC, sOut, M, N, m_pairs, n_groups, total, partials, flags);
+        epilogue(bars, tmem, rank, &tmC, sOut, M, N, m_pairs, n_tiles, total, partials, flags);
     }
     tc_fence_before();
     __syncthreads();
@@ -586,70 +542,39 @@ bool encode_map(CUtensorMap* map, const void* ptr, uint64_t rows, uint64_t cols,
 // Tensor maps, shared-memory opt-in and the persistent launch (clusters of two
 // CTAs, one CTA per SM, fewer if there are fewer tiles).  Arguments, including
 // where the operands live, are checked by the callers.
-// Tiles (groups of tiles, one for each pair of a cluster) of a problem.
 template <class R>
-int64_t tile_groups(int64_t M, int64_t N) {
-    return (((M + kBM - 1) / kBM + 1) / 2) * ((N + R::kPairs * kBN - 1) / (R::kPairs * kBN));
-}
-
-// Clusters that can be resident at once; 0 where a query fails.
-template <class R>
-int resident_clusters() {
-    constexpr int smem = kSmemBytes<R>;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(R::kCluster * 1024, 1, 1);
-    cfg.blockDim = dim3(kThreads, 1, 1);
-    cfg.dynamicSmemBytes = smem;
-    cudaLaunchAttribute attr;
-    attr.id = cudaLaunchAttributeClusterDimension;
-    attr.val.clusterDim.x = R::kCluster;
-    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
-    int n = 0;
-    if (cudaFuncSetAttribute(lmhead_kernel<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) == cudaSuccess &&
-        cudaOccupancyMaxActiveClusters(&n, lmhead_kernel<R>, &cfg) == cudaSuccess && n > 0)
-        return n;
-    (void)cudaGetLastError();
-    return 0;
-}
-
-template <class R>
-acrl_status launch_ring(int clusters, const acrl_bf16* hidden, int64_t M, int64_t K, int64_t ldh, const acrl_bf16* weight,
-                        int64_t N, int64_t ldw, acrl_bf16* logits, int64_t ldl, float4* partials, int32_t* flags,
-                        cudaStream_t s) {
-    if (clusters < 1) return ACRL_ERR_CUDA;
-    // the short ring's boxes have the tensor's rows, in eights; two pairs load half of their common rows each
-    const int a_rows = R::kARows == kBM ? kBM / R::kPairs : int((M + 7) / 8 * 8);
+acrl_status launch_ring(const acrl_bf16* hidden, int64_t M, int64_t K, int64_t ldh, const acrl_bf16* weight, int64_t N,
+                        int64_t ldw, acrl_bf16* logits, int64_t ldl, float4* partials, int32_t* flags, cudaStream_t s) {
+    // the short ring's boxes have the tensor's rows, in eights
+    const int a_rows = R::kARows == kBM ? kBM : int((M + 7) / 8 * 8);
     CUtensorMap tmA, tmB, tmC;
     if (!encode_map(&tmA, hidden, uint64_t(M), uint64_t(K), uint64_t(ldh), a_rows, kBK, CU_TENSOR_MAP_SWIZZLE_128B) ||
         !encode_map(&tmB, weight, uint64_t(N), uint64_t(K), uint64_t(ldw), kHalfBN, kBK, CU_TENSOR_MAP_SWIZZLE_128B) ||
         !encode_map(&tmC, logits, uint64_t(M), uint64_t(N), uint64_t(ldl), 32, 32, CU_TENSOR_MAP_SWIZZLE_64B))
         return ACRL_ERR_CUDA;
-    const int64_t total = tile_groups<R>(M, N);
-    const int grid = int(R::kCluster * (total < clusters ? total : clusters));
-    return launch(lmhead_kernel<R>, grid, kThreads, kSmemBytes<R>, R::kCluster, s, tmA, tmB, tmC, int(M), int(N), int(K),
-                  a_rows * R::kPairs * kBK * 2, partials, flags);
+    auto* kernel = lmhead_kernel<R>;
+    constexpr int smem = kSmemBytes<R>;
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
+        return ACRL_ERR_CUDA;
+    // 256 x 256 tiles; as many clusters as can be resident at once
+    const int64_t total = (((M + kBM - 1) / kBM + 1) / 2) * ((N + kBN - 1) / kBN);
+    if (total > kMaxGrid / 2) return ACRL_ERR_INVALID_ARG;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(2 * 1024, 1, 1);
+    cfg.blockDim = dim3(kThreads, 1, 1);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    int clusters = 0;
+    if (cudaOccupancyMaxActiveClusters(&clusters, kernel, &cfg) != cudaSuccess || clusters < 1) return ACRL_ERR_CUDA;
+    const int grid = int(2 * (total < clusters ? total : clusters));
+    return launch(kernel, grid, kThreads, smem, 0, s, tmA, tmB, tmC, int(M), int(N), int(K), a_rows * kBK * 2, partials,
+                  flags);
 }
 
 acrl_status launch_lmhead(const acrl_bf16* hidden, int64_t M, int64_t K, int64_t ldh, const acrl_bf16* weight, int64_t N,
                           int64_t ldw, acrl_bf16* logits, int64_t ldl, float4* partials, int32_t* flags, cudaStream_t s) {
-    const int64_t total = tile_groups<RingFull>(M, N);
-    if (total > kMaxGrid / 2) return ACRL_ERR_INVALID_ARG;
-    if (M <= Ring16::kARows)
-        return launch_ring<Ring16>(resident_clusters<Ring16>(), hidden, M, K, ldh, weight, N, ldw, logits, ldl, partials,
-                                   flags, s);
-    // Two pairs per cluster where their rounds of tiles, some 7 % shorter each, end sooner.  Not for problems of one
-    // or two rounds (260 x 1,000 x 10,000: 29 us in pairs, 33 in fours).
-    const int pairs = resident_clusters<RingFull>();
-    const int64_t rounds = pairs > 0 ? (total + pairs - 1) / pairs : 0;
-    if (rounds >= 3) {
-        const int fours = resident_clusters<RingWide>();
-        const int64_t wide_rounds = fours > 0 ? (tile_groups<RingWide>(M, N) + fours - 1) / fours : 0;
-        if (fours > 0 && wide_rounds * 93 < rounds * 100)
-            return launch_ring<RingWide>(fours, hidden, M, K, ldh, weight, N, ldw, logits, ldl, partials, flags, s);
-    }
-    return launch_ring<RingFull>(pairs, hidden, M, K, ldh, weight, N, ldw, logits, ldl, partials, flags, s);
+    auto* run = M <= Ring16::kARows ? launch_ring<Ring16> : launch_ring<RingFull>;
+    return run(hidden, M, K, ldh, weight, N, ldw, logits, ldl, partials, flags, s);
 }
 
 // True when every pointer is device memory of the current device: not managed

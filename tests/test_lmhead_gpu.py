@@ -77,13 +77,6 @@ def test_lmhead_small_shapes(M, N, K):
     assert_close_rel(host(ent), oH, floor=1e-5, what="entropy")
 
 
-# three rounds of tiles and more, which clusters of two pairs may take: an odd number of column tiles, a ragged last
-# row tile and one with a single row, K shorter than the ring and longer, off the slab
-@pytest.mark.parametrize("M,N,K", [(512, 33025, 72), (385, 36864, 136), (257, 38000, 520), (1030, 16100, 200)])
-def test_lmhead_several_rounds(M, N, K):
-    test_lmhead_small_shapes(M, N, K)
-
-
 # the ring for up to 16 rows at its ends, with boxes of one and two eights of rows; more K slabs than stages, so
 # that it wraps, with K on and off the slab
 @pytest.mark.parametrize("M,N,K", [(1, 513, 1000), (8, 700, 1032), (9, 300, 64), (16, 1000, 2048), (17, 513, 1000)])

@@ -41,7 +41,13 @@ constexpr int kCtaThreads = 512, kCtaUnroll = 4;
 // 8,000 x 2,600 21.1 / 19.2; 8,000 x 4,096 27.9 / 24.5; 1,000 x 5,003 11.7 / 8.4;
 // 8,000 x 5,003 38.1 / 30.7; 300 x 8,192 8.8 / 4.6; 30,000 x 8,192 150.8 / 144.7;
 // 8,000 x 10,007 68.3 / 52.1; 20,000 x 14,001 179.4 / 168.5; 600 x 16,384 18.4 /
-// 10.2; 20,000 x 16,384 208 / 189 (a copy of the bytes: 196).
+// 10.2; 20,000 x 16,384 208 / 189 (a copy of the bytes: 196).  With many short rows
+// there is enough in flight whatever the split, and the ragged steps and the CTAs'
+// ends weigh more: from kManyRows rows a warp each up to 4,095 columns (40,000 x
+// 3,333: 88 against 95 with 64 threads; 12,000: 31.7 against 33.4) and 64 threads up
+// to 8,191 (40,000 x 7,000: 169 against 177 with 128; 20,000 x 5,003: 66.7 against
+// 68.2).
+constexpr int64_t kManyRows = 12000;
 constexpr int kStreamStep = 8 * kCtaUnroll;   // columns of one thread's step
 // Rows of more than 65,536 columns are split between CTAs of 256 threads, two whole
 // steps and a little more for each (nine for 151,936 columns): more of the row is in
@@ -737,8 +743,9 @@ acrl_status launch_loss_grad(const acrl_bf16* logits, int64_t T, int V, int64_t 
         if (V >= 512 * kStreamStep) return run(loss_grad_cta<512, U, false, ENT>, 1, 512, 0);
         if (V >= 384 * kStreamStep) return run(loss_grad_cta<384, U, false, ENT>, 1, 384, 0);
         if (V >= 256 * kStreamStep) return run(loss_grad_cta<256, U, false, ENT>, 1, 256, 0);
-        if (V >= 128 * kStreamStep) return run(loss_grad_cta<128, U, false, ENT>, 1, 128, 0);
-        if (V >= 64 * kStreamStep) return run(loss_grad_cta<64, U, false, ENT>, 1, 64, 0);
+        const bool many = T >= kManyRows;
+        if (V >= 128 * kStreamStep && !many) return run(loss_grad_cta<128, U, false, ENT>, 1, 128, 0);
+        if (V >= (many ? 128 : 64) * kStreamStep) return run(loss_grad_cta<64, U, false, ENT>, 1, 64, 0);
         return run(loss_grad_warp<64, U, false, ENT>, 2, 64, 0);
     }
 }

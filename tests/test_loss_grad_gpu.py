@@ -20,6 +20,21 @@ def test_streaming_gradient_by_row_length(V, bonus):
     _check(V, bonus, recompute=False)
 
 
+@pytest.mark.parametrize("V", [2049, 4095, 4096, 8191])
+def test_many_short_rows_agree_with_few(V):
+    """The split of a row between threads does not show in its gradient."""
+    gen = torch.Generator(device=DEV).manual_seed(V)
+    T, few, ld = 12001, 5, (V + 7) // 8 * 8
+    x = torch.randn((T, ld), generator=gen, device=DEV).to(torch.bfloat16)
+    ids = torch.randint(0, V, (T,), generator=gen, device=DEV, dtype=torch.int32)
+    coef = torch.randn(T, generator=gen, device=DEV)
+    lse = x[:, :V].float().logsumexp(dim=1)
+    a, tl, _ = api.loss_grad_logits(x, ids, None, lse, None, coef, 0.2, V=V)
+    b, tl2, _ = api.loss_grad_logits(x[-few:], ids[-few:], None, lse[-few:], None, coef[-few:], 0.2, V=V)
+    assert torch.equal(a[-few:, :V].view(torch.int16), b[:, :V].view(torch.int16))
+    assert torch.equal(tl[-few:], tl2)
+
+
 @pytest.mark.parametrize("V", [1, 7, 1025, 4095, 4096, 4097, 7168, 7169, 10240, 10243, 20480, 20487, 20488, 24007, 36864, 40001,
                                40967, 40968, 49155, 61003, 65535, 65536, 70001])
 @pytest.mark.parametrize("bonus", [False, True])

@@ -99,7 +99,7 @@ class AcrlStep:
 
     def run(self, logits, ids, mask, logp_mu, rewards, seq_offsets, group_offsets, stream=None, exchange=None,
             **grad_kw):
-        if exchange is None and not grad_kw and self._whole(logits, seq_offsets, group_offsets):
+        if exchange is None and not grad_kw and self._whole(logits, rewards, seq_offsets, group_offsets):
             api.step(self.state, self.params, logits, ids, mask, logp_mu, rewards, seq_offsets, group_offsets, V=self.V,
                      lse=self.lse, logp=self.logp, entropy=self.entropy, out=self.disc, adv=self.adv,
                      weight=self.weight, coef=self.coef, alpha=self.alpha, ent_coef=self.ent_coef, grad=self.grad,
@@ -109,11 +109,12 @@ class AcrlStep:
                         exchange=exchange)
         self.gradient(logits, ids, mask, stream=stream, **grad_kw)
 
-    def _whole(self, logits, seq_offsets, group_offsets) -> bool:
+    def _whole(self, logits, rewards, seq_offsets, group_offsets) -> bool:
         """The batch is the one this object was built for, and its two halves are the ones below: one call does both."""
         cls = type(self)
         return (logits.shape[0] == self.T == self.logp.numel() and seq_offsets.numel() == self.S + 1 and
-                group_offsets.numel() == self.Gn + 1 and self.disc.S == self.S and self.disc.Gn == self.Gn and
+                group_offsets.numel() == self.Gn + 1 and rewards.numel() == self.S and self.disc.S == self.S and
+                self.disc.Gn == self.Gn and
                 cls.statistics is AcrlStep.statistics and cls.gradient is AcrlStep.gradient)
 
     @classmethod

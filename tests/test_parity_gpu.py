@@ -838,3 +838,19 @@ def test_autograd_backward_of_the_backward():
     ref = (step.grad[:, :b.V].float() * v.float()).sum()
     # bf16 rounding of the products' sum on torch's side: 2^-8 of the terms' magnitude
     assert abs(float(ds - ref)) <= 2.0 ** -8 * float((step.grad[:, :b.V].float() * v.float()).abs().sum())
+
+
+def test_one_call_refuses_what_the_calls_refuse():
+    """A batch that is not the step's goes through the separate calls and their checks."""
+    spec = W.small_variant(W.GRPO, name="refuse", n_prompts=2, group_size=2, len_lo=5, len_hi=20, V=1003)
+    b = _gen(spec, seed=4)
+    step = acrl.AcrlStep.for_batch(b, acrl.Params())
+    args = [b.logits, b.ids, b.mask, b.logp_mu, b.rewards, b.seq_offsets, b.group_offsets]
+    longer = torch.cat([b.rewards, b.rewards[:1]])
+    for i, bad in ((4, longer), (4, b.rewards.double()), (1, b.ids.long()), (3, b.logp_mu[:-1]), (5, b.seq_offsets.int()),
+                   (0, b.logits.float())):
+        with pytest.raises(acrl.AcrlError):
+            step.run(*(args[:i] + [bad] + args[i + 1:]))
+    step.reset_controller()
+    step.run(*args)
+    assert acrl.read_flags(step.flags) == 0

@@ -155,3 +155,28 @@ def test_one_call_on_uneven_prompts_and_bad_offsets():
     for args in ((pi, so, uneven), (pi, so, broken_go), (pi, broken_so, go), (nan, so, go)):
         a, b = _three_calls_and_one(p, 2, args[0], mu, mask, args[1], args[2], R, H, False)
         _assert_same_bytes(a, b)
+
+
+def test_fp64_quotients_and_roots_are_rounded_ones():
+    """The kernels' own fp64 quotient and square root (Newton-Raphson with a final residual) against IEEE division and
+    root: one ulp on D_i = sum_d / n as it comes out as Y of a prompt with one response, for many n and magnitudes; on
+    the token means; and on the standard deviation, whose argument is a difference of two of them."""
+    S = 1500
+    rng = np.random.default_rng(3)
+    n = rng.integers(1, 700, size=S)
+    so = np.concatenate([[0], np.cumsum(n)])
+    T = int(so[-1])
+    pi = (-rng.exponential(size=T) * np.repeat(10.0 ** rng.uniform(-6, 1.2, size=S), n)).astype(np.float32)
+    mu = np.minimum(pi + (0.3 * rng.normal(size=T)).astype(np.float32), 0.0)
+    f = lambda x, dt: torch.tensor(np.asarray(x), dtype=dt, device=DEV)  # noqa: E731
+    disc = api.seq_discrepancy(f(pi, torch.float32), f(mu, torch.float32), None, f(so, torch.int64),
+                               f(np.arange(S + 1), torch.int32))
+    seq, grp, b = disc.seq_host(), disc.grp_host(), disc.batch_host()
+    want = seq["sum_d"] / n
+    assert np.all(seq["n"] == n) and np.all(np.abs(grp["Y"] - want) <= 2.0 ** -52 * want)
+    assert float(seq["sum_d"].max() / seq["sum_d"].min()) > 1e3
+    # a mean is sum * (1 / N): two roundings, and the sums' own order
+    for got, v in ((b["d_mean"], seq["sum_d"]), (b["lr_mean"], seq["sum_lr"])):
+        assert abs(float(got) - float(v.sum()) / T) <= 1e-14 * float(np.abs(v).sum()) / T
+    var = float(seq["sum_d2"].sum()) / T - (float(seq["sum_d"].sum()) / T) ** 2
+    assert abs(float(b["d_std"]) - np.sqrt(var)) <= 1e-13 * float(seq["sum_d2"].sum()) / T / np.sqrt(var)

@@ -530,7 +530,8 @@ def check_flags(flags, stream=None) -> None:
 
 
 __all__ = ["Params", "AcrlError", "token_stats", "seq_discrepancy", "grpo_advantage", "controller_init",
-           "controller_step", "loss_grad_logits", "reduce_loss", "scale_grad", "read_flags", "check_flags", "read_state", "Discrepancy",
+           "controller_step", "importance_weights", "step", "loss_grad_logits", "reduce_loss", "scale_grad",
+           "read_flags", "check_flags", "read_state", "Discrepancy",
            "lmhead_logits_stats", "lmhead_merge", "lmhead_workspace_bytes", "lmhead_stats_noalloc", "save_state",
            "load_state", "controller_save", "controller_load", "selftest_wait_timeout",
            "host_pipeline_workspace_bytes", "host_pipeline_create", "host_pipeline_step", "host_pipeline_begin",

@@ -25,13 +25,13 @@ inline acrl_status launch_status() {
     return cudaGetLastError() == cudaSuccess ? ACRL_OK : ACRL_ERR_CUDA;
 }
 
-// Every kernel of the path is launched here, with programmatic dependent launch: it may
-// start while the previous kernel of the stream is still running, and every
-// kernel therefore begins with grid_begin(), which lets the next one start and
-// then waits until everything before it has completed.  That hides most of the
-// launch latency between the path's short kernels; against a predecessor that
-// is no kernel of this library it is an ordinary launch.  `cluster` CTAs form a
-// cluster (0: as the kernel declares).  An error is cleared as launch_status does.
+// Every kernel of the path is launched here, with programmatic dependent launch: it
+// may be placed while the previous kernel of the stream is still running, and every
+// kernel therefore begins with grid_begin(), which waits until everything before it
+// has completed and then lets the next one be placed.  That hides most of the launch
+// latency between the path's short kernels; against a predecessor that is no kernel
+// of this library it is an ordinary launch.  `cluster` CTAs form a cluster (0: as the
+// kernel declares).  An error is cleared as launch_status does.
 template <typename... P, typename... A>
 acrl_status launch(void (*kernel)(P...), int64_t grid, int threads, size_t smem, int cluster, cudaStream_t s,
                    const A&... args) {

@@ -1180,10 +1180,11 @@ extern "C" acrl_status acrl_importance_weights(acrl_controller_state* state, con
     acrl_status st;
     if (S > 0 && Gn > 0 && Gn <= kGrpoTeamPrompts) {
         cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-        st = launch_seq_stats(logp_pi, logp_mu, mask, T, seq_offsets, S, group_offsets, Gn, entropy, lr, d, seq, dev_flags, s);
+        st = launch_seq_stats(logp_pi, logp_mu, mask, T, seq_offsets, S, group_offsets, Gn, entropy, lr, d, seq, dev_flags,
+                              s);
         if (st == ACRL_OK)
-            st = launch(seq_finalize_grpo_kernel, 1 + (int64_t(Gn) * 8 + kGrpoThreads - 1) / kGrpoThreads, kFinThreads, 0, 0, s, T,
-                        seq_offsets, S, group_offsets, Gn, seq, grp, batch, rewards, p->adv_eps, p->adv_ddof,
+            st = launch(seq_finalize_grpo_kernel, 1 + (int64_t(Gn) * 8 + kGrpoThreads - 1) / kGrpoThreads, kFinThreads, 0,
+                        0, s, T, seq_offsets, S, group_offsets, Gn, seq, grp, batch, rewards, p->adv_eps, p->adv_ddof,
                         p->singleton_rule, adv, dev_flags);
     } else {
         st = acrl_seq_discrepancy(logp_pi, logp_mu, mask, T, seq_offsets, S, group_offsets, Gn, entropy, lr, d, seq, grp,

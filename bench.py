@@ -45,8 +45,8 @@ LMHEAD_METRIC = "tokens/s fused LM-head projection + logprob + discrepancy + gra
 UNIT = "tokens/s"
 FALLBACK_HBM_GBS = 6800.0
 # Kernel launches per step inside the timed region: token_stats 1, seq_discrepancy 2,
-# grpo_advantage 1, controller_step 2, loss_grad_logits 2.
-LAUNCHES_PER_STEP = 8
+# grpo_advantage 1, controller_step 3, loss_grad_logits 2.
+LAUNCHES_PER_STEP = 9
 # DRAM traffic of one launch of each kernel (dram__bytes_read.sum + dram__bytes_write.sum
 # from ncu, one pass), captured on a small case of its workload and scaled to a full
 # launch by the algorithmic bytes (or, for the GEMM, the flops) of each: the streaming
@@ -720,7 +720,7 @@ def lmhead_measure(workload, dev, steps, warmup):
                  "traffic_source": TRAFFIC_SOURCE},
         "merge_ms": merge_ms, "seq_discrepancy+grpo_advantage+controller_step_ms": ot_ms,
         "loss_grad_logits": {"ms": grad_ms, "GB/s": 4.0 * M * N / (grad_ms / 1e3) / 1e9},
-        "clocks": clocks.summary(), "gpu_launches": 9 * steps,
+        "clocks": clocks.summary(), "gpu_launches": 10 * steps,
     }
     return summary, b, p
 

@@ -27,7 +27,7 @@ def test_bench_line_has_the_contract_keys():
               "vs_baseline", "dtype", "data", "config", "roofline", "clocks", "gpu_launches", "e2e", "cpu_baseline"):
         assert k in out, k
     assert out["n_gpus"] == 1 and out["steps"] == 3 and out["warmup"] == 3 and out["higher_is_better"] is True
-    assert out["value"] > 0 and out["gpu_launches"] == 8 * 3
+    assert out["value"] > 0 and out["gpu_launches"] == 9 * 3
     rf = out["roofline"]
     assert rf["bound"] == "hbm" and rf["unit"] == "GB/s" and rf["peak"] > 0
     assert rf["frac"] == pytest.approx(rf["achieved"] / rf["peak"])

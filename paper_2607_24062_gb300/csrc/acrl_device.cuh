@@ -249,7 +249,10 @@ __device__ __forceinline__ uint32_t cluster_rank() {
     return r;
 }
 
+// All threads of the cluster's CTAs.  The barrier is the .aligned form, which a warp
+// executes as one: a caller may come from a block that one lane took.
 __device__ __forceinline__ void cluster_sync() {
+    __syncwarp();
     asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 

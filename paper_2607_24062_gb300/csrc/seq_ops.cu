@@ -906,7 +906,6 @@ __global__ void __launch_bounds__(kOneThreads) weights_cluster_kernel(
         state = *st;
         inv_X = recip64(state.X);
     }
-    __syncwarp();
     cluster_sync();  // every CTA's parts are in its shared memory, the advantages written
 
     // sums over the parts of this lane's response, in their order
@@ -989,7 +988,6 @@ __global__ void __launch_bounds__(kOneThreads) weights_cluster_kernel(
             s4 = warp_sum4(total(&part[0].sum[0]), total(&part[0].sum[1]), total(&part[0].sum[3]), total(&part[0].sum[2]));
         }
     }
-    __syncwarp();
     cluster_sync();  // the responses' scalars are in CTA 0's shared memory
 
     acrl_seq_stats o;
@@ -1085,7 +1083,6 @@ __global__ void __launch_bounds__(kOneThreads) weights_cluster_kernel(
             write_state(state, mv, mv.x_den > 0.0 ? div64(mv.x_num, mv.x_den) : 0.0, qv > 0 ? div64(Ysum, qv) : 0.0,
                         sv > 0 ? div64(sa, sv) : 0.0, p, st, batch, flags);
     }
-    __syncwarp();
     cluster_sync();  // every CTA's weight sums are in its shared memory, the other batch fields written
 
     if (role == kSums) {
@@ -1099,7 +1096,6 @@ __global__ void __launch_bounds__(kOneThreads) weights_cluster_kernel(
             batch->trunc_frac = N > 0 ? quot64(double(nt), double(N), inv_N) : 0.0;
         }
     }
-    __syncwarp();
     cluster_sync();  // no CTA leaves while CTA 0 may still read its shared memory
 }
 

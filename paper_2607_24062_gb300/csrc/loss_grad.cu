@@ -718,7 +718,9 @@ acrl_status launch_loss_grad(const acrl_bf16* logits, int64_t T, int V, int64_t 
                              float* token_loss, int32_t* flags, cudaStream_t s) {
     auto run = [&](auto kernel, int64_t rows_per_cta, int threads, int keep_vecs, int shares = 1) {
         const int smem = 16 * min(V >> 3, keep_vecs);
-        if (smem > 0 && cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
+        // the limit belongs to the kernel, not to the call: always its largest, so that threads with different V agree
+        if (keep_vecs > 0 &&
+            cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 16 * keep_vecs) != cudaSuccess)
             return ACRL_ERR_CUDA;
         return launch(kernel, grid_for(rows_per_cta, T * shares), threads, size_t(smem), 0, s, logits, T, V, ld, ids, mask,
                       lse, old_logp, coef, entropy, ent_coef, eps, grad, token_loss, flags, shares);

@@ -3,12 +3,15 @@ given and recomputed: rows one column short of, at and past the lines, rows
 shorter than a step, with one to seven columns beyond whole vectors and with a
 ragged rest beyond what the CTA keeps on chip, against float64."""
 
+import ctypes
+import threading
+
 import pytest
 import torch
 
 pytestmark = pytest.mark.gpu
 
-from paper_2607_24062_gb300 import api  # noqa: E402
+from paper_2607_24062_gb300 import _abi, api  # noqa: E402
 
 DEV = "cuda"
 
@@ -76,3 +79,38 @@ def _check(V, bonus, recompute):
     assert bool(((tl.double() - want_tl).abs() <= 2.0 ** -22 * (c.abs() + (e.double() * H if bonus else 0.0)) + 1e-30).all())
     whole = tl.double().sum()
     assert abs(float(loss) - float(whole)) <= 2.0 ** -21 * float(tl.double().abs().sum()) + 1e-30
+
+
+@pytest.mark.parametrize("short,long", [(41000, 65000), (20488, 36864), (7200, 20480), (4096, 7168), (70000, 151936)])
+def test_threads_with_rows_of_one_class(short, long):
+    """Two host threads whose rows take the same kernel with different amounts of shared memory: neither's call fails
+    for what the other sets in between."""
+    fn = _abi.lib().acrl_loss_grad_logits
+    start, bad = threading.Barrier(2), []
+
+    def work(V):
+        T, ld = 2, (V + 7) // 8 * 8
+        stream = torch.cuda.Stream()
+        with torch.cuda.stream(stream):
+            x = torch.randn((T, ld), device=DEV).to(torch.bfloat16)
+            ids = torch.zeros(T, dtype=torch.int32, device=DEV)
+            coef, tl, loss, flags = torch.ones(T, device=DEV), torch.empty(T, device=DEV), torch.empty(1, device=DEV), api.new_flags()
+            grad = torch.empty_like(x)
+        p = lambda t: ctypes.c_void_p(t.data_ptr())  # noqa: E731
+        args = (p(x), T, V, ld, p(ids), None, None, None, p(coef), None, None, 0.2, p(grad), p(tl), p(loss), p(flags),
+                ctypes.c_void_p(stream.cuda_stream))
+        start.wait()
+        for _ in range(4000):
+            st = fn(*args)
+            if st != 0:
+                bad.append((V, st))
+        stream.synchronize()
+        if api.read_flags(flags) != 0 or not bool(torch.isfinite(grad[:, :V]).all()):
+            bad.append((V, "result"))
+
+    threads = [threading.Thread(target=work, args=(V,)) for V in (short, long)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not bad, (len(bad), bad[:4])

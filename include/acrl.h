@@ -415,9 +415,10 @@ acrl_status acrl_reduce_loss(const float* token_loss, int64_t T, float* loss, ac
  * *scale is exactly 1 nothing is written: the caller uses `grad` as it is.
  *   grad   device bf16 [T, ld], as acrl_loss_grad_logits writes it.
  *   scale  device float [1].
- *   out    device bf16 [T, ldo] output, no overlap with grad; ldo >= V, a
- *          multiple of 8.  The columns from V up to the next multiple of 8 are
- *          written too (scaled like the rest, from grad's).
+ *   out    device bf16 [T, ldo] output, no overlap with grad; ldo is V (rows
+ *          without a gap) or a larger multiple of 8, with which the columns from V
+ *          up to the next multiple of 8 are written too (scaled like the rest,
+ *          from grad's).
  */
 acrl_status acrl_scale_grad(const acrl_bf16* grad, int64_t T, int64_t V, int64_t ld, const float* scale,
                             acrl_bf16* out, int64_t ldo, acrl_stream stream);

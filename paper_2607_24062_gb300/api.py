@@ -336,8 +336,9 @@ def reduce_loss(token_loss, *, loss=None, stream=None):
 
 
 def scale_grad(grad, scale, *, V=None, out=None, stream=None):
-    """acrl_scale_grad: grad (bf16 [T, ld]) times the float32 scalar on the device.  Returns bf16 [T, ldo], ldo = V
-    rounded up to a multiple of eight; its contents are undefined where the scalar is exactly 1."""
+    """acrl_scale_grad: grad (bf16 [T, ld]) times the float32 scalar on the device.  Returns `out` (row stride V, or a
+    multiple of eight), by default bf16 [T, ldo] with V rounded up to a multiple of eight; its contents are undefined
+    where the scalar is exactly 1."""
     T, ld = _rows(grad, "grad")
     V = grad.shape[1] if V is None else V
     if V > ld:

@@ -6,8 +6,8 @@
 The forward runs the whole pass of `AcrlStep` (statistics, discrepancy,
 advantages, controller, then the gradient kernel, which writes dL/dlogits in
 bf16 while it computes the loss), so the backward needs no second pass over
-the logits: it hands back that buffer, or a copy scaled by the incoming
-gradient when that is not 1.  The gradient is the one of Eq. ACRL on the on-policy step
+the logits: it hands back that buffer, or a contiguous copy scaled by the
+incoming gradient when that is not 1.  The gradient is the one of Eq. ACRL on the on-policy step
 (theta = theta_old, so r = 1), with the importance weights treated as
 constants, as the paper's rho is built from theta_old.
 
@@ -40,7 +40,7 @@ class _AcrlLoss(torch.autograd.Function):
             if torch.is_grad_enabled() or grad_out.dtype != torch.float32 or grad_out.device != g.device:
                 g = g * grad_out.to(g.dtype)  # a graph of the backward itself, or no scalar the kernel reads
             else:
-                g = api.scale_grad(g, grad_out)[:, : ctx.cols]
+                g = api.scale_grad(g, grad_out, out=torch.empty(g.shape, dtype=g.dtype, device=g.device))
         return g, None, None, None, None, None, None, None, None
 
 

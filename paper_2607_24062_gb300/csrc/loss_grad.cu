@@ -711,6 +711,77 @@ __global__ void __launch_bounds__(kScaleThreads)
     }
 }
 
+// Elements m .. m + 7 of the 16 in (lo, hi), m < 8.
+__device__ __forceinline__ uint4 shift_elems(const uint4& lo, const uint4& hi, int m) {
+    const uint32_t w[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
+    uint32_t y[6], z[5];
+#pragma unroll
+    for (int i = 0; i < 6; ++i) y[i] = m & 4 ? w[i + 2] : w[i];
+#pragma unroll
+    for (int i = 0; i < 5; ++i) z[i] = m & 2 ? y[i + 1] : y[i];
+    const int half = (m & 1) * 16;
+    return make_uint4(__funnelshift_r(z[0], z[1], half), __funnelshift_r(z[1], z[2], half),
+                      __funnelshift_r(z[2], z[3], half), __funnelshift_r(z[3], z[4], half));
+}
+
+// The same product into rows without a gap whose length is no multiple of eight (the
+// contiguous [T, V] tensor that a framework's own product is).  A thread takes
+// kScaleUnroll 16-byte vectors of the output as it lies in memory; one inside a row
+// comes from two neighbouring vectors of `grad`, shifted by the columns that the row
+// starts off a vector (the second is the next lane's first, from L1); one that holds a
+// row's end, or the end of the output, goes element by element.
+__global__ void __launch_bounds__(kScaleThreads)
+    scale_grad_dense_kernel(const acrl_bf16* __restrict__ grad, int64_t T, int V, int64_t ld,
+                            const float* __restrict__ scale, acrl_bf16* __restrict__ out) {
+    grid_begin();
+    const float f = *scale;
+    if (f == 1.f) return;  // the caller keeps `grad`
+    const float s = bf16_lo(pack_bf16x2(f, 0.f));
+    const int64_t total = T * V, nvec = (total + 7) >> 3, step = int64_t(gridDim.x) * kScaleThreads * kScaleUnroll;
+    constexpr int kApart = 8 * kScaleThreads;   // elements between two vectors of a thread
+    for (int64_t i = int64_t(blockIdx.x) * kScaleThreads * kScaleUnroll + threadIdx.x; i < nvec; i += step) {
+        int64_t row = i * 8 / V;
+        int col = int(i * 8 - row * V);
+        uint4 lo[kScaleUnroll], hi[kScaleUnroll];
+        int64_t at_row[kScaleUnroll];
+        int at_col[kScaleUnroll];
+#pragma unroll
+        for (int k = 0; k < kScaleUnroll; ++k) {
+            at_row[k] = row;
+            at_col[k] = col;
+            if (row < T && col + 8 <= V) {
+                const uint4* src = reinterpret_cast<const uint4*>(grad + row * ld) + (col >> 3);
+                lo[k] = __ldg(src);
+                hi[k] = col & 7 ? __ldg(src + 1) : lo[k];   // holds column col + 7 at the latest
+            }
+            col += kApart;
+            const int rows = col < V ? 0 : V >= kApart ? 1 : col / V;
+            row += rows;
+            col -= rows * V;
+        }
+#pragma unroll
+        for (int k = 0; k < kScaleUnroll; ++k) {
+            const int64_t v = i + k * kScaleThreads;
+            if (at_row[k] < T && at_col[k] + 8 <= V) {
+                const uint4 x = shift_elems(lo[k], hi[k], at_col[k] & 7);
+                st_stream(reinterpret_cast<uint4*>(out) + v,
+                          make_uint4(scale_pair(x.x, s), scale_pair(x.y, s), scale_pair(x.z, s), scale_pair(x.w, s)));
+            } else if (v < nvec) {
+                int64_t r = at_row[k];
+                int c = at_col[k];
+#pragma unroll 1
+                for (int64_t j = v * 8; j < min(total, v * 8 + 8); ++j) {
+                    out[j] = acrl_bf16(scale_pair(grad[r * ld + c], s) & 0xffffu);
+                    if (++c == V) {
+                        c = 0;
+                        ++r;
+                    }
+                }
+            }
+        }
+    }
+}
+
 template <bool RECOMPUTE, bool ENT>
 acrl_status launch_loss_grad(const acrl_bf16* logits, int64_t T, int V, int64_t ld, const int32_t* ids,
                              const uint8_t* mask, const float* lse, const float* old_logp, const float* coef,
@@ -797,7 +868,7 @@ extern "C" acrl_status acrl_reduce_loss(const float* token_loss, int64_t T, floa
 
 extern "C" acrl_status acrl_scale_grad(const acrl_bf16* grad, int64_t T, int64_t V, int64_t ld, const float* scale,
                                        acrl_bf16* out, int64_t ldo, acrl_stream stream) {
-    if (T < 0 || V < 1 || V > kMaxVocab || ld < V || (ld & 7) != 0 || ldo < V || (ldo & 7) != 0)
+    if (T < 0 || V < 1 || V > kMaxVocab || ld < V || (ld & 7) != 0 || ldo < V || (ldo != V && (ldo & 7) != 0))
         return ACRL_ERR_INVALID_ARG;
     if (T == 0) return ACRL_OK;
     if (!grad || !scale || !out || !aligned16(grad) || !aligned16(out)) return ACRL_ERR_INVALID_ARG;
@@ -805,6 +876,9 @@ extern "C" acrl_status acrl_scale_grad(const acrl_bf16* grad, int64_t T, int64_t
     // at most kMaxGrid CTAs: the kernel loops
     const int64_t per_cta = kScaleThreads * kScaleUnroll;
     const int64_t rows = T < kMaxGrid ? T : kMaxGrid;
+    if ((ldo & 7) != 0)
+        return launch(scale_grad_dense_kernel, grid_for(per_cta, rows * nvec), kScaleThreads, 0, 0,
+                      reinterpret_cast<cudaStream_t>(stream), grad, T, int(V), ld, scale, out);
     return launch(scale_grad_kernel, grid_for(per_cta, rows * nvec), kScaleThreads, 0, 0,
                   reinterpret_cast<cudaStream_t>(stream), grad, T, nvec, ld, scale, out, ldo);
 }

@@ -11,6 +11,8 @@ import torch
 
 pytestmark = pytest.mark.gpu
 
+import paper_2607_24062_gb300 as acrl  # noqa: E402
+import workloads as W  # noqa: E402
 from paper_2607_24062_gb300 import _abi, api  # noqa: E402
 
 DEV = "cuda"
@@ -114,3 +116,40 @@ def test_threads_with_rows_of_one_class(short, long):
     for t in threads:
         t.join()
     assert not bad, (len(bad), bad[:4])
+
+
+# vectors of the output that hold one row's end, several rows, the output's end; rows shorter and longer than the
+# 2,048 columns between two vectors of a thread; every shift of a row against its vectors
+@pytest.mark.parametrize("T,V,ld", [(1, 1, 8), (1, 3, 8), (9, 1, 8), (300, 7, 8), (5, 9, 16), (131, 15, 24), (40, 2047, 2048),
+                                    (17, 2049, 2056), (3, 6143, 6144), (1, 4099, 4104), (131, 20011, 20016), (9, 100003, 100008)])
+def test_scaled_gradient_without_gaps(T, V, ld):
+    """acrl_scale_grad into rows of V columns against torch's bf16 product, bit for bit, with nothing written beyond."""
+    gen = torch.Generator(device=DEV).manual_seed(T + V)
+    g = torch.full((T, ld), float("nan"), dtype=torch.bfloat16, device=DEV)   # columns past V are never used
+    g[:, :V] = torch.randn((T, V), generator=gen, device=DEV)
+    for f in (0.25, -3.7, 0.0):
+        s = torch.tensor(f, device=DEV)
+        whole = torch.full((T * V + 64,), 5.0, dtype=torch.bfloat16, device=DEV)
+        out = whole[: T * V].view(T, V)
+        assert api.scale_grad(g, s, V=V, out=out) is out
+        assert torch.equal(out.view(torch.int16), (g[:, :V] * s.to(torch.bfloat16)).view(torch.int16))
+        assert bool((whole[T * V:] == 5.0).all())
+    before = out.clone()
+    api.scale_grad(g, torch.ones((), device=DEV), V=V, out=out)
+    assert torch.equal(out.view(torch.int16), before.view(torch.int16))
+    with pytest.raises(acrl.AcrlError):   # neither V nor a multiple of eight
+        api.scale_grad(g, s, V=V, out=torch.empty((T, (V + 7) // 8 * 8 + 1), dtype=torch.bfloat16, device=DEV))
+
+
+@pytest.mark.parametrize("V", [1000, 1003])
+def test_gradient_of_a_scaled_loss_is_contiguous(V):
+    """As the product of the gradient with the scale is: a hook may flatten it."""
+    b = W.generate(W.small_variant(W.GRPO, name="contiguous", n_prompts=2, group_size=4, len_lo=5, len_hi=20, V=V), seed=6,
+                   device=DEV)
+    step = acrl.AcrlStep.for_batch(b, acrl.Params())
+    x = b.logits[:, :V].detach().requires_grad_(True)
+    seen = []
+    x.register_hook(lambda g: seen.append(g.view(-1)))
+    loss = acrl.acrl_loss(step, x, b.ids, b.mask, b.logp_mu, b.rewards, b.seq_offsets, b.group_offsets)
+    (loss * 0.25).backward()
+    assert torch.equal(seen[0].view(x.shape).view(torch.int16), (step.grad[:, :V] * 0.25).view(torch.int16))

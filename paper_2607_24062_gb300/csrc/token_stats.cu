@@ -181,19 +181,26 @@ constexpr int kDepth = 3;
 //   T = 1,000: 17.4 against 22.8; a warp per row, V = 16,384, T = 6,000: 34.1
 //   against 37.9.
 // - Many: the ring for rows of a warp or less (V = 16,384, T = 65,536: 296 us
-//   against 317; V = 8,192: 153 against 162; V = 4,096: 82 against 88), the
-//   same for four warps a row.  Two warps a row: registers where the row's last
-//   step is a large part of it (V = 20,011: a step of 12,000 rows 254 us against
-//   257, of 40,000 750 against 762) and up to some 2.5 waves (V = 32,000, 5,000
-//   rows: 174 against 181), except just past one wave (V = 32,000, T = 3,500: 45
-//   against 40); else the ring (V = 32,000, steps of 16,000 and 38,000 rows: 485
-//   and 1,084 against 480 and 1,072).
-bool use_ring(int64_t T, int team, int V) {
+//   against 317; V = 8,192: 153 against 162; V = 4,096: 82 against 88).  Two warps
+//   a row: registers where the row's last step is a large part of it (V = 20,011: a
+//   step of 12,000 rows 254 us against 257, of 40,000 750 against 762) and up to
+//   some 2.5 waves (V = 32,000, 5,000 rows: 174 against 181), except just past one
+//   wave (V = 32,000, T = 3,500: 45 against 40); else the ring (V = 32,000, steps of
+//   16,000 and 38,000 rows: 485 and 1,084 against 480 and 1,072).  Four warps a row:
+//   the ring (V = 72,000, T = 8,000: 181 us in registers, 170; V = 151,936, T =
+//   8,000: 361 / 351), except in the last third of the register path's second wave
+//   (T = 3,000: V = 128,256 115.5 in registers, 121.4 with the ring; V = 262,144 223
+//   / 236; T = 2,400: 188 / 186; T = 3,100, past that wave: 258 / 234) and for the
+//   shorter of many rows that do not begin on 128-byte lines (T = 40,000: V = 40,968
+//   465 / 475, V = 45,064 509 / 523, but V = 45,184 511 / 510; T = 12,000 and V =
+//   43,008: 146 / 141).
+bool use_ring(int64_t T, int team, int V, int64_t ld) {
     constexpr int64_t kSms = 152;
     const int64_t q = T >= (int64_t(1) << 40) ? INT64_MAX : T * team * 10 / (128 * kSms);
     if (team <= 16) return true;
     if (q < 52) return true;
     if (team == 64) return V >= 28672 ? q > 400 || (q > 104 && q < 140) : q > 104 && q < 140;
+    if (team == 128 && ((q > 168 && q <= 200) || (ld % 64 != 0 && V < 57344 && q > 1400))) return false;
     return q > 104;
 }
 
@@ -222,7 +229,7 @@ extern "C" acrl_status acrl_token_stats(const acrl_bf16* logits, int64_t T, int6
                      : V <= kWarpRowMaxV   ? 32
                      : V <= kMidRowMaxV    ? 64
                                            : 128;
-    const bool ring = use_ring(T, team, v);
+    const bool ring = use_ring(T, team, v, ld);
     if (team == 8) return run(token_stats_team<64, kUnroll, 8, kDepth>, 64, kDepth, 8);
     if (team == 16) return run(token_stats_team<64, kUnroll, 16, kDepth>, 64, kDepth, 4);
     if (team == 32)

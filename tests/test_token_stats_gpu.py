@@ -70,3 +70,21 @@ def test_undefined_rows_and_bad_ids(V):
     for x in (lse, logp, ent):
         assert bool(x[:-2].isnan().all()) and not bool(x[-2:].isnan().any())
     assert float(logp[-2]) == 0.0 and float(logp[-1]) == 0.0
+
+
+@pytest.mark.parametrize("V,ld,T", [(40968, 40968, 2553), (40968, 40968, 2600), (40968, 40968, 3040), (40968, 40968, 3041),
+                                    (40968, 40968, 21300), (40968, 41024, 21300), (65537, 65544, 2700), (262144, 262144, 2600)])
+def test_many_rows_of_four_warps_agree_with_few(V, ld, T):
+    """On both sides of the lines between ring and registers for rows of four warps, by rows and by row stride."""
+    gen = torch.Generator(device=DEV).manual_seed(V)
+    R = 7
+    base = torch.full((R, ld), float("nan"), dtype=torch.bfloat16, device=DEV)
+    base[:, :V] = torch.randn((R, V), generator=gen, device=DEV) * 3
+    ids = torch.randint(0, V, (R,), generator=gen, device=DEV, dtype=torch.int32)
+    flags = api.new_flags()
+    few = api.token_stats(base, ids, None, V=V, flags=flags)
+    pick = torch.arange(T, device=DEV) % R
+    many = api.token_stats(base[pick], ids[pick], None, V=V, flags=flags)
+    assert api.read_flags(flags) == 0
+    for a, b in zip(few, many):
+        assert torch.equal(a[pick].view(torch.int32), b.view(torch.int32))

@@ -107,8 +107,25 @@ __global__ void __launch_bounds__(THREADS) token_stats_warp(const acrl_bf16* __r
 // which matters where the merges' exponentials are a large share of the row's
 // (V = 2,048: 0.75 -> 0.94 of the copy rate with 8 lanes).  Every lane takes part
 // in the shuffles, whether its row is masked or not.
+// Sixteen lanes bring their sums to the team's maximum once and add them: a level of
+// merges more than eight lanes have, each with an exponential of its own, left the
+// entropy of V = 4,096 1.5-2.1 % further from float64 (rms) than eight lanes do.
 template <int LANES>
 __device__ __forceinline__ LseAcc team_lse(LseAcc a) {
+    if constexpr (LANES == 16) {
+        LseAcc r = a;
+#pragma unroll
+        for (int m = LANES / 2; m >= 1; m >>= 1) r.U = fmaxf(r.U, __shfl_xor_sync(0xffffffffu, r.U, m));
+        const float da = a.U - r.U, f = a.s0 > 0.f ? ex2(da) : 0.f;   // an empty lane contributes nothing
+        r.s0 = f * a.s0;
+        r.s1 = a.s0 > 0.f ? f * fmaf(da, a.s0, a.s1) : 0.f;
+#pragma unroll
+        for (int m = LANES / 2; m >= 1; m >>= 1) {
+            r.s0 += __shfl_xor_sync(0xffffffffu, r.s0, m);
+            r.s1 += __shfl_xor_sync(0xffffffffu, r.s1, m);
+        }
+        return r;
+    }
 #pragma unroll
     for (int m = LANES / 2; m >= 1; m >>= 1) a = lse_merge(a, shfl_xor(a, m));
     return a;

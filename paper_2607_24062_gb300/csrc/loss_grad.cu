@@ -381,34 +381,24 @@ __device__ __forceinline__ RowPlan make_plan(float c, float e, float L, float H,
     return rp;
 }
 
-// The online state without the entropy's sum, and its merge (lse_merge's).
-struct LseSum {
-    float U, s0;
-};
+// A thread's or a warp's sum of exponentials s, taken against its own maximum m,
+// brought to the maximum of all: one exponential for each, and the sums that follow
+// are plain (merging level by level, with an exponential each, the more warps of a
+// CTA have left the log-prob up to 1.1 % further from float64, rms).  A state's
+// exponent is its maximum times log2(e), rounded, as the folds keep it; an empty
+// state contributes nothing.
+__device__ __forceinline__ float lse_exponent(float m) { return __fmul_rn(m, kLog2e); }
 
-__device__ __forceinline__ LseSum sum_exp_merge(const LseSum& a, const LseSum& b) {
-    const float U = fmaxf(a.U, b.U);
-    const float fa = a.s0 > 0.f ? ex2(a.U - U) : 0.f;
-    const float fb = b.s0 > 0.f ? ex2(b.U - U) : 0.f;
-    return LseSum{U, fa * a.s0 + fb * b.s0};
+__device__ __forceinline__ float sum_at(float s, float m, float to) {
+    return (s > 0.f ? ex2(lse_exponent(m) - lse_exponent(to)) : 0.f) * s;
 }
 
-__device__ __forceinline__ LseSum shfl_xor(const LseSum& a, int m) {
-    return LseSum{__shfl_xor_sync(0xffffffffu, a.U, m), __shfl_xor_sync(0xffffffffu, a.s0, m)};
-}
-
-__device__ __forceinline__ LseSum warp_sum_exp(LseSum a) {
-#pragma unroll
-    for (int m = 16; m >= 1; m >>= 1) a = sum_exp_merge(a, shfl_xor(a, m));
-    return a;
-}
-
-// lse and logp = z_a - lse of a row from its merged state and maximum, in the
+// lse and logp = z_a - lse of a row from its sum and maximum, in the
 // same form as the statistics kernel (the rounding of max*log2(e) corrected
 // exactly through an FMA).
-__device__ __forceinline__ void lse_logp(const LseSum& acc, float mx, float za, float& L, float& lp) {
-    const float l2s0 = log2f(acc.s0);
-    const float c = fmaf(mx, kLog2e, -acc.U);
+__device__ __forceinline__ void lse_logp(float sum, float mx, float za, float& L, float& lp) {
+    const float l2s0 = log2f(sum);
+    const float c = fmaf(mx, kLog2e, -lse_exponent(mx));
     L = fmaf(kLn2, l2s0 - c, mx);
     lp = (za - mx) - kLn2 * (l2s0 - c);
 }
@@ -427,7 +417,7 @@ __device__ __forceinline__ void grad_row(const acrl_bf16* __restrict__ logits, i
                                          const float* __restrict__ lse, const float* __restrict__ old_logp,
                                          const float* __restrict__ coef, const float* __restrict__ entropy,
                                          const float* __restrict__ ent_coef, float eps, acrl_bf16* __restrict__ grad,
-                                         float* __restrict__ token_loss, int32_t* flags, int tid, LseSum* part,
+                                         float* __restrict__ token_loss, int32_t* flags, int tid, float* part,
                                          float* part_mx, int& par, const RowKeep& kp, const RowShare& sh) {
     const acrl_bf16* row = logits + t * ld;
     acrl_bf16* grow = grad + t * ld;
@@ -450,38 +440,38 @@ __device__ __forceinline__ void grad_row(const acrl_bf16* __restrict__ logits, i
         }
         za = bf16_to_float(row[a]);
         if (RECOMPUTE) {
-            float mx;
-            const LseAcc mine = recompute_partial<TEAM, UNROLL, TM>(row, V, tid, mx, kp, uint32_t(par), flags);
-            LseSum acc = warp_sum_exp(LseSum{mine.U, mine.s0});   // the entropy's sum is not wanted: the compiler drops it
+            float top;
+            const LseAcc mine = recompute_partial<TEAM, UNROLL, TM>(row, V, tid, top, kp, uint32_t(par), flags);
+            float mx = warp_max(top);
+            float sum = warp_sum(sum_at(mine.s0, top, mx));   // the entropy's sum is not wanted: the compiler drops it
             if (TM && kp.tm_chunks > 0)
                 tmem_wait_st();   // before the barrier: the row's tensor-memory part is written
-            mx = warp_max(mx);
             if (TEAM > 32) {
-                // Every warp combines the warps' states with the same butterfly, so all threads hold the same
+                // Every warp combines the warps' sums with the same butterfly, so all threads hold the same
                 // result with one barrier.  The next write to this buffer comes two rows later, after the next
                 // row's barrier, which every warp reaches only once it has read this one.
                 constexpr int NW = TEAM / 32;
                 static_assert(!RECOMPUTE || (NW <= 32 && (NW & (NW - 1)) == 0), "warps per team");
                 const int lane = tid & 31;
-                LseSum* pp = part + par * NW;
+                float* ps = part + par * NW;
                 float* pm = part_mx + par * NW;
                 if (lane == 0) {
-                    pp[tid >> 5] = acc;
+                    ps[tid >> 5] = sum;
                     pm[tid >> 5] = mx;
                 }
                 __syncthreads();
-                acc = lane < NW ? pp[lane] : LseSum{-INFINITY, 0.f};
-                mx = lane < NW ? pm[lane] : -INFINITY;
+                sum = lane < NW ? ps[lane] : 0.f;
+                top = mx = lane < NW ? pm[lane] : -INFINITY;
 #pragma unroll
-                for (int o = NW / 2; o >= 1; o >>= 1) {
-                    acc = sum_exp_merge(acc, shfl_xor(acc, o));
-                    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-                }
-                acc = LseSum{__shfl_sync(0xffffffffu, acc.U, 0), __shfl_sync(0xffffffffu, acc.s0, 0)};
+                for (int o = NW / 2; o >= 1; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+                sum = sum_at(sum, top, mx);
+#pragma unroll
+                for (int o = NW / 2; o >= 1; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+                sum = __shfl_sync(0xffffffffu, sum, 0);
                 mx = __shfl_sync(0xffffffffu, mx, 0);
                 par ^= 1;
             }
-            lse_logp(acc, mx, za, L, lp);
+            lse_logp(sum, mx, za, L, lp);
         } else {
             L = lse[t];
             lp = za - L;
@@ -518,7 +508,7 @@ __global__ void __launch_bounds__(THREADS) loss_grad_cta(
     const uint8_t* __restrict__ mask, const float* __restrict__ lse, const float* __restrict__ old_logp,
     const float* __restrict__ coef, const float* __restrict__ entropy, const float* __restrict__ ent_coef, float eps,
     acrl_bf16* __restrict__ grad, float* __restrict__ token_loss, int32_t* flags, int shares) {
-    __shared__ LseSum part[2 * (THREADS / 32)];
+    __shared__ float part[2 * (THREADS / 32)];
     __shared__ float part_mx[2 * (THREADS / 32)];
     __shared__ uint32_t tmem_base;
     __shared__ __align__(8) uint64_t keep_bar;

@@ -348,10 +348,11 @@ acrl_status acrl_importance_weights(acrl_controller_state* state, const acrl_par
  * The probabilities are never stored.  Rows with m_t = 0, or with no
  * gradient (coef_t g_t = 0 and no entropy bonus), get a zero gradient row
  * without reading the rest of their logits.  A row that carries a gradient
- * but whose lse (given or recomputed) or log-prob is not finite (a NaN or an
- * infinity among its logits), or whose old_logp is NaN, has no defined
- * surrogate: its gradient row and token_loss_t are NaN (and so is *loss), and
- * the call raises ACRL_FLAG_NONFINITE.
+ * but whose lse or log-prob is not finite, or whose old_logp is NaN, has no
+ * defined surrogate: its gradient row and token_loss_t are NaN (and so is
+ * *loss), and the call raises ACRL_FLAG_NONFINITE.  That is a row with a NaN or
+ * an infinity among its logits; with the lse recomputed, a column other than
+ * the sampled one may be -infinity, which is probability 0 there.
  *   logits  device bf16 [T, ld];  grad  device bf16 [T, ld] output (columns
  *           >= V untouched).  May be called on a chunk of rows: every
  *           per-token pointer then points at the chunk's first row.

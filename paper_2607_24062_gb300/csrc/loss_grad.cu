@@ -215,7 +215,7 @@ __device__ __forceinline__ uint4 grad_vec(const uint4 v, const RowPlan& rp, int 
 template <int TEAM, int UNROLL, bool TM>
 __device__ __forceinline__ LseAcc recompute_partial(const acrl_bf16* __restrict__ row, int V, int tid, float& mx,
                                                     const RowKeep& kp, uint32_t parity, int32_t* flags) {
-    LseAcc acc = lse_empty();
+    LseAcc acc{kLowestU, 0.f, 0.f};   // columns at -infinity add nothing, whichever the thread meets first
     mx = -INFINITY;
     const int nvec = V >> 3;
     const uint4* vrow = reinterpret_cast<const uint4*>(row);
@@ -230,14 +230,14 @@ __device__ __forceinline__ LseAcc recompute_partial(const acrl_bf16* __restrict_
             for (int k = 0; k < UNROLL; ++k) buf[k] = ld_policy(vrow + v + k * TEAM, once);
 #pragma unroll
             for (int k = 0; k < UNROLL; ++k) tmem_st4(kp.tbase + uint32_t(16 * ch + 4 * k), buf[k]);
-            fold_vectors<UNROLL>(acc, mx, buf);
+            fold_vectors<UNROLL, true>(acc, mx, buf);
         }
     }
     for (; v + (UNROLL - 1) * TEAM < nvec; v += UNROLL * TEAM) {
         uint4 buf[UNROLL];
 #pragma unroll
         for (int k = 0; k < UNROLL; ++k) buf[k] = ld_policy(vrow + v + k * TEAM, pol);
-        fold_vectors<UNROLL>(acc, mx, buf);
+        fold_vectors<UNROLL, true>(acc, mx, buf);
     }
     const int j = (nvec << 3) + tid;   // at most one column per thread beyond the whole vectors
     const float last = j < V ? bf16_to_float(row[j]) : 0.f;
@@ -245,20 +245,20 @@ __device__ __forceinline__ LseAcc recompute_partial(const acrl_bf16* __restrict_
         v, nvec, [&](int i) { return ld_policy(vrow + i, pol); },
         [&](const uint4& x, int) {
             const uint4 buf[1] = {x};
-            fold_vectors<1>(acc, mx, buf);
+            fold_vectors<1, true>(acc, mx, buf);
         });
-    if (j < V) fold_scalar(acc, mx, last);
+    if (j < V) fold_scalar<true>(acc, mx, last);
     if (s > 0) {
         if (!wait_phase(kp.bar, parity, nullptr)) raise_flag(flags, ACRL_FLAG_TIMEOUT);
         for (v = tid; v + (UNROLL - 1) * TEAM < s; v += UNROLL * TEAM) {
             uint4 buf[UNROLL];
 #pragma unroll
             for (int k = 0; k < UNROLL; ++k) buf[k] = kp.smem[v + k * TEAM];
-            fold_vectors<UNROLL>(acc, mx, buf);
+            fold_vectors<UNROLL, true>(acc, mx, buf);
         }
         for (; v < s; v += TEAM) {
             uint4 buf[1] = {kp.smem[v]};
-            fold_vectors<1>(acc, mx, buf);
+            fold_vectors<1, true>(acc, mx, buf);
         }
     }
     return acc;

@@ -13,8 +13,18 @@ __device__ __forceinline__ uint32_t max_bf16x2(uint32_t a, uint32_t b) {
     return r;
 }
 
+// A running maximum's exponent.  BOUNDED: the products of numbers near the type's
+// lowest stay finite, so that a thread which has met nothing else, or (with a state
+// that starts at kLowestU) only infinities, holds an empty sum.
+constexpr float kLowestU = -3.402823466e38f;
+
+template <bool BOUNDED>
+__device__ __forceinline__ float max_exponent(float m) {
+    return BOUNDED ? fmaxf(m * kLog2e, kLowestU) : m * kLog2e;
+}
+
 // Fold UNROLL 8-element vectors into the thread's running state.
-template <int UNROLL>
+template <int UNROLL, bool BOUNDED = false>
 __device__ __forceinline__ void fold_vectors(LseAcc& acc, float& mx, const uint4 (&v)[UNROLL]) {
     float f[UNROLL][8];
 #pragma unroll
@@ -31,7 +41,7 @@ __device__ __forceinline__ void fold_vectors(LseAcc& acc, float& mx, const uint4
         pm = max_bf16x2(pm, max_bf16x2(max_bf16x2(v[k].x, v[k].y), max_bf16x2(v[k].z, v[k].w)));
     const float vm = fmaxf(bf16_lo(pm), bf16_hi(pm));
     if (vm > mx) {  // new running maximum: rescale the partial sums
-        const float Un = vm * kLog2e;
+        const float Un = max_exponent<BOUNDED>(vm);
         if (acc.s0 > 0.f) {
             const float dl = acc.U - Un;
             const float s = ex2(dl);
@@ -59,9 +69,10 @@ __device__ __forceinline__ void fold_vectors(LseAcc& acc, float& mx, const uint4
     acc.s1 += s1a + s1b;
 }
 
+template <bool BOUNDED = false>
 __device__ __forceinline__ void fold_scalar(LseAcc& acc, float& mx, float z) {
     if (z > mx) {
-        const float Un = z * kLog2e;
+        const float Un = max_exponent<BOUNDED>(z);
         if (acc.s0 > 0.f) {
             const float dl = acc.U - Un;
             const float s = ex2(dl);

@@ -173,3 +173,38 @@ def test_recomputed_log_prob_is_as_close_as_with_fewer_warps(V, rms):
         sq += float((tl.double().log() + old.double() - lp).square().sum())
         rows += T
     assert (sq / rows) ** 0.5 <= rms, (sq / rows) ** 0.5
+
+
+@pytest.mark.parametrize("V", [7, 1001, 4097, 5003, 6143, 6145, 7168, 7170, 20011, 22001, 24583, 36870, 40967, 49155, 61003, 70001,
+                               151937])
+@pytest.mark.parametrize("mask_value", [float("-inf"), -3.3895313892515355e38])
+def test_recomputed_gradient_of_masked_columns(V, mask_value):
+    """Columns at -infinity or at bf16's lowest number have probability 0 wherever in the row they are: the ragged last
+    column, the last vectors, the first half, all but a few; the lse of the others is finite, and so is the gradient."""
+    gen = torch.Generator(device=DEV).manual_seed(V)
+    ld = (V + 7) // 8 * 8
+    few = torch.randperm(V, generator=gen, device=DEV)[:5]
+    off = torch.zeros((5, V), dtype=torch.bool, device=DEV)
+    off[0, V - 1:] = True
+    off[1, max(1, V - 27):] = True
+    off[2, : V // 2] = True
+    off[3, :] = True
+    off[3, few] = False
+    x = torch.full((5, ld), float("nan"), dtype=torch.bfloat16, device=DEV)
+    x[:, :V] = (torch.randn((5, V), generator=gen, device=DEV) * 2).masked_fill(off, mask_value)
+    ids = (~off).to(torch.uint8).argmax(dim=1).to(torch.int32)
+    coef = torch.tensor([0.5, -0.25, 1.0, -1.0, 0.125], device=DEV)
+    z = x[:, :V].double()
+    lp = z - z.logsumexp(dim=1)[:, None]
+    old = lp.gather(1, ids.long()[:, None])[:, 0].float()
+    flags = api.new_flags()
+    g, tl, _ = api.loss_grad_logits(x, ids, None, None, old, coef, 0.2, V=V, flags=flags)
+    assert api.read_flags(flags) == 0
+    c, p = coef.double(), lp.exp()
+    want = p * c[:, None]
+    want.scatter_add_(1, ids.long()[:, None], -c[:, None])
+    # as in _check, the ratio's rounding of 2^-22 besides
+    size = (p * c.abs()[:, None]).scatter_add_(1, ids.long()[:, None], c.abs()[:, None])
+    assert bool(((g[:, :V].double() - want).abs() <= 2.0 ** -8 * want.abs() + 2.0 ** -16 * size + 1e-38).all())
+    assert bool((g[:, :V][off] == 0).all())
+    assert bool(((tl.double() + c).abs() <= 2.0 ** -18 * c.abs()).all())

@@ -377,12 +377,12 @@ __device__ __forceinline__ void grpo_prompt(int64_t tid, const float* __restrict
     const int sub = int(tid % LANES);
     if (g >= Gn) return;  // the prompt's lanes leave together
     const unsigned team = LANES == 1 ? 0u : ((1u << LANES) - 1u) << (threadIdx.x & 31 & ~(LANES - 1));
-    const int b = goff[g], e = goff[g + 1];
+    const int64_t b = goff[g], e = goff[g + 1];   // 64 bits: the lanes step past e, which may be the type's largest
     if (b < 0 || b > e || e > S) {
         if (sub == 0) raise_flag(flags, ACRL_FLAG_BAD_OFFSETS);
         return;
     }
-    const int G = e - b;
+    const int G = int(e - b);
     if (G == 0) return;
     if (G == 1) {
         if (sub == 0) adv[b] = singleton_rule == ACRL_SINGLETON_MEAN0_STD1 ? R[b] : 0.f;
@@ -396,7 +396,7 @@ __device__ __forceinline__ void grpo_prompt(int64_t tid, const float* __restrict
     float r[KEEP];
 #pragma unroll
     for (int k = 0; k < KEEP; ++k) r[k] = b + sub + k * LANES < e ? R[b + sub + k * LANES] : 0.f;
-    const int rest = b + sub + KEEP * LANES;
+    const int64_t rest = b + sub + KEEP * LANES;
     double sum = 0.0;
 #pragma unroll
     for (int k = 0; k < KEEP; ++k)

@@ -106,3 +106,23 @@ def test_rows_beyond_32_bit_indices():
     resp = np.searchsorted(cuts, rows, side="right") - 1
     want = A[resp] / (Gn * G * n[resp])
     np.testing.assert_allclose(coef[torch.as_tensor(rows, device=dev)].cpu().numpy(), want, rtol=1e-5, atol=0)
+
+
+@pytest.mark.parametrize("size", [2048, 1 << 22])
+def test_advantages_up_to_the_last_32_bit_response(size):
+    """2^31 - 1 responses, the most that the call counts: a lane's steps beyond the last prompt's three responses leave
+    32 bits.  Prompts of 2,048 (a lane each) and of 2^22 (eight lanes each)."""
+    dev = torch.device("cuda")
+    torch.cuda.empty_cache()
+    S = (1 << 31) - 1
+    go = torch.cat([torch.arange(0, S - 3, size, dtype=torch.int64), torch.tensor([S - 3, S])]).to(torch.int32).to(dev)
+    R = torch.zeros(S, device=dev)
+    tail = torch.tensor([0.0, 1.0, 5.0], device=dev)
+    R[-3:] = tail
+    p, flags = acrl.Params(), api.new_flags(dev)
+    adv = api.grpo_advantage(R, go, p, adv=torch.full((S,), 7.0, device=dev), flags=flags)
+    assert api.read_flags(flags) == 0
+    want = (tail.double() - 2.0) / (tail.double().std(unbiased=p.adv_ddof == 1) + p.adv_eps)
+    assert float((adv[-3:].double() - want).abs().max()) <= 1e-6
+    for i in range(0, S - 3, 1 << 28):
+        assert not bool(adv[i: min(S - 3, i + (1 << 28))].any())

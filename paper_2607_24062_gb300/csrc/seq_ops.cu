@@ -537,77 +537,40 @@ __device__ __forceinline__ float token_weight(int mode, const RespScalars& r, fl
     return isnan(lrho) ? 0.f : expf(fminf(lrho, logC));
 }
 
-// The controller's new state and the batch fields that come from it; one thread.
-// X: the reference in force, Ymean: the batch's mean discrepancy.
-__device__ __forceinline__ void write_state(const acrl_controller_state& old, const ControllerMove& mv, double X,
-                                            double Ymean, double alpha_mean, const acrl_params& p,
-                                            acrl_controller_state* st, acrl_batch_stats* batch, int32_t* flags) {
-    const bool was_calibrated = old.calibrated != 0;
-    acrl_controller_state n = mv.next;
-    n.X = X;
-    const bool uses_x = p.mode == ACRL_MODE_ACRL || p.mode == ACRL_MODE_ACRL_FALLBACK;
-    if (uses_x && mv.apply && !(X > 0.0)) {
-        raise_flag(flags, ACRL_FLAG_X_NONPOS);
-        n.flags |= ACRL_FLAG_X_NONPOS;
-    }
-    // moving-average X (off by default): this step used X, the next one uses the update
-    if (was_calibrated && p.x_ema > 0.f) n.X = fma(double(p.x_ema), Ymean, (1.0 - double(p.x_ema)) * X);
-    *st = n;
-    batch->Y_mean = Ymean;
-    batch->X = mv.apply ? X : 0.0;
-    batch->alpha_mean = alpha_mean;
-}
-
-// K4a: the controller's new state and alpha per response, in a launch of its own
-// (acrl_controller_step; acrl_importance_weights folds both into the next two
-// kernels).  Warp 0 works out the X in force and writes the state.
-__global__ void __launch_bounds__(kFinThreads) controller_alpha_kernel(
-    acrl_controller_state* st, acrl_params p, int S, int Gn, acrl_seq_stats* seq,
-    const acrl_group_stats* __restrict__ grp, acrl_batch_stats* batch, const float* __restrict__ adv,
-    float* __restrict__ alpha_out, int32_t* flags) {
-    __shared__ double sh_X, sh_Y;   // the X in force, the batch's Y
-    __shared__ bool sh_apply;
+// K4a: alpha per response, in a launch of its own (acrl_controller_step;
+// acrl_importance_weights folds it into the next kernel).  Every warp works out the X
+// in force for itself; the finalising kernel writes the state.
+__global__ void __launch_bounds__(kSeqThreads) controller_alpha_kernel(
+    const acrl_controller_state* __restrict__ st, acrl_params p, int S, int Gn, acrl_seq_stats* seq,
+    const acrl_group_stats* __restrict__ grp, const acrl_batch_stats* __restrict__ batch, const float* __restrict__ adv,
+    float* __restrict__ alpha_out) {
     const int lane = threadIdx.x & 31;
     grid_begin();
-    if (threadIdx.x < 32) {
-        const int ngv = batch->n_groups_valid;
-        const double Ysum = batch->Y_sum;
-        const acrl_controller_state old = *st;
-        const ControllerMove mv = controller_move(old, p, Ysum, ngv);
-        // one division: X in lane 0, Y_mean (of the possibly all-reduced sum and prompt count) in lane 1
-        const double num = lane == 0 ? mv.x_num : Ysum, den = lane == 0 ? mv.x_den : double(ngv);
-        const double q = den > 0.0 ? div64(num, den) : 0.0;
-        const double Ymean = __shfl_sync(0xffffffffu, q, 1);
-        if (lane == 0) {
-            sh_X = q;
-            sh_Y = Ymean;
-            sh_apply = mv.apply;
-            write_state(old, mv, q, Ymean, 0.0, p, st, batch, flags);
-        }
-    }
-    __syncthreads();
-    const double X = sh_X, inv_X = recip64(X);
-    for (int64_t i = threadIdx.x; i < S; i += kFinThreads) {
-        const int n = seq[i].n, g = seq[i].group;
-        double num = 0.0, den = 1.0;
-        if (p.y_gran == ACRL_Y_SEQUENCE) {
-            num = seq[i].sum_d;
-            den = double(n);
-        } else if (p.y_gran == ACRL_Y_BATCH) {
-            num = sh_Y;
-        } else if (g >= 0 && g < Gn) {
-            num = grp[g].Y;
-        }
-        const float a = alpha_of(p, sh_apply, X, inv_X, den > 0.0 ? div64(num, den) : 0.0, adv[i], n);
-        seq[i].alpha = a;
-        if (alpha_out) alpha_out[i] = a;
-    }
+    const int ngv = batch->n_groups_valid;
+    const double Ysum = batch->Y_sum;
+    const ControllerMove mv = controller_move(*st, p, Ysum, ngv);
+    // one division: X in lane 0, the batch's Y (of the possibly all-reduced sum and prompt count) in lane 1
+    const double num = lane == 0 ? mv.x_num : Ysum, den = lane == 0 ? mv.x_den : double(ngv);
+    const double q = den > 0.0 ? div64(num, den) : 0.0;
+    const double X = __shfl_sync(0xffffffffu, q, 0), Ybatch = __shfl_sync(0xffffffffu, q, 1);
+    const int64_t i = int64_t(blockIdx.x) * kSeqThreads + threadIdx.x;
+    if (i >= S) return;
+    const int n = seq[i].n, g = seq[i].group;
+    double Y = 0.0;
+    if (p.y_gran == ACRL_Y_SEQUENCE)
+        Y = n > 0 ? div64(seq[i].sum_d, double(n)) : 0.0;
+    else if (p.y_gran == ACRL_Y_BATCH)
+        Y = Ybatch;
+    else if (g >= 0 && g < Gn)
+        Y = grp[g].Y;
+    const float a = alpha_of(p, mv.apply, X, recip64(X), Y, adv[i], n);
+    seq[i].alpha = a;
+    if (alpha_out) alpha_out[i] = a;
 }
 
 // K4b: per-token weights and loss coefficients; a cluster of CTAs per response as
-// in seq_stats_kernel.  FOLD: alpha per response too (every CTA works out the X in
-// force for itself; the finalising kernel writes the state); otherwise alpha is
-// controller_alpha_kernel's.
+// in seq_stats_kernel.  FOLD: alpha per response too, from the X in force as
+// controller_alpha_kernel works it out; otherwise alpha is that kernel's.
 template <bool FOLD>
 __global__ void __launch_bounds__(kSeqThreads) controller_weights_kernel(
     const acrl_controller_state* __restrict__ st, acrl_params p, const float* __restrict__ lr,
@@ -747,8 +710,28 @@ __global__ void __launch_bounds__(kSeqThreads) controller_weights_kernel(
     if (nct > 1) cluster_sync();  // no CTA leaves while rank 0 may still read its shared memory
 }
 
-// K4c: the batch metrics, and with FOLD the controller's new state.
-template <bool FOLD>
+// The controller's new state and the batch fields that come from it; one thread.
+// X: the reference in force, Ymean: the batch's mean discrepancy.
+__device__ __forceinline__ void write_state(const acrl_controller_state& old, const ControllerMove& mv, double X,
+                                            double Ymean, double alpha_mean, const acrl_params& p,
+                                            acrl_controller_state* st, acrl_batch_stats* batch, int32_t* flags) {
+    const bool was_calibrated = old.calibrated != 0;
+    acrl_controller_state n = mv.next;
+    n.X = X;
+    const bool uses_x = p.mode == ACRL_MODE_ACRL || p.mode == ACRL_MODE_ACRL_FALLBACK;
+    if (uses_x && mv.apply && !(X > 0.0)) {
+        raise_flag(flags, ACRL_FLAG_X_NONPOS);
+        n.flags |= ACRL_FLAG_X_NONPOS;
+    }
+    // moving-average X (off by default): this step used X, the next one uses the update
+    if (was_calibrated && p.x_ema > 0.f) n.X = fma(double(p.x_ema), Ymean, (1.0 - double(p.x_ema)) * X);
+    *st = n;
+    batch->Y_mean = Ymean;
+    batch->X = mv.apply ? X : 0.0;
+    batch->alpha_mean = alpha_mean;
+}
+
+// K4c: the controller's new state and the batch metrics.
 __global__ void __launch_bounds__(kFinThreads) controller_finalize_kernel(acrl_controller_state* st, acrl_params p,
                                                                           int S,
                                                                           const acrl_seq_stats* __restrict__ seq,
@@ -780,26 +763,19 @@ __global__ void __launch_bounds__(kFinThreads) controller_finalize_kernel(acrl_c
     const long long nt = warp_sum(lane < used ? sh_nt[lane] : 0ll);
     const int ngv = batch->n_groups_valid, nsv = batch->n_seqs_valid;
     const double Ysum = batch->Y_sum, N = double(batch->n_tokens);
-    acrl_controller_state old;
-    ControllerMove mv;
-    if (FOLD) {
-        old = *st;
-        mv = controller_move(old, p, Ysum, ngv);
-    }
+    const acrl_controller_state old = *st;
+    const ControllerMove mv = controller_move(old, p, Ysum, ngv);
     // one division: w_mean, alpha_mean, trunc_frac, Y_mean (of the possibly all-reduced sum and prompt count), X
     double num = s, den = N;
     if (lane == 1) den = double(nsv);
     if (lane == 2) num = double(nt);
-    if (FOLD && lane == 3) num = Ysum, den = double(ngv);
-    if (FOLD && lane == 4) num = mv.x_num, den = mv.x_den;
+    if (lane == 3) num = Ysum, den = double(ngv);
+    if (lane == 4) num = mv.x_num, den = mv.x_den;
     const double q = den > 0.0 ? div64(num, den) : 0.0;
     const double a_mean = __shfl_sync(0xffffffffu, q, 1), trunc = __shfl_sync(0xffffffffu, q, 2),
                  Ymean = __shfl_sync(0xffffffffu, q, 3), X = __shfl_sync(0xffffffffu, q, 4);
     if (lane == 0) {
-        if (FOLD)
-            write_state(old, mv, X, Ymean, a_mean, p, st, batch, flags);
-        else
-            batch->alpha_mean = a_mean;
+        write_state(old, mv, X, Ymean, a_mean, p, st, batch, flags);
         batch->trunc_frac = trunc;
         batch->w_mean = q;
     }
@@ -1136,8 +1112,7 @@ acrl_status launch_seq_stats(const float* logp_pi, const float* logp_mu, const u
                   group_offsets, Gn, entropy, lr, d, seq, flags);
 }
 
-// FOLD: two launches, the state and alpha made by the kernels of the weights and of
-// the metrics; otherwise three.  Same bits.
+// FOLD: two launches, alpha made by the weights' kernel; otherwise three.  Same bits.
 template <bool FOLD>
 acrl_status launch_controller(acrl_controller_state* state, const acrl_params& p, const float* lr, const uint8_t* mask,
                               int64_t T, const int64_t* seq_offsets, int32_t S, int32_t Gn, acrl_seq_stats* seq,
@@ -1145,13 +1120,14 @@ acrl_status launch_controller(acrl_controller_state* state, const acrl_params& p
                               float* coef, float* alpha, float* ent_coef, int32_t* flags, cudaStream_t s) {
     const int c = ctas_per_response(S, T);
     acrl_status st = ACRL_OK;
-    if (!FOLD)
-        st = launch(controller_alpha_kernel, 1, kFinThreads, 0, 0, s, state, p, S, Gn, seq, grp, batch, adv, alpha, flags);
+    if (!FOLD && S > 0)
+        st = launch(controller_alpha_kernel, (int64_t(S) + kSeqThreads - 1) / kSeqThreads, kSeqThreads, 0, 0, s, state, p, S,
+                    Gn, seq, grp, batch, adv, alpha);
     if (st == ACRL_OK && S > 0)
         st = launch(controller_weights_kernel<FOLD>, int64_t(S) * c, kSeqThreads, 0, c, s, state, p, lr, mask, T,
                     seq_offsets, Gn, seq, grp, batch, adv, weight, coef, alpha, ent_coef);
     if (st != ACRL_OK) return st;
-    return launch(controller_finalize_kernel<FOLD>, 1, kFinThreads, 0, 0, s, state, p, S, seq, batch, flags);
+    return launch(controller_finalize_kernel, 1, kFinThreads, 0, 0, s, state, p, S, seq, batch, flags);
 }
 
 }  // namespace

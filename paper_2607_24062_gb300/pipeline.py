@@ -110,12 +110,13 @@ class AcrlStep:
         self.gradient(logits, ids, mask, stream=stream, **grad_kw)
 
     def _whole(self, logits, rewards, seq_offsets, group_offsets) -> bool:
-        """The batch is the one this object was built for, and its two halves are the ones below: one call does both."""
-        cls = type(self)
+        """The batch is the one this object was built for, and its two halves are this module's, overridden neither by
+        a class nor on the object: one call does both."""
+        halves = (getattr(self, name, None) for name in ("statistics", "gradient"))
         return (logits.shape[0] == self.T == self.logp.numel() and seq_offsets.numel() == self.S + 1 and
                 group_offsets.numel() == self.Gn + 1 and rewards.numel() == self.S and self.disc.S == self.S and
                 self.disc.Gn == self.Gn and
-                cls.statistics is AcrlStep.statistics and cls.gradient is AcrlStep.gradient)
+                all(getattr(h, "__self__", None) is self and h.__func__ is own for h, own in zip(halves, _HALVES)))
 
     @classmethod
     def for_batch(cls, batch, params: Params, device="cuda", grad_rows=None):
@@ -156,6 +157,9 @@ class AcrlStep:
 
     def state_host(self):
         return api.read_state(self.state)
+
+
+_HALVES = (AcrlStep.statistics, AcrlStep.gradient)   # as defined above, whatever is set on the class later
 
 
 def _struct_out(dtype, n: int, dev) -> torch.Tensor:

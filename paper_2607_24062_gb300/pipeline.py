@@ -189,6 +189,8 @@ def importance_weights(state, params: Params, logp_old, logp_mu, mask, rewards, 
     flags = api.new_flags(logp_old.device) if flags is None else flags
     if exchange is None:
         dev, T, S, Gn = logp_old.device, logp_old.numel(), seq_offsets.numel() - 1, group_offsets.numel() - 1
+        if S < 0 or Gn < 0:
+            raise AcrlError("seq_offsets / group_offsets: empty")
         f32 = dict(dtype=torch.float32, device=dev)
         lr, d, weight, coef = (torch.empty(T, **f32) for _ in range(4))
         adv, alpha = torch.empty(rewards.numel(), **f32), torch.empty(S, **f32)

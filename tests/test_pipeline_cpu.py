@@ -57,3 +57,10 @@ def test_an_overridden_half_is_called(calls, monkeypatch, name, where):
         monkeypatch.setattr(acrl.AcrlStep, name, mine)
     step.run(*_args())
     assert "mine" in calls and "step" not in calls
+
+
+@pytest.mark.parametrize("so,go", [(0, 2), (3, 0)])
+def test_weights_refuse_empty_offsets(so, go):
+    with pytest.raises(acrl.AcrlError):
+        acrl.importance_weights(torch.zeros(48, dtype=torch.uint8), acrl.Params(), torch.zeros(4), torch.zeros(4), None,
+                                torch.zeros(2), torch.zeros(so, dtype=torch.int64), torch.zeros(go, dtype=torch.int32))

@@ -360,7 +360,7 @@ acrl_status acrl_importance_weights(acrl_controller_state* state, const acrl_par
  *   lse     device float [T] from acrl_token_stats on the same logits, or
  *           NULL to recompute it here (the cached-old path: a second sweep
  *           over each row; for rows of 4,096 columns or more each CTA keeps
- *           up to 20 KB (rows of up to 7,168 columns), 40 KB (up to 20,487),
+ *           up to 14 KB (rows of up to 7,168 columns), 40 KB (up to 20,487),
  *           72 KB (up to 40,967) or 96 KB of its row in shared memory, loaded
  *           by one bulk copy per row whose wait is bounded
  *           (ACRL_FLAG_TIMEOUT), and, from 65,536 columns, up to 128 KB in

@@ -53,7 +53,8 @@ constexpr int kHalfBN = kBN / 2;      // weight rows staged by each CTA of a pai
 constexpr int kBBytes = kHalfBN * kBK * 2;
 // The ring: STAGES stages of B and of AROWS rows of A per CTA.  Up to 16 rows of
 // H in all, a stage holds and loads only those (the MMA reads the 128 rows that its
-// shape has; what the others hold lands in accumulator rows that nothing reads):
+// shape has; what the others hold lands in accumulator rows of its own, which the
+// epilogue carries along and its row test and the bounds of the copy out drop):
 // a copy whose box of 128 rows has eight or fewer in the tensor is slow, and the
 // freed memory makes more stages for the weight's stream from HBM.  K = 4,096,
 // N = 151,936 with the merge, M = 1 / 4 / 8 / 16: 380 / 331 / 306 / 211 us with

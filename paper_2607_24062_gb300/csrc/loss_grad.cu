@@ -13,7 +13,7 @@
 // coefficient and no bonus, clipped) are written as zeros without reading
 // their logits.  With lse == NULL the row's log-sum-exp is first recomputed
 // by a sweep over the same row; the first 16-byte vectors of the row (up to
-// 20, 40, 72 or 96 KB, by the CTA's size) stay in the CTA's shared memory and, for
+// 14, 40, 72 or 96 KB, by the CTA's size) stay in the CTA's shared memory and, for
 // rows of 65,536 columns or more, the next up to kTmemVecs (128 KB) in its
 // tensor memory between the two sweeps, so that only the rest of the row is
 // read again, from L2.  The shared-memory part arrives by one bulk copy
@@ -81,7 +81,7 @@ static_assert(kCtaThreads == 512 && kCtaUnroll == 4, "column layout: 16 warps, 4
 // resident per SM against 30.7 for the same work without tcgen05 code.
 constexpr int kTmemMinVecs = kKeepVecs + kChunk;
 // Shorter rows take smaller CTAs, so that several fit on an SM with what they keep:
-//   from kRecomputeCtaMinV columns  64 threads,  up to 20 KB: rows of up to 7,168
+//   from kRecomputeCtaMinV columns  64 threads,  up to 14 KB: V <= 7,168
 //   up to kTinyKeepVecs vectors    128 threads,  up to 40 KB: V <= 20,487
 //   up to kSmallMaxVecs vectors    256 threads,  up to 72 KB: V <= 40,967 (of a row
 //                                  longer than 72 KB the rest, at most 8 KB, is read
@@ -94,8 +94,8 @@ constexpr int kTmemMinVecs = kKeepVecs + kChunk;
 // 44,000 79 with 256, 68 with 512; 30,000 x 3,333 77 with a warp (in CTAs of two; 83
 // in CTAs of eight), 84 with 64 threads.
 constexpr int kRecomputeCtaMinV = 4096;
-constexpr int kLeastThreads = 64, kLeastKeepVecs = 1280;
 constexpr int kLeastMaxV = 7168;
+constexpr int kLeastThreads = 64, kLeastKeepVecs = kLeastMaxV / 8;
 constexpr int kTinyThreads = 128, kTinyKeepVecs = 2560;
 constexpr int kSmallThreads = 256, kSmallKeepVecs = 4608;
 constexpr int kSmallMaxVecs = 5120;

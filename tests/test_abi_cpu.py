@@ -163,3 +163,18 @@ def test_kernels_do_not_spill_and_fit_their_occupancy(L):
         found = {k: v for k, v in regs.items() if re.search(pattern, k)}
         assert found, pattern
         assert all(v <= limit for v in found.values()), found
+
+
+def test_kernels_of_vocabulary_rows_fit_their_residency():
+    """The streaming gradient of more than 65,536 columns has six CTAs of 256 threads per SM (at most 42 registers a
+    thread), the statistics' register path 1,280 threads (at most 48)."""
+    import os
+    import re
+    path = os.path.join(build.BUILD, "ptxas.txt")
+    if not os.path.exists(path):
+        build.build(force=True)
+    report = re.findall(r"Compiling entry function '(\S+)'.*?Used (\d+) registers", open(path).read(), flags=re.S)
+    for pattern, limit, n in ((r"loss_grad_ctaILi256ELi4ELb0ELb[01]ELb0ELb1E", 42, 2),
+                              (r"token_stats_ctaILi(64|128)ELi4ELi0E", 48, 2), (r"token_stats_warpILi256ELi4ELi0E", 48, 1)):
+        found = {k: int(v) for k, v in report if re.search(pattern, k)}
+        assert len(found) == n and all(v <= limit for v in found.values()), (pattern, found)

@@ -78,8 +78,10 @@ def test_lmhead_small_shapes(M, N, K):
 
 
 # the ring for up to 16 rows at its ends, with boxes of one and two eights of rows; more K slabs than stages, so
-# that it wraps, with K on and off the slab
-@pytest.mark.parametrize("M,N,K", [(1, 513, 1000), (8, 700, 1032), (9, 300, 64), (16, 1000, 2048), (17, 513, 1000)])
+# that it wraps, with K on and off the slab; more tiles than the 76 CTA pairs, so that a pair goes on to a second and a
+# third with the stage and phase of the last and the other accumulator
+@pytest.mark.parametrize("M,N,K", [(1, 513, 1000), (8, 700, 1032), (9, 300, 64), (16, 1000, 2048), (17, 513, 1000),
+                                   (3, 20011, 72), (16, 40001, 1032), (8, 58880, 264)])
 def test_lmhead_few_rows(M, N, K):
     test_lmhead_small_shapes(M, N, K)
 

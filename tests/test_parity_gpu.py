@@ -742,14 +742,14 @@ def test_importance_weights_from_log_probs(mode):
                                32000, 36864, 36871, 36872, 40960, 40967, 40968, 49152, 49153, 49160, 65535, 65536,
                                65537, 65544, 81920, 100000, 114688, 114695])
 def test_row_size_class_boundaries(V):
-    """Vocabularies at the edges of the row-team size classes (eight lanes up
-    to 4,096 columns, one warp up to 16,384, 64 threads up to 65,536, 128
-    above for the statistics;
-    one warp, then 512 threads, then 768 above 65,536 for the gradient; one
-    warp up to 6,144 columns, 128 threads up to 24,583, 256 up to 40,967,
-    then 512 for the gradient with the lse recomputed), of the 8-column
-    vectors and of the parts of a row the recompute path holds on chip
-    (20,480 columns in shared memory for 128-thread CTAs, 36,864 for 256-
+    """Vocabularies at the edges of the row-team size classes (for the
+    statistics eight lanes up to 3,584 columns, sixteen up to 4,608, a warp up
+    to 16,384, 64 threads up to 40,960, 128 above; for the gradient a warp
+    below 2,048 columns, CTAs of 64 to 512 threads, and from 65,537 columns
+    several CTAs a row; with the lse recomputed a warp below 4,096 columns, 64
+    threads up to 7,168, 128 up to 20,487, 256 up to 40,967, then 512), of the
+    8-column vectors and of the parts of a row the recompute path holds on
+    chip (20,480 columns in shared memory for 128-thread CTAs, 36,864 for 256-
     thread ones, 49,152 for 512-thread ones, then whole chunks of 16,384
     columns in tensor memory: 0 to 4 chunks, with and without a ragged tail):
     statistics and gradient against the oracle on every element, with the lse

@@ -121,8 +121,8 @@ def _assert_same_bytes(a, b):
     assert not [(nm, np.flatnonzero(x != y)[:8].tolist()) for nm, x, y in zip(names, a, b) if not np.array_equal(x, y)]
 
 
-# one part and one prompt; two and four CTAs a response; parts that fill both groups and both passes of eight CTAs;
-# more than a round of tokens a thread; empty responses; the largest counts it takes and the next
+# one part and one prompt; two, four and eight parts a response; parts that fill one group and both groups of the
+# cluster's CTAs; more than a round of tokens a thread; empty responses; the largest counts it takes and the next
 _ONE_SHAPES = [(1, 1, 1, 1), (1, 1, 9000, 9000), (4, 1, 256, 256), (2, 4, 64, 1100), (1, 9, 0, 700), (4, 4, 100, 520),
                (8, 4, 0, 260), (32, 1, 1, 200), (33, 1, 1, 9), (1, 33, 1, 9), (3, 1, 300, 12000),
                # beyond it: advantages beside the batch statistics, in one, in several and (too many prompts) in no CTAs there

@@ -1,8 +1,9 @@
 """acrl_token_stats where its load path or its row team changes: a call of few
 rows (ring of loads in shared memory) and a call of many rows that takes the
-register path give the same rows the same bits, at row lengths around a whole
-step of the team's loads, around whole rings and around whole vectors; and
-both agree with a float64 log-softmax."""
+register path (from 4,609 columns; shorter rows have the ring alone) give the
+same rows the same bits, at row lengths around a whole step of the team's
+loads, around whole rings and around whole vectors; and both agree with a
+float64 log-softmax."""
 
 import pytest
 import torch
@@ -19,7 +20,8 @@ _WIDTHS = [1, 8, 63, 64, 255, 256, 257, 767, 768, 769, 1024, 4095, 4096, 4097, 5
 
 
 def _many(V):
-    """Rows that put the call on the register path (teams per SM between 5.2 and 7.5)."""
+    """Rows that put the call on the register path (between 5.2 and 10.4 teams of 128 threads per SM); up to 4,608
+    columns, where eight or sixteen lanes a row have the ring alone, more rows than are resident at once."""
     team = 8 if V <= 4608 else 32 if V <= 16384 else 64 if V <= 40960 else 128
     return 6 * 128 * 152 // team if team > 8 else 4096
 

@@ -32,8 +32,35 @@ __device__ __forceinline__ LseAcc team_partial(const acrl_bf16* row, int V, int 
 template <int THREADS, int DEPTH>
 constexpr int kMinCtas = DEPTH == 0 && THREADS <= 128 ? 1280 / THREADS : 1;
 
+// A team's states as one.  Merging them level by level takes an exponential at each;
+// here each state is brought to the common maximum once, and the rest are plain sums.
+// The lengths of rows whose team has a level more than eight lanes or two warps have
+// meet so (sixteen lanes, and four warps up to kMeetMaxV columns): merged, they came out
+// further from float64 (rms) than with the smaller team, meeting they are closer.
+// Entropy of normal logits (sd 2), V = 4,096: eight lanes 3.74e-7, sixteen merged
+// 3.79e-7, meeting 3.49e-7; V = 57,344: two warps 5.10e-7, four merged 5.28e-7, meeting
+// 4.77e-7; at the same speed.
+__device__ __forceinline__ LseAcc lse_at(const LseAcc& a, float U) {
+    const float da = a.U - U, f = a.s0 > 0.f ? ex2(da) : 0.f;   // an empty state contributes nothing
+    return LseAcc{U, f * a.s0, a.s0 > 0.f ? f * fmaf(da, a.s0, a.s1) : 0.f};
+}
+
+template <int LANES>
+__device__ __forceinline__ LseAcc lanes_meet(LseAcc a) {
+    float U = a.U;
+#pragma unroll
+    for (int m = LANES / 2; m >= 1; m >>= 1) U = fmaxf(U, __shfl_xor_sync(0xffffffffu, U, m));
+    a = lse_at(a, U);
+#pragma unroll
+    for (int m = LANES / 2; m >= 1; m >>= 1) {
+        a.s0 += __shfl_xor_sync(0xffffffffu, a.s0, m);
+        a.s1 += __shfl_xor_sync(0xffffffffu, a.s1, m);
+    }
+    return a;
+}
+
 // A whole CTA per row (vocabulary-size rows).
-template <int THREADS, int UNROLL, int DEPTH>
+template <int THREADS, int UNROLL, int DEPTH, bool MEET>
 __global__ void __launch_bounds__(THREADS, kMinCtas<THREADS, DEPTH>)
     token_stats_cta(const acrl_bf16* __restrict__ logits, int64_t T, int V, int64_t ld,
                     const int32_t* __restrict__ ids, const uint8_t* __restrict__ mask, float* __restrict__ lse,
@@ -54,7 +81,7 @@ __global__ void __launch_bounds__(THREADS, kMinCtas<THREADS, DEPTH>)
         if (threadIdx.x == 0) tgt = row_target(row, V, ids[t]);
         float mx;
         LseAcc acc = team_partial<THREADS, UNROLL, THREADS, DEPTH>(row, V, threadIdx.x, mx, ring);
-        acc = warp_lse(acc);
+        acc = MEET ? lanes_meet<32>(acc) : warp_lse(acc);
         mx = warp_max(mx);
         if (lane == 0) {
             part[wid] = acc;
@@ -64,9 +91,20 @@ __global__ void __launch_bounds__(THREADS, kMinCtas<THREADS, DEPTH>)
         if (threadIdx.x == 0) {
             LseAcc r = part[0];
             float m = pmax[0];
+            if (MEET) {
+#pragma unroll
+                for (int w = 1; w < NW; ++w) r.U = fmaxf(r.U, part[w].U);
+                r = lse_at(part[0], r.U);
+            }
 #pragma unroll
             for (int w = 1; w < NW; ++w) {
-                r = lse_merge(r, part[w]);
+                if (MEET) {
+                    const LseAcc a = lse_at(part[w], r.U);
+                    r.s0 += a.s0;
+                    r.s1 += a.s1;
+                } else {
+                    r = lse_merge(r, part[w]);
+                }
                 m = fmaxf(m, pmax[w]);
             }
             row_outputs(r, m, tgt, lse, logp, ent, t, flags);
@@ -107,25 +145,9 @@ __global__ void __launch_bounds__(THREADS) token_stats_warp(const acrl_bf16* __r
 // which matters where the merges' exponentials are a large share of the row's
 // (V = 2,048: 0.75 -> 0.94 of the copy rate with 8 lanes).  Every lane takes part
 // in the shuffles, whether its row is masked or not.
-// Sixteen lanes bring their sums to the team's maximum once and add them: a level of
-// merges more than eight lanes have, each with an exponential of its own, left the
-// entropy of V = 4,096 1.5-2.1 % further from float64 (rms) than eight lanes do.
 template <int LANES>
 __device__ __forceinline__ LseAcc team_lse(LseAcc a) {
-    if constexpr (LANES == 16) {
-        LseAcc r = a;
-#pragma unroll
-        for (int m = LANES / 2; m >= 1; m >>= 1) r.U = fmaxf(r.U, __shfl_xor_sync(0xffffffffu, r.U, m));
-        const float da = a.U - r.U, f = a.s0 > 0.f ? ex2(da) : 0.f;   // an empty lane contributes nothing
-        r.s0 = f * a.s0;
-        r.s1 = a.s0 > 0.f ? f * fmaf(da, a.s0, a.s1) : 0.f;
-#pragma unroll
-        for (int m = LANES / 2; m >= 1; m >>= 1) {
-            r.s0 += __shfl_xor_sync(0xffffffffu, r.s0, m);
-            r.s1 += __shfl_xor_sync(0xffffffffu, r.s1, m);
-        }
-        return r;
-    }
+    if constexpr (LANES == 16) return lanes_meet<LANES>(a);
 #pragma unroll
     for (int m = LANES / 2; m >= 1; m >>= 1) a = lse_merge(a, shfl_xor(a, m));
     return a;
@@ -181,7 +203,7 @@ __global__ void __launch_bounds__(THREADS) token_stats_team(const acrl_bf16* __r
 // 51.9, a warp 4.4 / 19.3 / 56.9.  V = 49,152, T = 300 / 1,340 / 4,000 / 16,000: two
 // warps 10.2 / 24.7 / 63.8 / 225, four 8.3 / 22.0 / 60.3 / 219; V = 40,000, T = 400 /
 // 3,000 / 10,000: two 10.8 / 39.3 / 123, four 8.9 / 40.8 / 119.
-constexpr int64_t kTeamRowMaxV = 3584, kTeam16RowMaxV = 4608, kMidRowMaxV = 40960;
+constexpr int64_t kTeamRowMaxV = 3584, kTeam16RowMaxV = 4608, kMidRowMaxV = 40960, kMeetMaxV = 65536;
 constexpr int kUnroll = 4;
 
 // Steps of the ring: with few rows per SM, one step of loads per thread leaves
@@ -253,8 +275,11 @@ extern "C" acrl_status acrl_token_stats(const acrl_bf16* logits, int64_t T, int6
         return ring ? run(token_stats_warp<64, kUnroll, kDepth>, 64, kDepth, 2)
                     : run(token_stats_warp<256, kUnroll, 0>, 256, 0, 8);
     if (team == 64)
-        return ring ? run(token_stats_cta<64, kUnroll, kDepth>, 64, kDepth, 1)
-                    : run(token_stats_cta<64, kUnroll, 0>, 64, 0, 1);
-    return ring ? run(token_stats_cta<128, kUnroll, kDepth>, 128, kDepth, 1)
-                : run(token_stats_cta<128, kUnroll, 0>, 128, 0, 1);
+        return ring ? run(token_stats_cta<64, kUnroll, kDepth, false>, 64, kDepth, 1)
+                    : run(token_stats_cta<64, kUnroll, 0, false>, 64, 0, 1);
+    if (V <= kMeetMaxV)
+        return ring ? run(token_stats_cta<128, kUnroll, kDepth, true>, 128, kDepth, 1)
+                    : run(token_stats_cta<128, kUnroll, 0, true>, 128, 0, 1);
+    return ring ? run(token_stats_cta<128, kUnroll, kDepth, false>, 128, kDepth, 1)
+                : run(token_stats_cta<128, kUnroll, 0, false>, 128, 0, 1);
 }

@@ -175,6 +175,6 @@ def test_kernels_of_vocabulary_rows_fit_their_residency():
         build.build(force=True)
     report = re.findall(r"Compiling entry function '(\S+)'.*?Used (\d+) registers", open(path).read(), flags=re.S)
     for pattern, limit, n in ((r"loss_grad_ctaILi256ELi4ELb0ELb[01]ELb0ELb1E", 42, 2),
-                              (r"token_stats_ctaILi(64|128)ELi4ELi0E", 48, 2), (r"token_stats_warpILi256ELi4ELi0E", 48, 1)):
+                              (r"token_stats_ctaILi(64|128)ELi4ELi0E", 48, 3), (r"token_stats_warpILi256ELi4ELi0E", 48, 1)):
         found = {k: int(v) for k, v in report if re.search(pattern, k)}
         assert len(found) == n and all(v <= limit for v in found.values()), (pattern, found)

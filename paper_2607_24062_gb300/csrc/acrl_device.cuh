@@ -121,6 +121,14 @@ __device__ __forceinline__ LseAcc lse_merge(const LseAcc& a, const LseAcc& b) {
     return r;
 }
 
+// A state's sums against another exponent, at least as large.  Where several states
+// become one, merging them level by level takes an exponential at each; brought to
+// their common maximum, each takes one, and the rest are plain sums.
+__device__ __forceinline__ LseAcc lse_at(const LseAcc& a, float U) {
+    const float da = a.U - U, f = a.s0 > 0.f ? ex2(da) : 0.f;   // an empty state contributes nothing
+    return LseAcc{U, f * a.s0, a.s0 > 0.f ? f * fmaf(da, a.s0, a.s1) : 0.f};
+}
+
 __device__ __forceinline__ LseAcc shfl_xor(const LseAcc& a, int m) {
     return LseAcc{__shfl_xor_sync(0xffffffffu, a.U, m), __shfl_xor_sync(0xffffffffu, a.s0, m),
                   __shfl_xor_sync(0xffffffffu, a.s1, m)};

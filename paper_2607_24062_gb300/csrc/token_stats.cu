@@ -32,19 +32,13 @@ __device__ __forceinline__ LseAcc team_partial(const acrl_bf16* row, int V, int 
 template <int THREADS, int DEPTH>
 constexpr int kMinCtas = DEPTH == 0 && THREADS <= 128 ? 1280 / THREADS : 1;
 
-// A team's states as one.  Merging them level by level takes an exponential at each;
-// here each state is brought to the common maximum once, and the rest are plain sums.
+// A team's states as one, brought to the common maximum (lse_at).
 // The lengths of rows whose team has a level more than eight lanes or two warps have
 // meet so (sixteen lanes, and four warps up to kMeetMaxV columns): merged, they came out
 // further from float64 (rms) than with the smaller team, meeting they are closer.
 // Entropy of normal logits (sd 2), V = 4,096: eight lanes 3.74e-7, sixteen merged
 // 3.79e-7, meeting 3.49e-7; V = 57,344: two warps 5.10e-7, four merged 5.28e-7, meeting
 // 4.77e-7; at the same speed.
-__device__ __forceinline__ LseAcc lse_at(const LseAcc& a, float U) {
-    const float da = a.U - U, f = a.s0 > 0.f ? ex2(da) : 0.f;   // an empty state contributes nothing
-    return LseAcc{U, f * a.s0, a.s0 > 0.f ? f * fmaf(da, a.s0, a.s1) : 0.f};
-}
-
 template <int LANES>
 __device__ __forceinline__ LseAcc lanes_meet(LseAcc a) {
     float U = a.U;

@@ -746,57 +746,75 @@ __device__ __forceinline__ uint4 shift_elems(const uint4& lo, const uint4& hi, i
                       __funnelshift_r(z[2], z[3], half), __funnelshift_r(z[3], z[4], half));
 }
 
+// bf16 products of two pairs (one rounding each, as the fp32 product's).
+__device__ __forceinline__ uint32_t mul_bf16x2(uint32_t a, uint32_t b) {
+    uint32_t r;
+    asm("mul.rn.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
+    return r;
+}
+
 // The same product into rows without a gap whose length is no multiple of eight (the
-// contiguous [T, V] tensor that a framework's own product is).  A thread takes
-// kScaleUnroll 16-byte vectors of the output as it lies in memory; one inside a row
-// comes from two neighbouring vectors of `grad`, shifted by the columns that the row
-// starts off a vector (the second is the next lane's first, from L1); one that holds a
-// row's end, or the end of the output, goes element by element.
+// contiguous [T, V] tensor that a framework's own product is).  A lane makes the
+// 16-byte vectors of the output as it lies in memory, so that a warp writes whole
+// lines; one inside a row is shifted together from the vector of `grad` that holds its
+// first column and the next one, which the next lane holds; one that holds a row's end,
+// or the output's, goes element by element.  4,992 rows of 20,011 columns: 70 us (the
+// next vector loaded again, through L1: 87; a row's vectors from its own start, so that
+// warps share 32-byte sectors of the output: 81; a row end's elements all at once, whose
+// registers cost residency: 86; a plain copy of the buffer 62; an elementwise product of
+// the strided view 216).
+constexpr int kDenseUnroll = 2;
+
 __global__ void __launch_bounds__(kScaleThreads)
     scale_grad_dense_kernel(const acrl_bf16* __restrict__ grad, int64_t T, int V, int64_t ld,
                             const float* __restrict__ scale, acrl_bf16* __restrict__ out) {
+    constexpr int U = kDenseUnroll, kApart = 8 * kScaleThreads;   // columns between two vectors of a thread
+    const int lane = threadIdx.x & 31;
     grid_begin();
     const float f = *scale;
     if (f == 1.f) return;  // the caller keeps `grad`
-    const float s = bf16_lo(pack_bf16x2(f, 0.f));
-    const int64_t total = T * V, nvec = (total + 7) >> 3, step = int64_t(gridDim.x) * kScaleThreads * kScaleUnroll;
-    constexpr int kApart = 8 * kScaleThreads;   // elements between two vectors of a thread
-    for (int64_t i = int64_t(blockIdx.x) * kScaleThreads * kScaleUnroll + threadIdx.x; i < nvec; i += step) {
+    const uint32_t s = pack_bf16x2(f, f);
+    const int64_t total = T * V, nvec = (total + 7) >> 3, step = int64_t(gridDim.x) * kScaleThreads * U;
+    // a warp's lanes stay together, those beyond the end with row >= T
+    for (int64_t i = int64_t(blockIdx.x) * kScaleThreads * U + threadIdx.x; i - lane < nvec; i += step) {
         int64_t row = i * 8 / V;
         int col = int(i * 8 - row * V);
-        uint4 lo[kScaleUnroll], hi[kScaleUnroll];
-        int64_t at_row[kScaleUnroll];
-        int at_col[kScaleUnroll];
+        uint4 lo[U];
+        int64_t rows[U];
+        int cols[U];
 #pragma unroll
-        for (int k = 0; k < kScaleUnroll; ++k) {
-            at_row[k] = row;
-            at_col[k] = col;
-            if (row < T && col + 8 <= V) {
-                const uint4* src = reinterpret_cast<const uint4*>(grad + row * ld) + (col >> 3);
-                lo[k] = __ldg(src);
-                hi[k] = col & 7 ? __ldg(src + 1) : lo[k];   // holds column col + 7 at the latest
-            }
+        for (int k = 0; k < U; ++k) {
+            rows[k] = row;
+            cols[k] = col;
+            lo[k] = make_uint4(0u, 0u, 0u, 0u);
+            if (row < T) lo[k] = ld_stream(reinterpret_cast<const uint4*>(grad + row * ld) + (col >> 3));
             col += kApart;
-            const int rows = col < V ? 0 : V >= kApart ? 1 : col / V;
-            row += rows;
-            col -= rows * V;
+            const int over = col < V ? 0 : V >= kApart ? 1 : col / V;
+            row += over;
+            col -= over * V;
         }
 #pragma unroll
-        for (int k = 0; k < kScaleUnroll; ++k) {
+        for (int k = 0; k < U; ++k) {
             const int64_t v = i + k * kScaleThreads;
-            if (at_row[k] < T && at_col[k] + 8 <= V) {
-                const uint4 x = shift_elems(lo[k], hi[k], at_col[k] & 7);
-                st_stream(reinterpret_cast<uint4*>(out) + v,
-                          make_uint4(scale_pair(x.x, s), scale_pair(x.y, s), scale_pair(x.z, s), scale_pair(x.w, s)));
+            const acrl_bf16* src = grad + rows[k] * ld;
+            const int c = cols[k], m = c & 7;
+            const bool whole = rows[k] < T && c + 8 <= V;
+            uint4 hi = make_uint4(__shfl_down_sync(0xffffffffu, lo[k].x, 1), __shfl_down_sync(0xffffffffu, lo[k].y, 1),
+                                  __shfl_down_sync(0xffffffffu, lo[k].z, 1), __shfl_down_sync(0xffffffffu, lo[k].w, 1));
+            // no next lane, or one that begins the next row; the vector holds column c + 7 at the latest
+            if (whole && m && (lane == 31 || c + 8 == V)) hi = ld_stream(reinterpret_cast<const uint4*>(src) + (c >> 3) + 1);
+            if (whole) {
+                const uint4 x = shift_elems(lo[k], hi, m);
+                st_stream(reinterpret_cast<uint4*>(out) + v, make_uint4(mul_bf16x2(x.x, s), mul_bf16x2(x.y, s),
+                                                                        mul_bf16x2(x.z, s), mul_bf16x2(x.w, s)));
             } else if (v < nvec) {
-                int64_t r = at_row[k];
-                int c = at_col[k];
+                int at = c;
 #pragma unroll 1
                 for (int64_t j = v * 8; j < min(total, v * 8 + 8); ++j) {
-                    out[j] = acrl_bf16(scale_pair(grad[r * ld + c], s) & 0xffffu);
-                    if (++c == V) {
-                        c = 0;
-                        ++r;
+                    out[j] = acrl_bf16(mul_bf16x2(src[at], s) & 0xffffu);
+                    if (++at == V) {
+                        at = 0;
+                        src += ld;
                     }
                 }
             }
@@ -899,7 +917,7 @@ extern "C" acrl_status acrl_scale_grad(const acrl_bf16* grad, int64_t T, int64_t
     const int64_t per_cta = kScaleThreads * kScaleUnroll;
     const int64_t rows = T < kMaxGrid ? T : kMaxGrid;
     if ((ldo & 7) != 0)
-        return launch(scale_grad_dense_kernel, grid_for(per_cta, rows * nvec), kScaleThreads, 0, 0,
+        return launch(scale_grad_dense_kernel, grid_for(kScaleThreads * kDenseUnroll, rows * nvec), kScaleThreads, 0, 0,
                       reinterpret_cast<cudaStream_t>(stream), grad, T, int(V), ld, scale, out);
     return launch(scale_grad_kernel, grid_for(per_cta, rows * nvec), kScaleThreads, 0, 0,
                   reinterpret_cast<cudaStream_t>(stream), grad, T, nvec, ld, scale, out, ldo);

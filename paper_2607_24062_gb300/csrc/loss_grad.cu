@@ -55,7 +55,9 @@ constexpr int kStreamStep = 8 * kCtaUnroll;   // columns of one thread's step
 // last step is short.  A CTA of 768 threads per row / split: 40 x 151,936 12.7 / 9.2
 // us, 408 x 151,936 42.4 / 41.2, 700 x 151,936 69.7 / 65.9, 3,000 x 151,936 268 / 262,
 // 3,000 x 65,544 123.5 / 117.8, 3,000 x 200,000 355 / 343; with 6 to 8 shares of
-// 151,936 columns 66.7, with 11 to 14 68.
+// 151,936 columns 66.7, with 11 to 14 68.  Lengths that make wider shares: 3,000 x
+// 80,000 (2.4 steps) 148 / 143, 20,000 919 / 917; 3,000 x 128,256 (2.2) 232 / 224, 8,000
+// 597 / 585; 300 x 72,000 (2.2) 22.7 / 18.0.
 constexpr int kShareThreads = 256, kShareVecs = 2 * kShareThreads * kCtaUnroll;
 constexpr int64_t kShareRowMinV = 65537;
 // A call of so many rows that the shares would not fit a grid takes a CTA per row.

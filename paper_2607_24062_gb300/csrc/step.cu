@@ -1,7 +1,7 @@
 // acrl_step: the whole on-policy pass in one call.  Host code only: with a small
 // batch the device waits for the host, and one call with every pointer costs less
 // than half of the five (a step of 4 x 256 tokens at V = 4,096 called from Python:
-// 75 us as five calls and eight launches, 35 as one call and four).
+// 82 us as five calls and nine launches, 35 as one call and four).
 #include "acrl_host.h"
 
 using namespace acrl;
